@@ -179,12 +179,13 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
 
 /* Advance n >= 0 time steps with the given scheme and relaxation time
  * tau > 1/2 (sigma is read by LBM_SCHEME_IMPROVED only).  Kernels are queued
- * on the context stream, one per step; on lattices of at most 2048^2 cells
- * runs of 16 steps go through a CUDA graph of 16 step kernels, captured on
- * first use for the current buffer and launch arguments and kept until the
- * context is destroyed (bit-identical to single launches); while the caller
- * captures the context stream into a graph of its own, lbm_step_async records
- * one launch per step instead.  The call then waits for the kernels and
+ * on the context stream, one per step, or one per two steps (FP32 storage,
+ * AUTO variant and band height, at least 176^2 cells; an odd last step goes
+ * alone); on lattices of at most 2048^2 cells runs of 16 steps go through a
+ * CUDA graph of these kernels, captured on first use for the current buffer
+ * and launch arguments and kept until the context is destroyed (bit-identical
+ * to single launches); while the caller captures the context stream into a
+ * graph of its own, lbm_step_async records the launches one by one instead.  The call then waits for the kernels and
  * reads the device status word once (so lbm_step itself cannot be
  * captured).  LBM_E_DIVERGED if psi became undefined in any step (the state
  * is then unspecified but the context stays usable and destroyable);

@@ -384,6 +384,7 @@ lbm_status launch_rows(lbm_ctx* c, int scheme, StripLaunch L, int r0, int r1, in
 // them with shorter gaps (~4 us per step there, a few per cent faster up to
 // 2048^2).  From 4096^2 on the step's own time hides the gap.
 constexpr int kGraphSteps = 16;
+constexpr int kPairsVariant = -1;  // step-graph key of the two-step launches
 constexpr size_t kGraphMaxCells = size_t(2048) * 2048;
 
 // One step kernel from buffer c->cur on `stream`, flipping c->cur.
@@ -404,6 +405,39 @@ cudaError_t launch_step(lbm_ctx* c, int scheme, StripLaunch& L, int grid, cudaSt
   return e;
 }
 
+// A step graph or a run of plain launches: n steps, two per launch where
+// `two` holds the two-step launch (a last odd step alone).
+struct StepPlan {
+  StripLaunch one;  // one step per launch
+  int one_grid = 0;
+  bool pairs = false;  // two_step_applies
+  StripLaunch two;     // two steps per launch
+  int two_grid = 0;
+};
+
+// Queue up to n steps on `stream`; *done counts the steps, *launches the
+// kernels.
+cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t stream,
+                     int* launches) {
+  for (int k = 0; k < n;) {
+    if (plan.pairs && n - k >= 2) {
+      const int s = c->cur, d = 1 - c->cur;
+      plan.two.src = c->f[s];
+      plan.two.dst = c->f[d];
+      const cudaError_t e = two_step_launch(scheme, plan.two, plan.two_grid, stream);
+      if (e != cudaSuccess) return e;
+      c->cur = d;
+      k += 2;
+    } else {
+      const cudaError_t e = launch_step(c, scheme, plan.one, plan.one_grid, stream);
+      if (e != cudaSuccess) return e;
+      k += 1;
+    }
+    ++*launches;
+  }
+  return cudaSuccess;
+}
+
 // Every argument a step kernel reads, compared field by field.
 bool same_launch(const StripLaunch& x, const StripLaunch& y) {
   return x.src == y.src && x.dst == y.dst && x.rho_src == y.rho_src && x.rho_dst == y.rho_dst &&
@@ -420,16 +454,19 @@ bool same_launch(const StripLaunch& x, const StripLaunch& y) {
 // The cached graph of kGraphSteps steps from the current buffer, captured
 // again when any kernel argument, the scheme, the kernel variant or the grid
 // changed; nullptr when capture is unavailable (the caller then launches
-// step by step).
-cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, StripLaunch L, int grid) {
+// step by step).  With pairs the steps are kGraphSteps / 2 two-step launches;
+// that count is even too, so a replay leaves the state in the same buffer.
+cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan) {
   lbm_ctx::StepGraph& g = c->graph[c->cur];
-  const int variant = pick_variant(c, kStepMode);
-  L.src = c->f[c->cur];
-  L.dst = c->f[1 - c->cur];
-  L.rho_src = c->rho[c->cur];
-  L.rho_dst = c->rho[1 - c->cur];
+  const int variant = plan.pairs ? kPairsVariant : pick_variant(c, kStepMode);
+  const int grid = plan.pairs ? plan.two_grid : plan.one_grid;
+  StripLaunch first = plan.pairs ? plan.two : plan.one;  // the key
+  first.src = c->f[c->cur];
+  first.dst = c->f[1 - c->cur];
+  first.rho_src = c->rho[c->cur];
+  first.rho_dst = c->rho[1 - c->cur];
   if (g.exec && g.scheme == scheme && g.variant == variant && g.grid == grid &&
-      same_launch(g.L, L))
+      same_launch(g.L, first))
     return g.exec;
   if (g.exec) {
     cudaGraphExecDestroy(g.exec);
@@ -441,13 +478,13 @@ cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, StripLaunch L, int grid) {
     c->cap_stream = nullptr;
     return nullptr;
   }
-  const StripLaunch first = L;  // the key: launch_step overwrites the buffers
+  StepPlan scratch = plan;  // run_plan sets the buffers
   const int cur0 = c->cur;
+  int launches = 0;
   cudaGraph_t graph = nullptr;
   bool ok = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) ==
             cudaSuccess;
-  for (int k = 0; ok && k < kGraphSteps; ++k)
-    ok = launch_step(c, scheme, L, grid, c->cap_stream) == cudaSuccess;
+  ok = ok && run_plan(c, scheme, scratch, kGraphSteps, c->cap_stream, &launches) == cudaSuccess;
   c->cur = cur0;  // capturing ran nothing
   const bool ended = cudaStreamEndCapture(c->cap_stream, &graph) == cudaSuccess;
   cudaGraphExec_t exec = nullptr;
@@ -476,31 +513,42 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
   if (c->band && n > 1)
     return fail(c, LBM_E_INVAL, "a band advances one step per call (exchange halos between)");
   if (n == 0) return LBM_OK;
-  StripLaunch L = step_launch(c, tau, sigma);
-  int grid = 0;
-  lbm_status st = geometry(c, scheme, kStepMode, L, grid);
+  StepPlan plan;
+  plan.one = step_launch(c, tau, sigma);
+  lbm_status st = geometry(c, scheme, kStepMode, plan.one, plan.one_grid);
   if (st != LBM_OK) return st;
-  int k = 0;
+  plan.pairs = !c->band && n >= 2 &&
+               two_step_applies(c->variant, c->p.precision, c->p.nx, c->p.ny,
+                                c->band_rows_override, c->p.b);
+  if (plan.pairs) {
+    const StripGeometry g = two_step_geometry(c->p.nx, c->p.ny, c->sm_count);
+    plan.two = plan.one;
+    plan.two.n_strips = g.n_strips;
+    plan.two.band_rows = g.band_rows;
+    plan.two.n_bands = g.n_bands;
+    plan.two_grid = g.grid;
+  }
+  int k = 0, launches = 0;
   // (not while the caller captures the context stream into a graph of its
   // own: the steps are then recorded one launch at a time)
+  const bool graphs =
+      !c->band && n >= kGraphSteps && size_t(c->p.nx) * c->p.ny <= kGraphMaxCells;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (!c->band && n >= kGraphSteps && size_t(c->p.nx) * c->p.ny <= kGraphMaxCells &&
-      cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) {
+  if (graphs && cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) {
     cudaGetLastError();  // treated as capturing: plain launches
     capturing = cudaStreamCaptureStatusActive;
   }
-  if (!c->band && n >= kGraphSteps && size_t(c->p.nx) * c->p.ny <= kGraphMaxCells &&
-      capturing == cudaStreamCaptureStatusNone) {
-    const cudaGraphExec_t g = step_graph(c, scheme, L, grid);
+  if (graphs && capturing == cudaStreamCaptureStatusNone) {
+    const cudaGraphExec_t g = step_graph(c, scheme, plan);
     if (g)
-      for (; k + kGraphSteps <= n; k += kGraphSteps)
+      for (; k + kGraphSteps <= n; k += kGraphSteps) {
         LBM_CUDA(c, cudaGraphLaunch(g, c->stream));  // the state returns to c->cur
+        launches += plan.pairs ? kGraphSteps / 2 : kGraphSteps;
+      }
   }
-  for (; k < n; ++k) {
-    const cudaError_t e = launch_step(c, scheme, L, grid, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
-  }
-  count_launches((unsigned long long)n);
+  const cudaError_t e = run_plan(c, scheme, plan, n - k, c->stream, &launches);
+  if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+  count_launches((unsigned long long)launches);
   c->last_scheme = scheme;
   return LBM_OK;
 }

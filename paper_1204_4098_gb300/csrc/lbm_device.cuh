@@ -144,19 +144,45 @@ __device__ __forceinline__ Pair<C> fast_div(Pair<C> a, Pair<C> b) {
   return Pair<C>(fast_div(a.x(), b.x()), fast_div(a.y(), b.y()));
 }
 
+// The same reciprocal and root for operands known to be normal, with normal
+// results: without the handling of subnormal and huge operands around it,
+// each is one hardware instruction (the full forms above take 4-6 more per
+// cell).  For normal operands they give the bits of the functions above.
+__device__ __forceinline__ float rcp_normal(float b) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_normal(float a) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
+// a / b; kNormal: b and 1 / b are normal numbers (FP32)
+template <bool kNormal, class V>
+__device__ __forceinline__ V quot(V a, V b) {
+  if constexpr (!kNormal) {
+    return fast_div(a, b);
+  } else if constexpr (std::is_same<V, float>::value) {
+    return mul_rn(a, rcp_normal(b));
+  } else {
+    return V(mul_rn(a.x(), rcp_normal(b.x())), mul_rn(a.y(), rcp_normal(b.y())));
+  }
+}
+
 // psi of Eq. 8 with the Carnahan-Starling p_EOS of Eq. 23.  Flags (and
 // returns 0 for) densities outside the domain of psi: rho <= 0, eta >= 1,
 // a negative or non-finite radicand.  psi_radicand holds the arithmetic
 // (for a scalar or a pair), psi_finish the per-cell domain check and root.
-template <class V, class C>
-__device__ __forceinline__ void psi_radicand(V rho, const Phys<C>& P, V& eta, V& arg) {
+template <bool kNormal = false, class V, class C>
+__device__ __forceinline__ void psi_radicand(V rho, const Phys<C>& P, V& eta, V& om, V& arg) {
   const V one = V(C(1));
   eta = mul_rn(V(P.b4), rho);
-  const V om = sub_rn(one, eta);
+  om = sub_rn(one, eta);
   // 1 + eta + eta^2 - eta^3 = 1 + eta (1 + eta (1 - eta))
   const V num = fma_rn(eta, fma_rn(eta, om, one), one);
   const V den = mul_rn(mul_rn(om, om), om);
-  const V p = sub_rn(fast_div(mul_rn(mul_rn(rho, V(P.RT)), num), den),
+  const V p = sub_rn(quot<kNormal>(mul_rn(mul_rn(rho, V(P.RT)), num), den),
                      mul_rn(mul_rn(V(P.a), rho), rho));
   arg = mul_rn(V(P.two_over_G), sub_rn(p, mul_rn(rho, V(C(1) / C(3)))));
 }
@@ -168,14 +194,14 @@ __device__ __forceinline__ C psi_finish(C rho, C eta, C arg, bool& bad) {
 }
 template <class C>
 __device__ __forceinline__ C psi_of_rho(C rho, const Phys<C>& P, bool& bad) {
-  C eta, arg;
-  psi_radicand(rho, P, eta, arg);
+  C eta, om, arg;
+  psi_radicand(rho, P, eta, om, arg);
   return psi_finish(rho, eta, arg, bad);
 }
 template <class C>
 __device__ __forceinline__ Pair<C> psi_of_rho(Pair<C> rho, const Phys<C>& P, bool& bad) {
-  Pair<C> eta, arg;
-  psi_radicand(rho, P, eta, arg);
+  Pair<C> eta, om, arg;
+  psi_radicand(rho, P, eta, om, arg);
   return Pair<C>(psi_finish(rho.x(), eta.x(), arg.x(), bad),
                  psi_finish(rho.y(), eta.y(), arg.y(), bad));
 }
@@ -225,7 +251,7 @@ constexpr int kAnyForced = -1;
 // parameters stay scalars of type C and are broadcast where they meet a
 // per-cell value.  The sequence of rounded operations per cell is the same
 // either way.
-template <class V, class C>
+template <bool kNormal, class V, class C>
 __device__ __forceinline__ void collide_mrt(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
                                             const Phys<C>& P) {
   const V ax = sub_rn(f[1], f[3]), ay = sub_rn(f[2], f[4]);  // axis odd parts
@@ -240,11 +266,11 @@ __device__ __forceinline__ void collide_mrt(V (&f)[kQ], V rho, V Fx, V Fy, V psi
   const V pxx = sub_rn(add_rn(f[1], f[3]), add_rn(f[2], f[4]));
   const V pxy = sub_rn(add_rn(f[5], f[7]), add_rn(f[6], f[8]));
 
-  const V inv_rho = fast_div(V(C(1)), rho);
+  const V inv_rho = quot<kNormal>(V(C(1)), rho);
   const V half_inv = mul_rn(V(C(0.5)), inv_rho);
   const V vx = fma_rn(half_inv, Fx, mul_rn(jx, inv_rho));
   const V vy = fma_rn(half_inv, Fy, mul_rn(jy, inv_rho));
-  const V sg = fast_div(V(P.sigma_ups), mul_rn(psi, psi));
+  const V sg = quot<kNormal>(V(P.sigma_ups), mul_rn(psi, psi));
   const V wx = fma_rn(sg, Fx, vx), wy = fma_rn(sg, Fy, vy);  // v'
   const V v2 = fma_rn(vx, vx, mul_rn(vy, vy));
   const V rv2 = mul_rn(V(C(3)), mul_rn(rho, v2));
@@ -289,12 +315,12 @@ __device__ __forceinline__ void collide_mrt(V (&f)[kQ], V rho, V Fx, V Fy, V psi
   f[0] = sub_rn(rho, rest);
 }
 
-template <int SCHEME, class V, class C>
+template <int SCHEME, bool kNormal = false, class V, class C>
 __device__ __forceinline__ void collide(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
                                         const Phys<C>& P) {
   if constexpr (SCHEME == kMRT) {
     if constexpr (std::is_same<V, C>::value) {
-      collide_mrt(f, rho, Fx, Fy, psi, P);
+      collide_mrt<kNormal>(f, rho, Fx, Fy, psi, P);
     } else {
       // Element by element: in this body the packed FP32x2 instructions were
       // measured a few ulps away from the scalar ones on ~0.6 % of the values
@@ -307,8 +333,8 @@ __device__ __forceinline__ void collide(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
         fa[a] = f[a].x();
         fb[a] = f[a].y();
       }
-      collide_mrt(fa, rho.x(), Fx.x(), Fy.x(), psi.x(), P);
-      collide_mrt(fb, rho.y(), Fx.y(), Fy.y(), psi.y(), P);
+      collide_mrt<kNormal>(fa, rho.x(), Fx.x(), Fy.x(), psi.x(), P);
+      collide_mrt<kNormal>(fb, rho.y(), Fx.y(), Fy.y(), psi.y(), P);
 #pragma unroll
       for (int a = 0; a < kQ; ++a) f[a] = V(fa[a], fb[a]);
     }
@@ -317,7 +343,7 @@ __device__ __forceinline__ void collide(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
   const int sch = SCHEME == kAnyForced ? P.scheme : SCHEME;
   const V jx = add_rn(add_rn(sub_rn(f[1], f[3]), sub_rn(f[5], f[6])), sub_rn(f[8], f[7]));
   const V jy = sub_rn(add_rn(sub_rn(f[2], f[4]), add_rn(f[5], f[6])), add_rn(f[7], f[8]));
-  const V inv_rho = fast_div(V(C(1)), rho);
+  const V inv_rho = quot<kNormal>(V(C(1)), rho);
   const V ux = mul_rn(jx, inv_rho), uy = mul_rn(jy, inv_rho);
   const V half_inv = mul_rn(V(C(0.5)), inv_rho);
 
@@ -337,7 +363,7 @@ __device__ __forceinline__ void collide(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
   } else if (sch == kImproved) {
     qx = fma_rn(half_inv, Fx, ux);
     qy = fma_rn(half_inv, Fy, uy);
-    const V s = fast_div(V(P.sigma_ups), mul_rn(psi, psi));
+    const V s = quot<kNormal>(V(P.sigma_ups), mul_rn(psi, psi));
     Vx = fma_rn(s, Fx, qx);
     Vy = fma_rn(s, Fy, qy);
     Be = P.guo;

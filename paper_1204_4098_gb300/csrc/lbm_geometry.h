@@ -82,4 +82,52 @@ inline StripGeometry strip_geometry(int nx, int ny, int variant, long long resid
   return g;
 }
 
+// ---------------------------------------------------------------------------
+// two steps per launch (lbm_two_step.cuh)
+// ---------------------------------------------------------------------------
+constexpr int kTwoStepCols = 56;   // columns of a strip
+constexpr int kTwoStepWarps = 12;  // resident warps per SM
+
+// Whether steps of a whole nx x ny FP32 lattice may go two per launch: AUTO
+// variant and band height (a requested kernel or height runs as requested),
+// a lattice large enough to gain, 32-bit byte offsets within a plane, and a
+// covolume for which every density inside the domain of psi (b rho / 4 < 1)
+// has a normal reciprocal.
+constexpr long long kTwoStepMinCells = 176LL * 176;
+constexpr long long kTwoStepMaxCells = 1LL << 30;
+inline bool two_step_applies(int requested, int precision, int nx, int ny,
+                             int band_rows_override, double b) {
+  const long long cells = (long long)nx * ny;
+  return requested == LBM_VARIANT_AUTO && band_rows_override == 0 && precision == LBM_FP32 &&
+         cells >= kTwoStepMinCells && cells <= kTwoStepMaxCells && b > 1e-12 && b < 1e12;
+}
+
+// Strips of 56 columns and the band height that ends first.  A band of n rows
+// runs n + 7 iterations; with 4, 8 or 12 warps per SM (1, 2 or 3 per
+// scheduler; numbers between leave one scheduler with more than the others
+// and end no earlier) an iteration takes 0.60, 0.94 and 1.32 us (1024^2,
+// improved scheme), so short bands of many warps pay only while the rows
+// dominate: 512^2 takes 4 warps per SM (5.2 us per step against 5.9 with 7 and 6.9
+// with 12), 1024^2 8 (10.9; 11.7 with 4, 11.9 with 12), 2048^2 12 (31.9; 32.2).
+inline StripGeometry two_step_geometry(int nx, int ny, int sm_count) {
+  StripGeometry g;
+  g.n_strips = (nx + kTwoStepCols - 1) / kTwoStepCols;
+  const double cost[3] = {0.60, 0.94, 1.32};
+  double best = 0.0;
+  g.band_rows = ny;
+  for (int k = 0; k < 3; ++k) {
+    const long long resident = (long long)sm_count * kTwoStepWarps * (k + 1) / 3;
+    const long long bands = std::min<long long>(std::max<long long>(1, resident / g.n_strips), ny);
+    const int rows = int((ny + bands - 1) / bands);
+    const double t = (rows + 7) * cost[k];
+    if (k == 0 || t < best) {
+      best = t;
+      g.band_rows = rows;
+    }
+  }
+  g.n_bands = (ny + g.band_rows - 1) / g.band_rows;
+  g.grid = g.n_strips * g.n_bands;
+  return g;
+}
+
 }  // namespace lbm

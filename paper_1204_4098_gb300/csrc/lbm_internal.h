@@ -57,6 +57,9 @@ cudaError_t strip2_occupancy(int precision, int scheme, int mode, int* blocks_pe
 cudaError_t strip_tma_launch(int precision, int scheme, const StripLaunch& L, int grid,
                              cudaStream_t s);
 cudaError_t strip_tma_occupancy(int precision, int scheme, int* blocks_per_sm);
+// Two steps from L.src to L.dst in one launch (FP32 storage, any nx, at most
+// kTwoStepMaxCells cells; L as two_step_geometry sets it).
+cudaError_t two_step_launch(int scheme, const StripLaunch& L, int grid, cudaStream_t s);
 
 // f*_a(x') = f_a(x' + e_a) from f_eq(rho, u) (f_in == NULL) or from f_in;
 // with f_in == NULL and chk.status set, flags rho outside the domain of psi.

@@ -1,0 +1,320 @@
+// Two time steps in one pass over the lattice (FP32 storage).
+//
+// The one-step kernels move 72 B per cell update and run at 0.93 of the copy
+// bandwidth on large lattices: they cannot get faster without moving less.
+// Here a warp marches down a band of rows as they do, but carries every row
+// through two steps before it is stored: the step-1 populations of the last
+// three rows stay on chip (registers, and two rows of the warp's shared
+// memory), so a launch reads and writes each population once per TWO steps
+// (36 B per cell update).  Every per-cell expression is the one of the
+// one-step kernels, so the populations are the same bits.
+//
+// Columns.  A row's step-2 result needs step-1 results one column further
+// out for the pull and one more for psi, and those need the same again: a
+// warp loads 64 columns (two per lane) and owns the inner 56.  Nothing is
+// exchanged between warps, and the halo columns are ordinary columns of the
+// march (the one-step kernel's extra halo loads, shuffles and psi evaluation,
+// ~10 % of its instructions, have no counterpart); 8 of 64 columns are
+// computed twice.  At the wrong side of the strip's edge, lanes compute
+// values that nothing uses.  Rows likewise: a band of n rows runs n + 7
+// iterations (6 rows of halo, and one of pipeline delay, below).
+//
+// Balance.  With the traffic halved the kernel is bound by its instructions,
+// first by the latency of dependent ones (three warps per scheduler).  Step 2
+// therefore works one row behind, on the row that the previous iteration
+// completed, so that the two steps of an iteration do not depend on each
+// other and the loop has no branch the scheduler could not move them across.
+// Divisions and roots take the bare hardware instructions; their operands are
+// checked as part of the domain check (psi_normal), and a band in which a
+// check fails is run again with the full forms (strip_run_two<kNormal =
+// false>), which also report divergence.  One warp per CTA: strip, band and
+// row are then block-uniform and their address arithmetic leaves the lanes
+// (4096^2: 114.1 us per step against 116.8 with four warps per CTA).
+//
+// Measured on the way (improved scheme, 4096^2, us per step; one-step kernel
+// 197.5): first version 141; unrolled by two 134; bare divisions and roots
+// 128; no branches 123; step 2 one row behind 118; one warp per CTA 114
+// (147k MLUPS, DRAM at 0.77 of the measured copy bandwidth, FMA pipes 60 %
+// busy, 158 registers, 12 warps per SM).  13 to 16 warps per SM (128
+// registers, spilling) 119-122; rows of step 1 kept in registers 141 (spills).
+#pragma once
+
+#include "lbm_kernels.cuh"
+
+namespace lbm {
+
+constexpr int kTwoHalo = 4;                  // columns loaded on each side of a strip
+constexpr int kTwoCols = 64 - 2 * kTwoHalo;  // columns a strip owns
+constexpr int kTwoStages = 3;                // rows in shared memory: one read, two in flight
+constexpr int kTwoThreads = 32;              // one warp per CTA
+constexpr int kTwoMinBlocks = 12;            // CTAs per SM (168 registers at most)
+
+// One row of a warp in shared memory: the 9 planes' pairs, lane-major.
+struct TwoRow {
+  float2 d[kQ][32];
+};
+
+// psi of a row: the x neighbours only enter the force (Eq. 3) as their
+// difference and sum, formed once per row.
+struct PsiRow {
+  F2 c, d, s;  // psi, psi(x + 1) - psi(x - 1), psi(x + 1) + psi(x - 1)
+};
+
+// Smallest of three with NaN kept (one instruction).
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+// psi of a pair, and whether it holds as it stands: every operand of the
+// reciprocals and the root (and of the reciprocals in collide, which take rho
+// and psi^2) is normal and the density is inside the domain of psi.  The pair
+// must be evaluated again with psi_of_rho and the full divisions where not.
+constexpr float kNormalMin = 0x1p-100f;
+__device__ __forceinline__ F2 psi_normal(F2 rho, const Phys<float>& P, bool& ok) {
+  F2 eta, om, arg;
+  psi_radicand<true>(rho, P, eta, om, arg);
+  const float lo = min3_nan(min3_nan(rho.x(), om.x(), arg.x()), min3_nan(rho.y(), om.y(), arg.y()),
+                            1.f);
+  ok = lo >= kNormalMin && max_nan(arg.x(), arg.y()) <= 1e30f;
+  return F2(mul_rn(arg.x(), rsqrt_normal(arg.x())), mul_rn(arg.y(), rsqrt_normal(arg.y())));
+}
+
+// Two steps of one strip x band.  kOdd: odd nx (the two columns of a lane are
+// not aligned to 8 bytes: copied and stored one by one).  st: the warp's
+// kTwoStages + 2 rows of shared memory.  kNormal: returns false as soon as a
+// value fails psi_normal's check; the band then has to be run again with
+// kNormal = false.
+template <int SCHEME, bool kOdd, bool kNormal>
+__device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int strip, int band,
+                                              int lane, TwoRow* st) {
+  constexpr bool kNeedPsi = SCHEME != kNoForce;
+  const unsigned FULL = 0xffffffffu;
+  const int nx = A.nx, ny = A.ny;
+  const int y0 = A.y_begin + band * A.band_rows;
+  const int y1 = min(y0 + A.band_rows, A.y_end);
+  const int xo = strip * kTwoCols - kTwoHalo + 2 * lane;  // left column of this lane
+  // loaded columns, wrapped (even nx: the pair stays adjacent and aligned)
+  const int ca = ((xo % nx) + nx) % nx;
+  const int cb = ca + 1 == nx ? 0 : ca + 1;
+  // columns whose step-1 and step-2 densities are the lattice's
+  const bool valid1 = lane >= 1 && lane < 31, valid2 = lane >= 2 && lane < 30;
+  const bool store_a = valid2 && xo < nx, store_b = valid2 && xo + 1 < nx;
+  bool bad = false;  // a density outside the domain of psi
+  bool fine = true;  // kNormal: every check held so far
+
+  // Rows are fetched in sequence.  om, oz, op: byte offsets of the lane's
+  // pair in the rows before, at and after the pulled row (a plane has at most
+  // 2^30 elements, so 32 bits hold them).
+  auto wrap_row = [ny](int y) { return ((y % ny) + ny) % ny; };
+  int nrow = wrap_row(y0 - 2);  // the row after the next pulled one
+  unsigned om = (unsigned(wrap_row(y0 - 4)) * unsigned(nx) + unsigned(ca)) * 4u;
+  unsigned oz = (unsigned(wrap_row(y0 - 3)) * unsigned(nx) + unsigned(ca)) * 4u;
+  auto fetch = [&](TwoRow& R) {
+    const unsigned op = (unsigned(nrow) * unsigned(nx) + unsigned(ca)) * 4u;
+#pragma unroll
+    for (int a = 0; a < kQ; ++a) {
+      const unsigned o = ey_of(a) == 0 ? oz : (ey_of(a) == 1 ? om : op);
+      const char* p = reinterpret_cast<const char*>(A.src + a * A.plane) + o;
+      if constexpr (kOdd) {
+        cp_async<4>(&R.d[a][lane].x, p);
+        cp_async<4>(&R.d[a][lane].y, p + 4 * (cb - ca));
+      } else {
+        cp_async<8>(&R.d[a][lane], p);
+      }
+    }
+    cp_async_commit();
+    om = oz;
+    oz = op;
+    nrow = nrow + 1 == ny ? 0 : nrow + 1;
+  };
+  // pull in x of plane a's values v at the lane's two columns
+  auto pull_x = [&](int a, F2 v) {
+    const int ex = ex_of(a);
+    if (ex == 0) return v;
+    if (ex == 1) return F2(__shfl_up_sync(FULL, v.y(), 1), v.x());
+    return F2(v.y(), __shfl_down_sync(FULL, v.x(), 1));
+  };
+  auto assemble = [&](const TwoRow& R, F2 (&P)[kQ]) {
+#pragma unroll
+    for (int a = 0; a < kQ; ++a) P[a] = pull_x(a, F2(R.d[a][lane]));
+  };
+  auto rho_of = [](const F2 (&P)[kQ]) {
+    F2 r = P[0];
+#pragma unroll
+    for (int a = 1; a < kQ; ++a) r = add_rn(r, P[a]);
+    return r;
+  };
+  auto psi_row = [&](F2 r, bool valid) {
+    PsiRow p;
+    if constexpr (kNormal) {
+      bool ok;
+      p.c = psi_normal(r, A.P, ok);
+      fine = fine && (ok || !valid);
+    } else {
+      bool f = false;
+      p.c = psi_of_rho(r, A.P, f);
+      bad |= f && valid;
+    }
+    const F2 W = F2(__shfl_up_sync(FULL, p.c.y(), 1), p.c.x());
+    const F2 E = F2(p.c.y(), __shfl_down_sync(FULL, p.c.x(), 1));
+    p.d = sub_rn(E, W);
+    p.s = add_rn(E, W);
+    return p;
+  };
+  // without psi only the reciprocal of the density has to be normal
+  auto rho_check = [&](F2 r, bool valid) {
+    if constexpr (kNormal && !kNeedPsi)
+      fine = fine && ((min3_nan(r.x(), r.y(), 1.f) >= kNormalMin &&
+                       max_nan(r.x(), r.y()) <= 1.f / kNormalMin) || !valid);
+  };
+  auto force = [&](const PsiRow& m, const PsiRow& z, const PsiRow& p, F2& Fx, F2& Fy) {
+    const F2 third = F2(1.f / 3.f), twelfth = F2(1.f / 12.f);
+    const F2 sx = fma_rn(third, z.d, mul_rn(twelfth, add_rn(p.d, m.d)));
+    const F2 sy = fma_rn(third, sub_rn(p.c, m.c), mul_rn(twelfth, sub_rn(p.s, m.s)));
+    const F2 gpsi = mul_rn(F2(A.P.minus_G), z.c);
+    Fx = mul_rn(gpsi, sx);
+    Fy = mul_rn(gpsi, sy);
+  };
+  const F2 zero = F2(0.f);
+  const PsiRow none{zero, zero, zero};
+
+  const int n_rows = y1 - y0 + 6;    // pulled rows y0 - 3 .. y1 + 2
+  constexpr int D = kTwoStages - 1;  // rows in flight
+#pragma unroll
+  for (int k = 0; k < D; ++k) fetch(st[k]);  // n_rows >= 7
+  TwoRow* const qrow = st + kTwoStages;  // step 2's last two pulled rows
+
+  // In iteration k the pulled row r = y0 - 3 + k arrives.  Step 1 has its
+  // pulled row r - 1 (P0, rho0) and the psi of rows r - 2 (m1) and r - 1 (z1).
+  F2 P0[kQ], rho0 = zero;
+  PsiRow m1 = none, z1 = none;
+  // Step-1 populations already pulled in x: e_y = 0 of row r - 2 (d0: a = 0,
+  // 1, 3), e_y = 1 of rows r - 2 and r - 3 (dn, dnn: a = 2, 5, 6).
+  F2 d0[3], dn[3], dnn[3];
+  // Step 2, one row behind: densities of its pulled rows r - 4 (qrhoA) and
+  // r - 3 (qrhoB), psi of rows r - 5 (m2) and r - 4 (z2).
+  F2 qrhoA = zero, qrhoB = zero;
+  PsiRow m2 = none, z2 = none;
+#pragma unroll
+  for (int a = 0; a < kQ; ++a) P0[a] = zero;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) d0[k] = dn[k] = dnn[k] = zero;
+
+  unsigned out = (unsigned(y0) * unsigned(nx) + unsigned(xo)) * 4u;
+  int sg = 0, sf = D % kTwoStages;  // stages of row r and of row r + D
+  bool go = true;
+#pragma unroll 2
+  for (int k = 0; k <= n_rows && go; ++k) {
+    // step 2: psi of row r - 3, output row r - 4 (the first rows of the march
+    // run on values that no later row uses)
+    TwoRow& slot = qrow[k & 1];
+    {
+      const bool use = valid2 && k >= 5;
+      PsiRow p2 = none;
+      F2 Gx = zero, Gy = zero, Q0[kQ];
+      if constexpr (kNeedPsi) {
+        p2 = psi_row(qrhoB, use);
+        force(m2, z2, p2, Gx, Gy);
+      } else {
+        rho_check(qrhoB, use);
+      }
+#pragma unroll
+      for (int a = 0; a < kQ; ++a) Q0[a] = F2(slot.d[a][lane]);
+      collide<SCHEME, kNormal>(Q0, qrhoA, Gx, Gy, z2.c, A.P);
+      if (store_a && k >= 7) {
+#pragma unroll
+        for (int a = 0; a < kQ; ++a) {
+          float* const at =
+              reinterpret_cast<float*>(reinterpret_cast<char*>(A.dst + a * A.plane) + out);
+          if constexpr (kOdd) {
+            at[0] = Q0[a].x();
+            if (store_b) at[1] = Q0[a].y();
+          } else {
+            *reinterpret_cast<float2*>(at) = Q0[a].v;
+          }
+        }
+      }
+      if (k >= 7) out += unsigned(nx) * 4u;
+      m2 = z2;
+      z2 = p2;
+    }
+    // step 1: row r arrives (the last iteration only completes step 2)
+    cp_async_wait<D - 1>();
+    F2 P1[kQ];
+    assemble(st[sg], P1);
+    sg = sg == kTwoStages - 1 ? 0 : sg + 1;
+    if (k + D < n_rows) fetch(st[sf]);  // into the stage read in iteration k - 1
+    else cp_async_commit();             // an empty group keeps the count per row
+    sf = sf == kTwoStages - 1 ? 0 : sf + 1;
+    const F2 rho1 = rho_of(P1);
+    PsiRow p1 = none;
+    F2 Fx = zero, Fy = zero;
+    if constexpr (kNeedPsi) {
+      p1 = psi_row(rho1, valid1 && k < n_rows);
+      force(m1, z1, p1, Fx, Fy);
+    } else {
+      rho_check(rho1, valid1 && k < n_rows);
+    }
+    collide<SCHEME, kNormal>(P0, rho0, Fx, Fy, z1.c, A.P);  // row r - 1
+    // step 2's pulled row r - 2 is complete
+    F2 Q1[kQ];
+    Q1[0] = d0[0];
+    Q1[1] = d0[1];
+    Q1[3] = d0[2];
+    Q1[2] = dnn[0];
+    Q1[5] = dnn[1];
+    Q1[6] = dnn[2];
+    Q1[4] = P0[4];
+    Q1[7] = pull_x(7, P0[7]);
+    Q1[8] = pull_x(8, P0[8]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) dnn[j] = dn[j];
+    dn[0] = P0[2];
+    dn[1] = pull_x(5, P0[5]);
+    dn[2] = pull_x(6, P0[6]);
+    d0[0] = P0[0];
+    d0[1] = pull_x(1, P0[1]);
+    d0[2] = pull_x(3, P0[3]);
+    qrhoA = qrhoB;
+    qrhoB = rho_of(Q1);
+#pragma unroll
+    for (int a = 0; a < kQ; ++a) slot.d[a][lane] = Q1[a].v;
+    m1 = z1;
+    z1 = p1;
+    rho0 = rho1;
+#pragma unroll
+    for (int a = 0; a < kQ; ++a) P0[a] = P1[a];
+    if constexpr (kNormal) go = __all_sync(FULL, fine);
+  }
+  cp_async_wait<0>();
+  if constexpr (!kNormal)
+    if (__any_sync(FULL, bad) && lane == 0) atomicOr(A.status, kStatusDiverged);
+  return go;
+}
+
+// The band again with the full divisions and domain checks (rare).
+template <int SCHEME, bool kOdd>
+__device__ __noinline__ void strip_run_two_general(const StripArgs<StoreF32>& A, int strip,
+                                                   int band, int lane, TwoRow* st) {
+  strip_run_two<SCHEME, kOdd, false>(A, strip, band, lane, st);
+}
+
+template <int SCHEME, bool kOdd>
+__global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
+two_step_kernel(const __grid_constant__ StripArgs<StoreF32> A) {
+  __shared__ TwoRow rows[kTwoStages + 2];
+  const int lane = threadIdx.x;
+  const int strip = blockIdx.x % A.n_strips;  // strips of kTwoCols columns
+  const int band = blockIdx.x / A.n_strips;
+  if (!strip_run_two<SCHEME, kOdd, true>(A, strip, band, lane, rows))
+    strip_run_two_general<SCHEME, kOdd>(A, strip, band, lane, rows);
+}
+
+}  // namespace lbm

@@ -1,0 +1,86 @@
+"""The two-step launches of the automatic kernel choice against the one-step,
+one-column kernel (VARIANT_REGISTER): the same populations, bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1204_4098_gb300 import inputs, lbm
+
+pytestmark = pytest.mark.gpu
+
+T = 0.9
+SCHEMES = [lbm.SC, lbm.EDM, lbm.IMPROVED, lbm.NOFORCE, lbm.EDM_MOD, lbm.LADD, lbm.MRT]
+
+
+def field(nx, ny, seed):
+    g, l, _ = lbm.maxwell(lbm.temperature(T))
+    rng = np.random.default_rng(seed)
+    rho = inputs.spinodal(nx, ny, 0.5 * (g + l), amp=0.02, seed=seed)
+    return rho, rng.uniform(-0.02, 0.02, (ny, nx)), rng.uniform(-0.02, 0.02, (ny, nx))
+
+
+def populations(nx, ny, state, steps, scheme, variant):
+    with lbm.Lattice(nx, ny, T) as lat:
+        lat.set_variant(variant)
+        lat.set_mrt_rates(0.8, 1.1, 1.3)
+        lat.init_density(*state)
+        st = lat.step(steps, scheme, 0.8, 0.1, raise_on_error=False)
+        return st, lat.populations()
+
+
+def check(nx, ny, state, steps, scheme):
+    st_a, auto = populations(nx, ny, state, steps, scheme, lbm.VARIANT_AUTO)
+    st_r, ref = populations(nx, ny, state, steps, scheme, lbm.VARIANT_REGISTER)
+    assert st_a == st_r
+    return auto, ref
+
+
+# around the 56 columns of a strip and its 64 loaded ones, widths and heights
+# below the halo (wrapped several times), odd and even, bands of one row to many
+@pytest.mark.parametrize("nx,ny", [
+    (1, 31001), (2, 15500), (3, 10400), (8, 4000), (9, 3500), (55, 600), (56, 600), (57, 601),
+    (64, 512), (111, 300), (112, 300), (113, 301), (176, 176), (177, 179), (4099, 9), (4100, 8),
+    (8000, 4), (10400, 3), (15501, 2), (31000, 1), (31001, 1), (640, 333)])
+@pytest.mark.parametrize("steps", [2, 5])
+def test_sizes(nx, ny, steps):
+    auto, ref = check(nx, ny, field(nx, ny, nx + ny), steps, lbm.IMPROVED)
+    assert np.array_equal(auto, ref)
+
+
+@pytest.mark.parametrize("scheme", SCHEMES)
+@pytest.mark.parametrize("nx,ny", [(200, 190), (333, 150)])
+def test_schemes_and_step_graphs(scheme, nx, ny):
+    # 35 steps: two replays of a graph of 16, one two-step launch, one step
+    auto, ref = check(nx, ny, field(nx, ny, 5), 35, scheme)
+    assert np.array_equal(auto, ref)
+
+
+@pytest.mark.parametrize("rows", [slice(None), slice(100, 140)])
+@pytest.mark.parametrize("scheme", [lbm.IMPROVED, lbm.NOFORCE])
+def test_densities_that_take_the_full_divisions(rows, scheme):
+    # 1e-32 is inside the domain of psi but below the range in which the
+    # reciprocals are taken without subnormal handling
+    nx, ny = 190, 240
+    rho = np.full((ny, nx), 0.1)
+    rho[rows] = 1e-32 * np.random.default_rng(1).uniform(1.0, 2.0, rho[rows].shape)
+    auto, ref = check(nx, ny, (rho,), 2, scheme)
+    assert np.array_equal(auto, ref, equal_nan=True)
+
+
+def test_divergence_is_reported_in_either_step_of_a_launch():
+    nx = ny = 192
+    rho, ux, uy = field(nx, ny, 3)
+    with lbm.Lattice(nx, ny, T) as lat:
+        lat.init_density(rho, ux, uy)
+        good = lat.populations()
+    for bad_steps in (1, 2):  # a population lost at the start, or one that leaves later
+        f = good.copy()
+        f[1, 50, 60] = np.nan if bad_steps == 1 else 0.9
+        for variant in (lbm.VARIANT_AUTO, lbm.VARIANT_REGISTER):
+            with lbm.Lattice(nx, ny, T) as lat:
+                lat.set_variant(variant)
+                lat.set_populations(f)
+                st = lat.step(2, lbm.SC, 0.8, raise_on_error=False)
+                assert st == lbm.LBM_E_DIVERGED
+                # the context stays usable
+                lat.set_populations(good)
+                assert lat.step(4, lbm.SC, 0.8, raise_on_error=False) == lbm.LBM_OK
