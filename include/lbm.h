@@ -292,8 +292,10 @@ lbm_status lbm_get_kernel_variant(lbm_ctx *ctx, int *variant);
  * owns whole instances and synchronises only its own threads between steps;
  * COOPERATIVE: one cooperative launch per window (every CTA resident) whose
  * warps take the work-list items of each step and meet at a bounded grid
- * barrier between steps (LBM_E_TIMEOUT if it ever gives up).  AUTO times the
- * candidates on live windows and keeps the fastest.  After every window an FP64 reduction per instance gives the
+ * barrier between steps (LBM_E_TIMEOUT if it ever gives up).  AUTO advances
+ * every active instance two steps per launch (one launch for all of them) and
+ * times a few band heights on live windows to keep the fastest; with the
+ * REGISTER variant it times the modes above instead.  After every window an FP64 reduction per instance gives the
  * coexistence densities of the flat interface (Eq. 36 slab: rho_g from rows
  * 0 and ny-1, rho_l from rows ny/2-1 and ny/2), the interface width
  * (rho_l - rho_g) / max_y |d rho_row / dy|, the mass, and the largest density
@@ -318,8 +320,10 @@ typedef struct {
  * BALANCED: per step and class, one wave of resident warps, each taking an
  * equal share of all the class's rows (the rows of every strip laid end to
  * end and cut into equal pieces, at least 8 rows each; rows_per_item does
- * not apply).  AUTO times the candidates on live windows and keeps the
- * fastest.  Every mode gives the same results bit for bit. */
+ * not apply).  AUTO: two steps per launch for all active instances, with a band
+ * height timed on live windows (reported as WORKLIST with that height); with
+ * the REGISTER variant, the fastest of the modes above.  Every mode gives the
+ * same results bit for bit. */
 enum { LBM_BATCH_AUTO = 0, LBM_BATCH_WORKLIST = 1, LBM_BATCH_PERSISTENT = 2,
        LBM_BATCH_COOPERATIVE = 3, LBM_BATCH_WORKLIST_DYNAMIC = 4, LBM_BATCH_BALANCED = 5 };
 /* Convergence rules.  CELL: every cell changed by less than
@@ -344,6 +348,8 @@ enum { LBM_BATCH_AUTO = 0, LBM_BATCH_WORKLIST = 1, LBM_BATCH_PERSISTENT = 2,
  * convergence, warm against cold starts). */
 enum { LBM_CONV_COEX = 0, LBM_CONV_CELL = 1, LBM_CONV_NONE = 2 /* run to max_steps */,
        LBM_CONV_TREND = 3 };
+/* An instance that diverges has its verdict at the end of the window; its state
+ * and the other values of its result are then unspecified. */
 enum { LBM_RUN_ACTIVE = 0, LBM_RUN_CONVERGED = 1, LBM_RUN_DIVERGED = 2, LBM_RUN_CAPPED = 3 };
 
 typedef struct {

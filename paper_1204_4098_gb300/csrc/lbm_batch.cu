@@ -9,8 +9,9 @@
 // column, the other two by the lanes holding columns 1 and 2), so pairs stay
 // aligned and the last column meets its periodic neighbours.  Instances fall
 // in two classes by body, each with kernels of its own (separate register
-// budgets).  A window of `window` steps is one CUDA graph, in one of
-// three launch modes:
+// budgets).  A window of `window` steps is one CUDA graph.  By default it is
+// two-step launches over one list of items for all instances
+// (batch_two_step_kernel); the launch modes that can be asked for are
 //   work list   -- per step, one launch per class; warps take strip x band
 //                  items of the class's active instances from a prefix table
 //                  (balanced for any mix of sizes); the two class kernels are
@@ -43,6 +44,7 @@
 #include "lbm_batch_host.h"
 #include "lbm_internal.h"
 #include "lbm_kernels.cuh"
+#include "lbm_two_step.cuh"
 
 namespace lbm {
 
@@ -228,6 +230,82 @@ batch_balanced_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
     }
     __syncwarp();
     run_item<kPair, false>(args[warp], I.scheme, it.y, 0, lane);
+  }
+}
+
+// Two steps of every active instance in one launch (strip_run_two): CTA b (one
+// warp) runs items[b], a row range of one strip -- of the whole width, in two
+// halves where half-warps take a band each.  The items are sorted longest
+// first, so the launch's last CTAs are its shortest; grids are rounded up
+// (CTAs past the end leave) to keep the number of captured graphs small.
+// Every forced scheme runs as kBlend: one body without scheme branches.
+//
+// Against the work list it halves the traffic and the launches, keeps 12
+// warps per SM in flight whatever the item lengths, and gives lattices of up
+// to 64 even columns whole rows (the work list's 64-column strips leave half
+// of a 32-column lattice's lanes idle).  Measured, us per step, best work-list
+// or balanced mode -> this: 96 slabs of 32 columns 31.3 -> 11.4 (95k MLUPS),
+// 600 of them 148 -> 44.2, 48 mixed slabs (4.7 M cells) 79 -> 48.1, 128 mixed
+// slabs 179 -> 104 (110k MLUPS), 2 slabs 14.2 -> 6.1.  Bound by the latency
+// and issue of its instructions, like two_step_kernel.
+template <int SCHEME, int LAYOUT>
+__device__ __noinline__ void batch_two_general(const StripArgs<StoreF32>& A, int strip, int lane,
+                                               TwoRow* rows) {
+  if constexpr (SCHEME == kNoForce)
+    if (strip_run_two<kNoForce, LAYOUT, true>(A, strip, 0, lane, rows)) return;
+  strip_run_two<SCHEME, LAYOUT, false>(A, strip, 0, lane, rows);
+}
+
+template <int LAYOUT>
+__device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int scheme, int strip,
+                                               int lane, TwoRow* rows,
+                                               StripArgs<StoreF32>& shared) {
+  if (scheme != kNoForce && strip_run_two<kBlend, LAYOUT, true>(A, strip, 0, lane, rows)) return;
+  if (lane == 0) shared = A;
+  __syncwarp();
+  if (scheme == kNoForce)
+    batch_two_general<kNoForce, LAYOUT>(shared, strip, lane, rows);
+  else
+    batch_two_general<kAnyForced, LAYOUT>(shared, strip, lane, rows);
+}
+
+__global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
+batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict__ items,
+                      const int* __restrict__ n_items, const float* src, float* dst,
+                      unsigned* inst_status) {
+  __shared__ TwoRow rows[kTwoStages + 2];
+  __shared__ StripArgs<StoreF32> shared;
+  const int lane = threadIdx.x;
+  if (int(blockIdx.x) >= *n_items) return;
+  const int4 it = items[blockIdx.x];  // instance, strip, first row, end row
+  const int i = it.x;
+  // An instance that has left the domain of psi has its verdict; its state is
+  // of no further use and is not advanced.
+  if (inst_status[i] & kStatusDiverged) return;
+  const BatchInst& I = inst[i];
+  StripArgs<StoreF32> A;  // (field by field: a copy of the whole record spills)
+  A.src = src + I.off;
+  A.dst = dst + I.off;
+  A.status = inst_status + i;
+  A.nx = I.nx;
+  A.ny = I.ny;
+  A.pitch = I.pitch;
+  A.plane = size_t(I.pitch) * I.ny;
+  A.P = I.P;
+  A.y_begin = it.z;
+  A.y_end = it.w;
+  A.band_rows = it.w - it.z;
+  const int strip = it.y;
+  if (A.nx <= 64 && A.nx % 2 == 0) {
+    if (A.nx <= 32) A.band_rows = (A.band_rows + 1) / 2;
+    batch_two_item<kRing>(A, A.P.scheme, strip, lane, rows, shared);
+  } else if (A.nx % 2 == 0) {
+    batch_two_item<kFlatEven>(A, A.P.scheme, strip, lane, rows, shared);
+  } else {
+    if (A.pitch == A.nx)  // nx = 1
+      batch_two_item<kFlatOdd>(A, A.P.scheme, strip, lane, rows, shared);
+    else
+      batch_two_item<kPadOdd>(A, A.P.scheme, strip, lane, rows, shared);
   }
 }
 
@@ -550,6 +628,11 @@ struct lbm_batch {
   int4* h_bal_items = nullptr;
   int* h_bal_begin = nullptr;
   int bal_cap = 0;               // items per class table
+  int4* d_two_items = nullptr;   // two-step windows: items and their number
+  int* d_two_count = nullptr;
+  int4* h_two_items = nullptr;
+  int* h_two_count = nullptr;
+  int two_cap = 0;
   int* h_active = nullptr;
   int* h_prefix = nullptr;
   int* h_cta_begin = nullptr;
@@ -567,9 +650,9 @@ struct lbm_batch {
   unsigned* d_sync = nullptr;    // grid barrier: arrivals, generation, error
   cudaStream_t side = nullptr;   // second branch of the window graph
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  // window graphs by (mode, grid of the two-column kernel, grid of the
-  // one-column kernel); a grid of 0 leaves that class's kernel out
-  std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;
+  // window graphs by (mode, grid of the two-step kernel, grid of the two-column
+  // kernel, grid of the one-column kernel); a grid of 0 leaves a kernel out
+  std::map<std::tuple<int, int, int, int>, cudaGraphExec_t> graphs;
   int class_items[2] = {0, 0};  // work-list items of the active instances per class
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   bool initialized = false;
@@ -619,10 +702,30 @@ void set_geometry(BatchInst& d, int rows) {
 
 constexpr int kBalancedMinRows = 8;
 
+// Internal window mode: two steps per launch (LBM_BATCH_AUTO; reported as a
+// work list).
+constexpr int kBatchTwoStep = 100;
+constexpr int kTwoMinRows = 4;  // shortest band of a two-step window
+
+// AUTO runs two-step windows, unless one column per lane was asked for or the
+// covolume is outside the range of two_step_applies.  (A window of fewer than
+// four steps has no even number of two-step launches.)
+bool two_step_windows(const lbm_batch* b) {
+  return b->p.mode == LBM_BATCH_AUTO && b->p.variant != LBM_VARIANT_REGISTER &&
+         b->p.window >= 4 && b->p.b > 1e-12 && b->p.b < 1e12;
+}
+
+std::vector<TwoLattice> two_lattices(const lbm_batch* b) {
+  std::vector<TwoLattice> lat;
+  lat.reserve(b->active.size());
+  for (int i : b->active) lat.push_back(TwoLattice{i, b->desc[i].nx, b->desc[i].ny});
+  return lat;
+}
+
 // Rebuild the active list (two-column instances first), the work-list prefix
 // and the persistent assignment of each class; for a balanced window also
 // each class's one-wave schedule.
-lbm_status upload_tables(lbm_batch* b, int mode) {
+lbm_status upload_tables(lbm_batch* b, int mode, int rows) {
   const int na = int(b->active.size());
   std::vector<int> cls[2];  // [0] two columns per lane, [1] one
   for (int i : b->active) cls[b->desc[i].pair ? 0 : 1].push_back(i);
@@ -659,6 +762,18 @@ lbm_status upload_tables(lbm_batch* b, int mode) {
                                b->stream));
   LBM_BCUDA(b, cudaMemcpyAsync(b->d_cta_list, b->h_cta_list, std::max(pos, 1) * sizeof(int),
                                cudaMemcpyHostToDevice, b->stream));
+  if (mode == kBatchTwoStep) {
+    std::vector<TwoItem> items;
+    two_items(two_lattices(b), rows, items);
+    const int n = int(items.size());
+    *b->h_two_count = n;
+    static_assert(sizeof(TwoItem) == sizeof(int4), "an item is one 16-byte load");
+    std::memcpy(b->h_two_items, items.data(), n * sizeof(TwoItem));
+    LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_items, b->h_two_items, n * sizeof(int4),
+                                 cudaMemcpyHostToDevice, b->stream));
+    LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_count, b->h_two_count, sizeof(int),
+                                 cudaMemcpyHostToDevice, b->stream));
+  }
   if (mode == LBM_BATCH_BALANCED)
     for (int c = 0; c < 2; ++c) {
       std::vector<BalColumn> cols;
@@ -692,9 +807,16 @@ int class_grid(const lbm_batch* b, int mode, int cls) {
 // so the graph stays valid as instances leave.
 lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
   const bool coop = mode == LBM_BATCH_COOPERATIVE;
-  const int g0 = coop ? b->coop_grid : class_grid(b, mode, 0);
-  const int g1 = coop ? 0 : class_grid(b, mode, 1);
-  const auto key = std::make_tuple(mode, g0, g1);
+  const int W = b->p.window;
+  // Two-step windows: an even number of two-step launches, so that the state
+  // ends in buf[0]; the two steps left over where W / 2 is odd go one by one.
+  const bool two = mode == kBatchTwoStep;
+  const int two_launches = two ? W / 4 * 2 : 0;
+  const int two_grid = two ? two_item_grid(*b->h_two_count) : 0;
+  const bool singles = !two || W % 4 != 0;
+  const int g0 = coop ? b->coop_grid : (singles ? class_grid(b, mode, 0) : 0);
+  const int g1 = coop || !singles ? 0 : class_grid(b, mode, 1);
+  const auto key = std::make_tuple(mode, two_grid, g0, g1);
   const auto it = b->graphs.find(key);
   if (it != b->graphs.end()) {
     *out = it->second;
@@ -702,7 +824,6 @@ lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
   }
   cudaGraph_t g = nullptr;
   LBM_BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-  const int W = b->p.window;
   const int span = b->pers_grid_max + 1;
   // with both classes active they run as two branches of the graph, joined
   // after each step (work list) or before the reduction (persistent).  (Run
@@ -745,8 +866,12 @@ lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
       cudaGetLastError();
       return bfail(b, LBM_E_CUDA, std::string("cooperative launch: ") + cudaGetErrorString(le));
     }
-  } else if (mode == LBM_BATCH_WORKLIST) {
-    for (int s = 0; s < W; ++s) {
+  } else if (mode == LBM_BATCH_WORKLIST || two) {
+    for (int s = 0; s < two_launches; ++s)
+      batch_two_step_kernel<<<two_grid, kTwoThreads, 0, b->stream>>>(
+          b->d_inst, b->d_two_items, b->d_two_count, b->buf[s & 1], b->buf[(s + 1) & 1],
+          b->d_status);
+    for (int s = 2 * two_launches; s < W; ++s) {
       fork();
       if (g0 > 0)
         batch_worklist_kernel<true><<<g0, kWorklistThreads, 0, b->stream>>>(
@@ -839,6 +964,21 @@ void choose_config(lbm_batch* b, int& mode, int& rows) {
     return;
   }
   const size_t cells = active_cells(b);
+  if (two_step_windows(b)) {
+    mode = kBatchTwoStep;
+    if (b->p.rows_per_item > 0) {
+      rows = std::max(b->p.rows_per_item, kTwoMinRows);
+      return;
+    }
+    // the two or three candidate heights around the model's choice compete
+    const int model = two_item_rows(two_lattices(b), b->sm_count);
+    const auto near = [&](size_t k) {
+      const double r = b->tuner.candidates[k].second;
+      return r >= 0.6 * model && r <= 1.7 * model;
+    };
+    rows = b->tuner.choose(cells, near).second;
+    return;
+  }
   const auto eligible = [&](size_t k) {
     const auto& c = b->tuner.candidates[k];
     if (b->p.rows_per_item > 0 &&
@@ -937,6 +1077,7 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
     d.P.guo = float(1.0 - 1.0 / (2.0 * s.tau));
     d.P.scheme = s.scheme;
     d.P.s_e = d.P.s_eps = d.P.s_q = d.P.omega;  // unused: the batch has no MRT scheme
+    blend_coefficients(s.scheme, s.tau, d.P);
     set_geometry(d, 32);
     const size_t cells = size_t(s.nx) * s.ny;
     off += (9 * size_t(d.pitch) * s.ny + 31) / 32 * 32;
@@ -1003,7 +1144,17 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
     ok &= cudaMalloc(&b->d_bal_begin, 2 * size_t(warps_max(b) + 1) * sizeof(int)) ==
           cudaSuccess;
   }
+  {
+    long long items = 0;
+    for (const BatchInst& d : b->desc)
+      items += (long long)two_item_strips(d.nx) * two_item_bands(d.nx, d.ny, kTwoMinRows);
+    b->two_cap = int(items);
+    ok &= cudaMalloc(&b->d_two_items, size_t(b->two_cap) * sizeof(int4)) == cudaSuccess;
+    ok &= cudaMalloc(&b->d_two_count, sizeof(int)) == cudaSuccess;
+  }
   if (!ok) return bail(LBM_E_NOMEM, "cudaMalloc");
+  ok &= cudaMallocHost(&b->h_two_items, size_t(b->two_cap) * sizeof(int4)) == cudaSuccess;
+  ok &= cudaMallocHost(&b->h_two_count, sizeof(int)) == cudaSuccess;
   ok &= cudaMallocHost(&b->h_active, count * sizeof(int)) == cudaSuccess;
   ok &= cudaMallocHost(&b->h_prefix, (count + 3) * sizeof(int)) == cudaSuccess;
   ok &= cudaMallocHost(&b->h_cta_begin, 2 * (b->pers_grid_max + 1) * sizeof(int)) ==
@@ -1025,10 +1176,16 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
       cudaMemsetAsync(b->buf[1], 0, off * sizeof(float), b->stream) != cudaSuccess ||
       cudaStreamSynchronize(b->stream) != cudaSuccess)
     return bail(LBM_E_CUDA, "memset");
-  for (int rows : {8, 16, 32, 64, 128}) b->tuner.add(LBM_BATCH_WORKLIST, rows);
-  for (int rows : {8, 16, 32, 64}) b->tuner.add(LBM_BATCH_WORKLIST_DYNAMIC, rows);
-  b->tuner.add(LBM_BATCH_BALANCED, 0);
-  b->tuner.add(LBM_BATCH_PERSISTENT, 0);
+  const bool two = two_step_windows(b);
+  if (two) {
+    for (int rows : {4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256})
+      b->tuner.add(kBatchTwoStep, rows);
+  } else {
+    for (int rows : {8, 16, 32, 64, 128}) b->tuner.add(LBM_BATCH_WORKLIST, rows);
+    for (int rows : {8, 16, 32, 64}) b->tuner.add(LBM_BATCH_WORKLIST_DYNAMIC, rows);
+    b->tuner.add(LBM_BATCH_BALANCED, 0);
+    b->tuner.add(LBM_BATCH_PERSISTENT, 0);
+  }
   {
     // cooperative windows: every CTA resident, one launch per window
     int coop = 0, occ = 0;
@@ -1039,7 +1196,7 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
         occ > 0)
       b->coop_grid = occ * b->sm_count;
     cudaGetLastError();
-    if (b->coop_grid > 0)
+    if (b->coop_grid > 0 && !two)
       for (int rows : {16, 32, 64}) b->tuner.add(LBM_BATCH_COOPERATIVE, rows);
   }
   for (int i = 0; i < count; ++i) b->active.push_back(i);
@@ -1072,6 +1229,10 @@ lbm_status lbm_batch_destroy(lbm_batch* b) {
   cudaFree(b->d_sync);
   cudaFree(b->d_bal_items);
   cudaFree(b->d_bal_begin);
+  cudaFree(b->d_two_items);
+  cudaFree(b->d_two_count);
+  if (b->h_two_items) cudaFreeHost(b->h_two_items);
+  if (b->h_two_count) cudaFreeHost(b->h_two_count);
   if (b->h_bal_items) cudaFreeHost(b->h_bal_items);
   if (b->h_bal_begin) cudaFreeHost(b->h_bal_begin);
   if (b->h_active) cudaFreeHost(b->h_active);
@@ -1214,7 +1375,7 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     int mode = LBM_BATCH_WORKLIST, rows = 32;
     choose_config(b, mode, rows);
     for (auto& d : b->desc) set_geometry(d, rows > 0 ? rows : 32);
-    lbm_status st = upload_tables(b, mode);
+    lbm_status st = upload_tables(b, mode, rows);
     if (st != LBM_OK) return st;
     cudaGraphExec_t g = nullptr;
     st = window_graph(b, mode, &g);
@@ -1230,16 +1391,17 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     LBM_BCUDA(b, cudaEventRecord(b->ev0, b->stream));
     LBM_BCUDA(b, cudaGraphLaunch(g, b->stream));
     LBM_BCUDA(b, cudaEventRecord(b->ev1, b->stream));
-    // two class kernels per step (work list) or per window (persistent), and
-    // the reduction
-    // (one cooperative kernel per window)
-    const unsigned long long kernels =
-        mode == LBM_BATCH_COOPERATIVE
-            ? 1
-            : (class_grid(b, mode, 0) > 0 ? 1 : 0) + (class_grid(b, mode, 1) > 0 ? 1 : 0);
-    const bool per_step = mode == LBM_BATCH_WORKLIST || mode == LBM_BATCH_WORKLIST_DYNAMIC ||
-                          mode == LBM_BATCH_BALANCED;
-    const unsigned long long nl = (per_step ? kernels * b->p.window : kernels) + 1;
+    // two class kernels per step (work list) or per window (persistent), one
+    // kernel per two steps (two-step) or per window (cooperative), and the
+    // reduction
+    const unsigned long long classes =
+        (class_grid(b, mode, 0) > 0 ? 1 : 0) + (class_grid(b, mode, 1) > 0 ? 1 : 0);
+    const unsigned long long W = b->p.window;
+    const unsigned long long nl =
+        1 + (mode == kBatchTwoStep           ? W / 4 * 2 + (W % 4 ? 2 * classes : 0)
+             : mode == LBM_BATCH_COOPERATIVE ? 1
+             : mode == LBM_BATCH_PERSISTENT  ? classes
+                                             : classes * W);
     count_launches(nl);
     b->stats.launches += nl;
     LBM_BCUDA(b, cudaMemcpyAsync(b->h_out, b->d_out, b->count * sizeof(BatchOut),
@@ -1256,7 +1418,7 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     LBM_BCUDA(b, cudaEventElapsedTime(&ms, b->ev0, b->ev1));
     b->stats.gpu_ms += ms;
     b->stats.windows += 1;
-    b->stats.mode = mode;
+    b->stats.mode = mode == kBatchTwoStep ? int(LBM_BATCH_WORKLIST) : mode;
     b->stats.rows_per_item = rows;
     if (b->p.mode == LBM_BATCH_AUTO)
       b->tuner.record(mode, rows, ms * 1e6 / (double(cells) * b->p.window));

@@ -110,6 +110,85 @@ inline int balanced_schedule(const std::vector<BalColumn>& cols, int warps, int 
   return n;
 }
 
+// Two-step windows (one CTA of one warp per item): the items of the active
+// lattices, each a row range [y0, y1) of one strip.
+struct TwoItem {
+  int inst, strip, y0, y1;
+};
+struct TwoLattice {
+  int inst, nx, ny;
+};
+constexpr int kTwoItemCols = 56;  // columns of a strip
+
+// A lattice of at most 64 even columns is one strip of whole rows; up to 32
+// columns a warp takes two bands of it at once.
+inline bool two_item_ring(int nx) { return nx % 2 == 0 && nx <= 64; }
+inline int two_item_strips(int nx) {
+  return two_item_ring(nx) ? 1 : (nx + kTwoItemCols - 1) / kTwoItemCols;
+}
+// Items over the height of one strip for bands of `rows` rows.
+inline int two_item_bands(int nx, int ny, int rows) {
+  const int span = two_item_ring(nx) && nx <= 32 ? 2 * rows : rows;
+  return (ny + span - 1) / span;
+}
+
+// Items for bands of about `rows` rows (each strip cut evenly), longest first.
+inline void two_items(const std::vector<TwoLattice>& lat, int rows, std::vector<TwoItem>& out) {
+  out.clear();
+  for (const TwoLattice& t : lat) {
+    const int n = two_item_bands(t.nx, t.ny, rows), strips = two_item_strips(t.nx);
+    for (int b = 0; b < n; ++b)
+      for (int s = 0; s < strips; ++s)
+        out.push_back(TwoItem{t.inst, s, int((long long)t.ny * b / n),
+                              int((long long)t.ny * (b + 1) / n)});
+  }
+  std::stable_sort(out.begin(), out.end(), [](const TwoItem& x, const TwoItem& y) {
+    return x.y1 - x.y0 > y.y1 - y.y0;
+  });
+}
+
+// CTAs launched for `items` items: rounded up in steps of an eighth of the
+// leading power of two, so that a shrinking active set needs few graphs.
+inline int two_item_grid(int items) {
+  int step = 64;
+  while (step * 16 <= items) step <<= 1;
+  return (items + step - 1) / step * step;
+}
+
+// Band height of a two-step launch over the active lattices, to start the
+// tuning from.  An item of n rows runs n + 7 iterations, of about 0.70, 1.10
+// or 1.45 us with 1, 2 or 3 warps per scheduler.  All items resident: the
+// launch ends with its longest; more items than resident warps: with the
+// work, plus the last items' share.
+inline int two_item_rows(const std::vector<TwoLattice>& lat, int sm_count) {
+  const double iter[3] = {0.70, 1.10, 1.45};
+  const double resident = 12.0 * sm_count;
+  int best_rows = 32;
+  double best = 0.0;
+  for (int rows : {4, 5, 6, 7, 8, 9, 10, 11, 12, 14, 16, 18, 20, 23, 26, 30, 34, 39, 45, 52, 60, 69,
+                   80, 92, 106, 122, 140, 161, 185, 213, 256}) {
+    double items = 0.0, work = 0.0, longest = 0.0;
+    for (const TwoLattice& t : lat) {
+      const int n = two_item_bands(t.nx, t.ny, rows), strips = two_item_strips(t.nx);
+      const int halves = two_item_ring(t.nx) && t.nx <= 32 ? 2 : 1;
+      const double len = std::ceil(std::ceil(double(t.ny) / n) / halves) + 7.0;
+      items += double(n) * strips;
+      work += double(n) * strips * len;
+      longest = std::max(longest, len);
+    }
+    double t;
+    if (items <= resident)
+      t = longest * iter[items * 3 <= resident ? 0 : (items * 3 <= 2 * resident ? 1 : 2)];
+    else
+      t = (work / resident + 0.5 * longest) * iter[2];
+    if (best == 0.0 || t < best) {
+      best = t;
+      best_rows = rows;
+    }
+  }
+  return best_rows;
+}
+
 // Window-level autotuner.  Each candidate (mode, rows) is timed on one live
 // window, the cheapest per cell update is kept, and tuning starts again once
 // the active work has halved or the chosen candidate has become 30 % dearer

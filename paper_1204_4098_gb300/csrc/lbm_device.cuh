@@ -128,6 +128,7 @@ struct Phys {
   C guo;        // 1 - 1 / (2 tau)  (B_e = C_e of Eq. 13)
   int scheme;   // forcing scheme, read only by collide<kAnyForced>
   C s_e, s_eps, s_q;  // MRT rates of the energy, energy-square, energy-flux moments
+  C kq, kv, be, ce;   // coefficients of the scheme, read only by collide<kBlend>
 };
 
 // Reciprocal and square root for the per-cell physics.  FP64 keeps the IEEE
@@ -214,6 +215,21 @@ enum Scheme { kSC = 0, kEDM = 1, kImproved = 2, kNoForce = 3, kEDMMod = 4, kLadd
 // read from Phys::scheme at run time.  One inlined body then serves every
 // instance of a mixed batch, instead of one body per scheme.
 constexpr int kAnyForced = -1;
+// Template value: every forced scheme as one branch-free form,
+//   u_eq = u + kq F / rho,  V = u + kv F / rho + s F,  s = sigma_ups / psi^2
+// with the scheme's kq, kv, B_e, C_e in Phys (blend_coefficients) and
+// sigma_ups = 0 for all but the improved scheme.  A term a scheme does not
+// have is an exact "+ 0 x finite" here, so the values are those of the
+// scheme's own form.
+constexpr int kBlend = -2;
+inline void blend_coefficients(int scheme, double tau, Phys<float>& P) {
+  P.kq = scheme == kSC ? float(tau) : (scheme == kImproved ? 0.5f : 0.f);
+  P.kv = scheme == kSC || scheme == kLadd ? 0.f : 0.5f;
+  P.be = scheme == kSC ? 0.f : (scheme == kImproved ? P.guo : 1.f);
+  P.ce = scheme == kSC ? 0.f
+                       : (scheme == kImproved ? P.guo : (scheme == kEDMMod ? P.omega : 1.f));
+  if (scheme != kImproved) P.sigma_ups = 0.f;
+}
 
 // Every scheme of Table I is BGK towards f_eq(rho, u_eq) plus Guo's general
 // forcing term (Eq. 12) with B = B_e F and C = C_e (V F + F V):
@@ -340,7 +356,7 @@ __device__ __forceinline__ void collide(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
     }
     return;
   }
-  const int sch = SCHEME == kAnyForced ? P.scheme : SCHEME;
+  const int sch = SCHEME == kAnyForced || SCHEME == kBlend ? P.scheme : SCHEME;
   const V jx = add_rn(add_rn(sub_rn(f[1], f[3]), sub_rn(f[5], f[6])), sub_rn(f[8], f[7]));
   const V jy = sub_rn(add_rn(sub_rn(f[2], f[4]), add_rn(f[5], f[6])), add_rn(f[7], f[8]));
   const V inv_rho = quot<kNormal>(V(C(1)), rho);
@@ -350,8 +366,17 @@ __device__ __forceinline__ void collide(V (&f)[kQ], V rho, V Fx, V Fy, V psi,
   V qx = ux, qy = uy;  // velocity in f_eq
   V Vx = V(C(0)), Vy = V(C(0));
   C Be = C(0), Ce = C(0);
-  const bool forcing = sch != kSC && sch != kNoForce;
-  if (sch == kSC) {
+  const bool forcing = SCHEME == kBlend || (sch != kSC && sch != kNoForce);
+  if constexpr (SCHEME == kBlend) {
+    const V tq = mul_rn(V(P.kq), inv_rho), tv = mul_rn(V(P.kv), inv_rho);
+    qx = fma_rn(tq, Fx, ux);
+    qy = fma_rn(tq, Fy, uy);
+    const V s = quot<kNormal>(V(P.sigma_ups), mul_rn(psi, psi));
+    Vx = fma_rn(s, Fx, fma_rn(tv, Fx, ux));
+    Vy = fma_rn(s, Fy, fma_rn(tv, Fy, uy));
+    Be = P.be;
+    Ce = P.ce;
+  } else if (sch == kSC) {
     const V t = mul_rn(V(P.tau), inv_rho);
     qx = fma_rn(t, Fx, ux);
     qy = fma_rn(t, Fy, uy);

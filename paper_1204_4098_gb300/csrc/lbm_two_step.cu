@@ -11,9 +11,9 @@ template <int SCHEME>
 cudaError_t launch(const StripLaunch& L, int grid, cudaStream_t s) {
   const StripArgs<StoreF32> A = make_args<StoreF32>(L);
   if (L.nx % 2)
-    two_step_kernel<SCHEME, true><<<grid, kTwoThreads, 0, s>>>(A);
+    two_step_kernel<SCHEME, kFlatOdd><<<grid, kTwoThreads, 0, s>>>(A);
   else
-    two_step_kernel<SCHEME, false><<<grid, kTwoThreads, 0, s>>>(A);
+    two_step_kernel<SCHEME, kFlatEven><<<grid, kTwoThreads, 0, s>>>(A);
   return cudaGetLastError();
 }
 

@@ -86,26 +86,66 @@ __device__ __forceinline__ F2 psi_normal(F2 rho, const Phys<float>& P, bool& ok)
   return F2(mul_rn(arg.x(), rsqrt_normal(arg.x())), mul_rn(arg.y(), rsqrt_normal(arg.y())));
 }
 
-// Two steps of one strip x band.  kOdd: odd nx (the two columns of a lane are
-// not aligned to 8 bytes: copied and stored one by one).  st: the warp's
-// kTwoStages + 2 rows of shared memory.  kNormal: returns false as soon as a
-// value fails psi_normal's check; the band then has to be run again with
-// kNormal = false.
-template <int SCHEME, bool kOdd, bool kNormal>
+// Row layouts.
+//  kFlatEven  even nx = pitch: a lane's two columns are one aligned pair;
+//  kFlatOdd   odd nx = pitch: columns copied and stored one by one;
+//  kPadOdd    odd nx, pitch nx + 3 with columns nx .. nx + 2 copying columns
+//             0 .. 2 (the batch engine's odd lattices): stored as pairs, the
+//             copies refreshed as the one-step kernels do, loaded one by one
+//             (wrapped columns are not aligned);
+//  kRing      even nx <= 64 = pitch: the warp holds whole rows, its shuffles
+//             wrap around them, and no column is computed twice.  Up to 32
+//             columns each half-warp takes a band of its own.
+enum TwoLayout { kFlatEven, kFlatOdd, kPadOdd, kRing };
+
+// Two steps of one strip x band item.  st: the warp's kTwoStages + 2 rows of
+// shared memory.  kNormal: returns false as soon as a value fails
+// psi_normal's check; the item then has to be run again with kNormal = false.
+template <int SCHEME, int LAYOUT, bool kNormal>
 __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int strip, int band,
                                               int lane, TwoRow* st) {
   constexpr bool kNeedPsi = SCHEME != kNoForce;
+  constexpr bool kOneByOne = LAYOUT == kFlatOdd || LAYOUT == kPadOdd;  // row copies of 4 bytes
   const unsigned FULL = 0xffffffffu;
   const int nx = A.nx, ny = A.ny;
-  const int y0 = A.y_begin + band * A.band_rows;
-  const int y1 = min(y0 + A.band_rows, A.y_end);
-  const int xo = strip * kTwoCols - kTwoHalo + 2 * lane;  // left column of this lane
-  // loaded columns, wrapped (even nx: the pair stays adjacent and aligned)
-  const int ca = ((xo % nx) + nx) % nx;
-  const int cb = ca + 1 == nx ? 0 : ca + 1;
-  // columns whose step-1 and step-2 densities are the lattice's
-  const bool valid1 = lane >= 1 && lane < 31, valid2 = lane >= 2 && lane < 30;
-  const bool store_a = valid2 && xo < nx, store_b = valid2 && xo + 1 < nx;
+  const unsigned pitch = LAYOUT == kPadOdd ? unsigned(A.pitch) : unsigned(nx);
+  int y0, y1, n_rows;  // rows of this lane's band; pulled rows of the march
+  int xo, ca, cb;      // left column of this lane; its loaded columns (wrapped)
+  int from_l = 0, from_r = 0;  // kRing: lanes holding the columns beside
+  bool valid1, valid2;  // the lane's step-1 / step-2 densities are the lattice's
+  bool store_a, store_b;
+  if constexpr (LAYOUT == kRing) {
+    const int width = nx / 2;                   // lanes of a row
+    const int half = nx <= 32 ? lane >> 4 : 0;  // which of the warp's bands
+    const int base = half << 4, l = lane - base;
+    const bool in_row = l < width;
+    const int b = nx <= 32 ? 2 * band + half : band;
+    y0 = A.y_begin + b * A.band_rows;
+    y1 = min(y0 + A.band_rows, A.y_end);
+    n_rows = A.band_rows + 6;
+    xo = ca = in_row ? 2 * l : 0;
+    cb = ca + 1;
+    from_l = l == 0 ? base + width - 1 : lane - 1;
+    from_r = l == width - 1 ? base : lane + 1;
+    valid1 = valid2 = in_row;
+    store_a = store_b = in_row;
+    if (y0 >= y1) {  // a half-warp without a band: marches along, stores nothing
+      y0 = A.y_begin;
+      y1 = y0;
+    }
+  } else {
+    y0 = A.y_begin + band * A.band_rows;
+    y1 = min(y0 + A.band_rows, A.y_end);
+    n_rows = y1 - y0 + 6;  // pulled rows y0 - 3 .. y1 + 2
+    xo = strip * kTwoCols - kTwoHalo + 2 * lane;
+    // (even nx: the wrapped pair stays adjacent and aligned)
+    ca = ((xo % nx) + nx) % nx;
+    cb = ca + 1 == nx ? 0 : ca + 1;
+    valid1 = lane >= 1 && lane < 31;
+    valid2 = lane >= 2 && lane < 30;
+    store_a = valid2 && xo < nx;
+    store_b = valid2 && xo + 1 < nx;
+  }
   bool bad = false;  // a density outside the domain of psi
   bool fine = true;  // kNormal: every check held so far
 
@@ -114,15 +154,15 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
   // 2^30 elements, so 32 bits hold them).
   auto wrap_row = [ny](int y) { return ((y % ny) + ny) % ny; };
   int nrow = wrap_row(y0 - 2);  // the row after the next pulled one
-  unsigned om = (unsigned(wrap_row(y0 - 4)) * unsigned(nx) + unsigned(ca)) * 4u;
-  unsigned oz = (unsigned(wrap_row(y0 - 3)) * unsigned(nx) + unsigned(ca)) * 4u;
+  unsigned om = (unsigned(wrap_row(y0 - 4)) * pitch + unsigned(ca)) * 4u;
+  unsigned oz = (unsigned(wrap_row(y0 - 3)) * pitch + unsigned(ca)) * 4u;
   auto fetch = [&](TwoRow& R) {
-    const unsigned op = (unsigned(nrow) * unsigned(nx) + unsigned(ca)) * 4u;
+    const unsigned op = (unsigned(nrow) * pitch + unsigned(ca)) * 4u;
 #pragma unroll
     for (int a = 0; a < kQ; ++a) {
       const unsigned o = ey_of(a) == 0 ? oz : (ey_of(a) == 1 ? om : op);
       const char* p = reinterpret_cast<const char*>(A.src + a * A.plane) + o;
-      if constexpr (kOdd) {
+      if constexpr (kOneByOne) {
         cp_async<4>(&R.d[a][lane].x, p);
         cp_async<4>(&R.d[a][lane].y, p + 4 * (cb - ca));
       } else {
@@ -135,11 +175,17 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
     nrow = nrow + 1 == ny ? 0 : nrow + 1;
   };
   // pull in x of plane a's values v at the lane's two columns
+  auto left = [&](float v) {
+    return LAYOUT == kRing ? __shfl_sync(FULL, v, from_l) : __shfl_up_sync(FULL, v, 1);
+  };
+  auto right = [&](float v) {
+    return LAYOUT == kRing ? __shfl_sync(FULL, v, from_r) : __shfl_down_sync(FULL, v, 1);
+  };
   auto pull_x = [&](int a, F2 v) {
     const int ex = ex_of(a);
     if (ex == 0) return v;
-    if (ex == 1) return F2(__shfl_up_sync(FULL, v.y(), 1), v.x());
-    return F2(v.y(), __shfl_down_sync(FULL, v.x(), 1));
+    if (ex == 1) return F2(left(v.y()), v.x());
+    return F2(v.y(), right(v.x()));
   };
   auto assemble = [&](const TwoRow& R, F2 (&P)[kQ]) {
 #pragma unroll
@@ -162,8 +208,8 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
       p.c = psi_of_rho(r, A.P, f);
       bad |= f && valid;
     }
-    const F2 W = F2(__shfl_up_sync(FULL, p.c.y(), 1), p.c.x());
-    const F2 E = F2(p.c.y(), __shfl_down_sync(FULL, p.c.x(), 1));
+    const F2 W = F2(left(p.c.y()), p.c.x());
+    const F2 E = F2(p.c.y(), right(p.c.x()));
     p.d = sub_rn(E, W);
     p.s = add_rn(E, W);
     return p;
@@ -185,7 +231,6 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
   const F2 zero = F2(0.f);
   const PsiRow none{zero, zero, zero};
 
-  const int n_rows = y1 - y0 + 6;    // pulled rows y0 - 3 .. y1 + 2
   constexpr int D = kTwoStages - 1;  // rows in flight
 #pragma unroll
   for (int k = 0; k < D; ++k) fetch(st[k]);  // n_rows >= 7
@@ -207,7 +252,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
 #pragma unroll
   for (int k = 0; k < 3; ++k) d0[k] = dn[k] = dnn[k] = zero;
 
-  unsigned out = (unsigned(y0) * unsigned(nx) + unsigned(xo)) * 4u;
+  unsigned out = (unsigned(y0) * pitch + unsigned(xo)) * 4u;
   int sg = 0, sf = D % kTwoStages;  // stages of row r and of row r + D
   bool go = true;
 #pragma unroll 2
@@ -228,20 +273,25 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
 #pragma unroll
       for (int a = 0; a < kQ; ++a) Q0[a] = F2(slot.d[a][lane]);
       collide<SCHEME, kNormal>(Q0, qrhoA, Gx, Gy, z2.c, A.P);
-      if (store_a && k >= 7) {
+      if (store_a && k >= 7 && (LAYOUT != kRing || k - 7 < y1 - y0)) {
+        // (kPadOdd: columns 0, 1 and 2 are copied to nx .. nx + 2; column nx is
+        // also the second cell of the lane that holds the last column)
+        const bool copies = LAYOUT == kPadOdd && xo < 4;
+        const int goff = xo == 0 ? nx + 1 : nx;
 #pragma unroll
         for (int a = 0; a < kQ; ++a) {
           float* const at =
               reinterpret_cast<float*>(reinterpret_cast<char*>(A.dst + a * A.plane) + out);
-          if constexpr (kOdd) {
+          if constexpr (LAYOUT == kFlatOdd) {
             at[0] = Q0[a].x();
             if (store_b) at[1] = Q0[a].y();
           } else {
             *reinterpret_cast<float2*>(at) = Q0[a].v;
+            if (copies) at[goff] = xo == 0 ? Q0[a].y() : Q0[a].x();
           }
         }
       }
-      if (k >= 7) out += unsigned(nx) * 4u;
+      if (k >= 7) out += pitch * 4u;
       m2 = z2;
       z2 = p2;
     }
@@ -299,22 +349,22 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
   return go;
 }
 
-// The band again with the full divisions and domain checks (rare).
-template <int SCHEME, bool kOdd>
+// The item again with the full divisions and domain checks (rare).
+template <int SCHEME, int LAYOUT>
 __device__ __noinline__ void strip_run_two_general(const StripArgs<StoreF32>& A, int strip,
                                                    int band, int lane, TwoRow* st) {
-  strip_run_two<SCHEME, kOdd, false>(A, strip, band, lane, st);
+  strip_run_two<SCHEME, LAYOUT, false>(A, strip, band, lane, st);
 }
 
-template <int SCHEME, bool kOdd>
+template <int SCHEME, int LAYOUT>
 __global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
 two_step_kernel(const __grid_constant__ StripArgs<StoreF32> A) {
   __shared__ TwoRow rows[kTwoStages + 2];
   const int lane = threadIdx.x;
   const int strip = blockIdx.x % A.n_strips;  // strips of kTwoCols columns
   const int band = blockIdx.x / A.n_strips;
-  if (!strip_run_two<SCHEME, kOdd, true>(A, strip, band, lane, rows))
-    strip_run_two_general<SCHEME, kOdd>(A, strip, band, lane, rows);
+  if (!strip_run_two<SCHEME, LAYOUT, true>(A, strip, band, lane, rows))
+    strip_run_two_general<SCHEME, LAYOUT>(A, strip, band, lane, rows);
 }
 
 }  // namespace lbm

@@ -84,3 +84,46 @@ def test_divergence_is_reported_in_either_step_of_a_launch():
                 # the context stays usable
                 lat.set_populations(good)
                 assert lat.step(4, lbm.SC, 0.8, raise_on_error=False) == lbm.LBM_OK
+
+
+# every row layout of the batch's two-step windows: whole rows in a half-warp
+# (even nx <= 32) and in a warp (<= 64), strips of even and of padded odd
+# widths, nx = 1; heights below and around a band
+BATCH = [dict(nx=nx, ny=ny, T_over_Tc=T, tau=tau, sigma=0.1, scheme=scheme)
+         for k, (nx, ny) in enumerate([(2, 9), (30, 41), (32, 128), (32, 5), (34, 37), (62, 20),
+                                       (64, 33), (66, 19), (56, 7), (112, 40), (114, 3), (1, 21),
+                                       (3, 33), (57, 30), (63, 1), (65, 18), (113, 25)])
+         for scheme, tau in [(SCHEMES[k % 6], 0.8 + 0.02 * k)]]
+
+
+@pytest.mark.parametrize("window,rows", [(20, 0), (20, 4), (10, 7), (14, 300)])
+def test_batch_windows(window, rows):
+    b = lbm.Batch(BATCH, window=window, tol=0.0, max_steps=10 ** 6, rows_per_item=rows,
+                  conv=lbm.CONV_NONE)
+    start = [field(d["nx"], d["ny"], k)[0] for k, d in enumerate(BATCH)]
+    for k, r in enumerate(start):
+        b.init_density(k, r)
+    assert b.run(2) == len(BATCH)
+    for k, d in enumerate(BATCH):
+        with lbm.Lattice(d["nx"], d["ny"], T) as lat:
+            lat.set_variant(lbm.VARIANT_REGISTER)
+            lat.init_density(start[k])
+            lat.step(2 * window, d["scheme"], d["tau"], d["sigma"])
+            for got, want in zip(b.moments(k), lat.observe()):
+                assert np.array_equal(got, want), d
+
+
+def test_batch_instance_that_diverges_leaves_the_others_alone():
+    inst = [dict(d) for d in BATCH[:4]]
+    inst[1].update(T_over_Tc=0.45, tau=0.6, scheme=lbm.SC)
+    b = lbm.Batch(inst, window=400, conv=lbm.CONV_NONE, max_steps=10 ** 6)
+    alone = lbm.Batch(inst[2:3], window=400, conv=lbm.CONV_NONE, max_steps=10 ** 6)
+    for k, d in enumerate(inst):
+        g, l, _ = lbm.maxwell(lbm.temperature(d["T_over_Tc"]))
+        rho = inputs.slab_step(d["nx"], d["ny"], g, l)
+        b.init_density(k, rho)
+        if k == 2:
+            alone.init_density(0, rho)
+    assert b.run(1) == 3 and alone.run(1) == 1
+    assert b.result(1)["status"] == lbm.RUN_DIVERGED
+    assert np.array_equal(b.density(2), alone.density(0))
