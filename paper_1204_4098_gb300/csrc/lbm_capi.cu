@@ -384,7 +384,8 @@ lbm_status launch_rows(lbm_ctx* c, int scheme, StripLaunch L, int r0, int r1, in
 // them with shorter gaps (~4 us per step there, a few per cent faster up to
 // 2048^2).  From 4096^2 on the step's own time hides the gap.
 constexpr int kGraphSteps = 16;
-constexpr int kPairsVariant = -1;  // step-graph key of the two-step launches
+static_assert(kGraphSteps % 4 == 0 && kGraphSteps / kTileSteps % 2 == 0,
+              "a graph is an even number of launches of each kind");
 constexpr size_t kGraphMaxCells = size_t(2048) * 2048;
 
 // One step kernel from buffer c->cur on `stream`, flipping c->cur.
@@ -405,34 +406,44 @@ cudaError_t launch_step(lbm_ctx* c, int scheme, StripLaunch& L, int grid, cudaSt
   return e;
 }
 
-// A step graph or a run of plain launches: n steps, two per launch where
-// `two` holds the two-step launch (a last odd step alone).
+// The launches of a run of steps: `one` step each, and where the lattice takes
+// them `many`: up to kTileSteps on tiles, or two.
+enum { kSingleSteps = 0, kTwoSteps = 1, kTileRuns = 2 };
 struct StepPlan {
-  StripLaunch one;  // one step per launch
+  StripLaunch one;
   int one_grid = 0;
-  bool pairs = false;  // two_step_applies
-  StripLaunch two;     // two steps per launch
-  int two_grid = 0;
+  int kind = kSingleSteps;
+  StripLaunch many;
+  int many_grid = 0, many_threads = 0;
 };
+
+// Steps of the next launch when n are left.
+int next_launch(const StepPlan& plan, int n) {
+  if (plan.kind == kTileRuns) return std::min(n, kTileSteps);
+  return plan.kind == kTwoSteps && n >= 2 ? 2 : 1;
+}
 
 // Queue up to n steps on `stream`; *done counts the steps, *launches the
 // kernels.
 cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t stream,
                      int* launches) {
   for (int k = 0; k < n;) {
-    if (plan.pairs && n - k >= 2) {
-      const int s = c->cur, d = 1 - c->cur;
-      plan.two.src = c->f[s];
-      plan.two.dst = c->f[d];
-      const cudaError_t e = two_step_launch(scheme, plan.two, plan.two_grid, stream);
-      if (e != cudaSuccess) return e;
-      c->cur = d;
-      k += 2;
+    const int steps = next_launch(plan, n - k);
+    cudaError_t e;
+    if (steps == 1) {
+      e = launch_step(c, scheme, plan.one, plan.one_grid, stream);
     } else {
-      const cudaError_t e = launch_step(c, scheme, plan.one, plan.one_grid, stream);
-      if (e != cudaSuccess) return e;
-      k += 1;
+      const int s = c->cur, d = 1 - c->cur;
+      plan.many.src = c->f[s];
+      plan.many.dst = c->f[d];
+      e = plan.kind == kTileRuns
+              ? tile_steps_launch(scheme, plan.many, steps, plan.many_grid, plan.many_threads,
+                                  stream)
+              : two_step_launch(scheme, plan.many, plan.many_grid, stream);
+      if (e == cudaSuccess) c->cur = d;
     }
+    if (e != cudaSuccess) return e;
+    k += steps;
     ++*launches;
   }
   return cudaSuccess;
@@ -454,13 +465,14 @@ bool same_launch(const StripLaunch& x, const StripLaunch& y) {
 // The cached graph of kGraphSteps steps from the current buffer, captured
 // again when any kernel argument, the scheme, the kernel variant or the grid
 // changed; nullptr when capture is unavailable (the caller then launches
-// step by step).  With pairs the steps are kGraphSteps / 2 two-step launches;
-// that count is even too, so a replay leaves the state in the same buffer.
+// step by step).  With two or kTileSteps steps per launch the number of
+// launches is even too, so a replay leaves the state in the same buffer.
 cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan) {
   lbm_ctx::StepGraph& g = c->graph[c->cur];
-  const int variant = plan.pairs ? kPairsVariant : pick_variant(c, kStepMode);
-  const int grid = plan.pairs ? plan.two_grid : plan.one_grid;
-  StripLaunch first = plan.pairs ? plan.two : plan.one;  // the key
+  const bool single = plan.kind == kSingleSteps;
+  const int variant = single ? pick_variant(c, kStepMode) : -plan.kind;
+  const int grid = single ? plan.one_grid : plan.many_grid;
+  StripLaunch first = single ? plan.one : plan.many;  // the key
   first.src = c->f[c->cur];
   first.dst = c->f[1 - c->cur];
   first.rho_src = c->rho[c->cur];
@@ -517,16 +529,26 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
   plan.one = step_launch(c, tau, sigma);
   lbm_status st = geometry(c, scheme, kStepMode, plan.one, plan.one_grid);
   if (st != LBM_OK) return st;
-  plan.pairs = !c->band && n >= 2 &&
-               two_step_applies(c->variant, c->p.precision, c->p.nx, c->p.ny,
-                                c->band_rows_override, c->p.b);
-  if (plan.pairs) {
-    const StripGeometry g = two_step_geometry(c->p.nx, c->p.ny, c->sm_count);
-    plan.two = plan.one;
-    plan.two.n_strips = g.n_strips;
-    plan.two.band_rows = g.band_rows;
-    plan.two.n_bands = g.n_bands;
-    plan.two_grid = g.grid;
+  if (!c->band && n >= 2) {
+    const TileGeometry t = tile_geometry(c->variant, c->p.precision, c->p.nx, c->p.ny,
+                                         c->band_rows_override, c->p.b, c->sm_count);
+    if (t.rows > 0) {
+      plan.kind = kTileRuns;
+      plan.many = plan.one;
+      plan.many.n_strips = t.n_cols;
+      plan.many.band_rows = t.rows;
+      plan.many_grid = t.grid;
+      plan.many_threads = t.threads;
+    } else if (two_step_applies(c->variant, c->p.precision, c->p.nx, c->p.ny,
+                                c->band_rows_override, c->p.b)) {
+      const StripGeometry g = two_step_geometry(c->p.nx, c->p.ny, c->sm_count);
+      plan.kind = kTwoSteps;
+      plan.many = plan.one;
+      plan.many.n_strips = g.n_strips;
+      plan.many.band_rows = g.band_rows;
+      plan.many.n_bands = g.n_bands;
+      plan.many_grid = g.grid;
+    }
   }
   int k = 0, launches = 0;
   // (not while the caller captures the context stream into a graph of its
@@ -543,7 +565,7 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
     if (g)
       for (; k + kGraphSteps <= n; k += kGraphSteps) {
         LBM_CUDA(c, cudaGraphLaunch(g, c->stream));  // the state returns to c->cur
-        launches += plan.pairs ? kGraphSteps / 2 : kGraphSteps;
+        launches += kGraphSteps / next_launch(plan, kGraphSteps);
       }
   }
   const cudaError_t e = run_plan(c, scheme, plan, n - k, c->stream, &launches);

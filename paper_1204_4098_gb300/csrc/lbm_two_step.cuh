@@ -39,12 +39,14 @@
 // registers, spilling) 119-122; rows of step 1 kept in registers 141 (spills).
 #pragma once
 
+#include "lbm_geometry.h"
 #include "lbm_kernels.cuh"
 
 namespace lbm {
 
-constexpr int kTwoHalo = 4;                  // columns loaded on each side of a strip
-constexpr int kTwoCols = 64 - 2 * kTwoHalo;  // columns a strip owns
+constexpr int kTwoHalo = 4;              // columns loaded on each side of a strip
+constexpr int kTwoCols = kTwoStepCols;   // columns a strip owns
+static_assert(kTwoCols + 2 * kTwoHalo == 64, "a warp loads two columns per lane");
 constexpr int kTwoStages = 3;                // rows in shared memory: one read, two in flight
 constexpr int kTwoThreads = 32;              // one warp per CTA
 constexpr int kTwoMinBlocks = 12;            // CTAs per SM (168 registers at most)

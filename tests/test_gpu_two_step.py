@@ -1,5 +1,6 @@
-"""The two-step launches of the automatic kernel choice against the one-step,
-one-column kernel (VARIANT_REGISTER): the same populations, bit for bit."""
+"""The launches of several steps that the automatic kernel choice makes (two
+steps on strips, up to four on tiles) against the one-step, one-column kernel
+(VARIANT_REGISTER): the same populations, bit for bit."""
 import numpy as np
 import pytest
 
@@ -46,28 +47,39 @@ def test_sizes(nx, ny, steps):
     assert np.array_equal(auto, ref)
 
 
+# tiles: one cell to the largest lattice they cover in a wave, widths around
+# the 16 columns of a tile, odd and even rows per tile, a ragged last tile
+@pytest.mark.parametrize("nx,ny", [
+    (1, 1), (2, 9), (1, 152), (15, 33), (16, 16), (17, 5), (32, 32), (40, 36), (33, 47), (64, 64),
+    (100, 3), (3, 100), (2432, 1), (2417, 32), (120, 128), (270, 250), (48, 1600), (257, 101)])
+@pytest.mark.parametrize("steps", [2, 3, 4, 9])
+def test_tiles(nx, ny, steps):
+    auto, ref = check(nx, ny, field(nx, ny, nx + ny), steps, lbm.IMPROVED)
+    assert np.array_equal(auto, ref)
+
+
 @pytest.mark.parametrize("scheme", SCHEMES)
-@pytest.mark.parametrize("nx,ny", [(200, 190), (333, 150)])
+@pytest.mark.parametrize("nx,ny", [(200, 190), (97, 60), (600, 300), (601, 301)])
 def test_schemes_and_step_graphs(scheme, nx, ny):
-    # 35 steps: two replays of a graph of 16, one two-step launch, one step
+    # 35 steps: two replays of a graph of 16 and what is left
     auto, ref = check(nx, ny, field(nx, ny, 5), 35, scheme)
     assert np.array_equal(auto, ref)
 
 
 @pytest.mark.parametrize("rows", [slice(None), slice(100, 140)])
 @pytest.mark.parametrize("scheme", [lbm.IMPROVED, lbm.NOFORCE])
-def test_densities_that_take_the_full_divisions(rows, scheme):
+@pytest.mark.parametrize("nx,ny", [(190, 240), (590, 240)])
+def test_densities_that_take_the_full_divisions(rows, scheme, nx, ny):
     # 1e-32 is inside the domain of psi but below the range in which the
     # reciprocals are taken without subnormal handling
-    nx, ny = 190, 240
     rho = np.full((ny, nx), 0.1)
     rho[rows] = 1e-32 * np.random.default_rng(1).uniform(1.0, 2.0, rho[rows].shape)
     auto, ref = check(nx, ny, (rho,), 2, scheme)
     assert np.array_equal(auto, ref, equal_nan=True)
 
 
-def test_divergence_is_reported_in_either_step_of_a_launch():
-    nx = ny = 192
+@pytest.mark.parametrize("nx,ny", [(192, 192), (600, 400)])
+def test_divergence_is_reported_in_any_step_of_a_launch(nx, ny):
     rho, ux, uy = field(nx, ny, 3)
     with lbm.Lattice(nx, ny, T) as lat:
         lat.init_density(rho, ux, uy)

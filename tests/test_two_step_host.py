@@ -16,6 +16,10 @@ void geometry(int nx, int ny, int* out) {
   const lbm::StripGeometry g = lbm::two_step_geometry(nx, ny, 152);
   out[0] = g.n_strips; out[1] = g.band_rows; out[2] = g.n_bands; out[3] = g.grid;
 }
+void tiles(int nx, int ny, int* out) {
+  const lbm::TileGeometry g = lbm::tile_geometry(0, 0, nx, ny, 0, 4.0, 152);
+  out[0] = g.n_cols; out[1] = g.rows; out[2] = g.grid; out[3] = g.threads;
+}
 int applies(int variant, int precision, int nx, int ny, int rows, double b) {
   return lbm::two_step_applies(variant, precision, nx, ny, rows, b);
 }
@@ -63,6 +67,21 @@ def test_bands_cover_the_rows_in_one_wave(H):
         assert n_strips == (nx + 55) // 56 and grid == n_strips * bands
         assert bands * rows >= ny > (bands - 1) * rows
         assert grid <= max(152 * 12, n_strips)
+
+
+def test_tiles_cover_the_lattice_in_one_wave(H):
+    rng = np.random.default_rng(1)
+    for nx, ny in [(1, 1), (2432, 1), (2433, 1), (1, 4864), (1, 4865)] + \
+            [tuple(int(2 ** v) for v in rng.uniform(0, 12, 2)) for _ in range(300)]:
+        out = (ctypes.c_int * 4)()
+        H.tiles(nx, ny, out)
+        cols, rows, grid, threads = out
+        if rows == 0:  # too large for one wave of tiles of at most 32 rows
+            assert (nx + 15) // 16 > 152 or -(-ny // (152 // ((nx + 15) // 16))) > 32
+            continue
+        assert cols == (nx + 15) // 16 and grid % cols == 0 and grid <= 152
+        assert grid // cols * rows >= ny > (grid // cols - 1) * rows
+        assert 2 * (threads // 32) >= rows + 16 and threads <= 768
 
 
 def test_only_automatic_fp32_lattices_take_two_steps(H):
