@@ -179,10 +179,10 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
 
 /* Advance n >= 0 time steps with the given scheme and relaxation time
  * tau > 1/2 (sigma is read by LBM_SCHEME_IMPROVED only).  Kernels are queued
- * on the context stream: one per step, or, for FP32 storage with the AUTO
- * variant and band height, one per up to four steps on small lattices (up to
- * about 270^2 cells) and one per two steps on larger ones (an odd last step
- * goes alone); on lattices of at most 2048^2 cells runs of 16 steps go through a
+ * on the context stream: one per step, or, with the AUTO variant and band
+ * height, one per up to four steps on small FP32 lattices (up to about 270^2
+ * cells) and one per two steps on larger ones and for 16-bit storage with even
+ * nx (an odd last step goes alone); on lattices of at most 2048^2 cells runs of 16 steps go through a
  * CUDA graph of these kernels, captured on first use for the current buffer
  * and launch arguments and kept until the context is destroyed (bit-identical
  * to single launches); while the caller captures the context stream into a

@@ -250,30 +250,31 @@ batch_balanced_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
 // and issue of its instructions, like two_step_kernel.
 template <int SCHEME, int LAYOUT>
 __device__ __noinline__ void batch_two_general(const StripArgs<StoreF32>& A, int strip, int lane,
-                                               TwoRow* rows) {
+                                               TwoSmem<StoreF32>& sm) {
   if constexpr (SCHEME == kNoForce)
-    if (strip_run_two<kNoForce, LAYOUT, true>(A, strip, 0, lane, rows)) return;
-  strip_run_two<SCHEME, LAYOUT, false>(A, strip, 0, lane, rows);
+    if (strip_run_two<StoreF32, kNoForce, LAYOUT, true>(A, strip, 0, lane, sm)) return;
+  strip_run_two<StoreF32, SCHEME, LAYOUT, false>(A, strip, 0, lane, sm);
 }
 
 template <int LAYOUT>
 __device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int scheme, int strip,
-                                               int lane, TwoRow* rows,
+                                               int lane, TwoSmem<StoreF32>& sm,
                                                StripArgs<StoreF32>& shared) {
-  if (scheme != kNoForce && strip_run_two<kBlend, LAYOUT, true>(A, strip, 0, lane, rows)) return;
+  if (scheme != kNoForce && strip_run_two<StoreF32, kBlend, LAYOUT, true>(A, strip, 0, lane, sm))
+    return;
   if (lane == 0) shared = A;
   __syncwarp();
   if (scheme == kNoForce)
-    batch_two_general<kNoForce, LAYOUT>(shared, strip, lane, rows);
+    batch_two_general<kNoForce, LAYOUT>(shared, strip, lane, sm);
   else
-    batch_two_general<kAnyForced, LAYOUT>(shared, strip, lane, rows);
+    batch_two_general<kAnyForced, LAYOUT>(shared, strip, lane, sm);
 }
 
 __global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
 batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict__ items,
                       const int* __restrict__ n_items, const float* src, float* dst,
                       unsigned* inst_status) {
-  __shared__ TwoRow rows[kTwoStages + 2];
+  __shared__ TwoSmem<StoreF32> sm;
   __shared__ StripArgs<StoreF32> shared;
   const int lane = threadIdx.x;
   if (int(blockIdx.x) >= *n_items) return;
@@ -298,14 +299,14 @@ batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
   const int strip = it.y;
   if (A.nx <= 64 && A.nx % 2 == 0) {
     if (A.nx <= 32) A.band_rows = (A.band_rows + 1) / 2;
-    batch_two_item<kRing>(A, A.P.scheme, strip, lane, rows, shared);
+    batch_two_item<kRing>(A, A.P.scheme, strip, lane, sm, shared);
   } else if (A.nx % 2 == 0) {
-    batch_two_item<kFlatEven>(A, A.P.scheme, strip, lane, rows, shared);
+    batch_two_item<kFlatEven>(A, A.P.scheme, strip, lane, sm, shared);
   } else {
     if (A.pitch == A.nx)  // nx = 1
-      batch_two_item<kFlatOdd>(A, A.P.scheme, strip, lane, rows, shared);
+      batch_two_item<kFlatOdd>(A, A.P.scheme, strip, lane, sm, shared);
     else
-      batch_two_item<kPadOdd>(A, A.P.scheme, strip, lane, rows, shared);
+      batch_two_item<kPadOdd>(A, A.P.scheme, strip, lane, sm, shared);
   }
 }
 

@@ -145,6 +145,16 @@ cudaError_t strip_tma_occupancy(int precision, int scheme, int* b) {
   if (precision != kFP32) return cudaErrorNotSupported;
   return strip_tma_occupancy_f32(scheme, b);
 }
+cudaError_t two_step_launch_f32(int, const StripLaunch&, int, cudaStream_t);
+cudaError_t two_step_launch_bf16(int, const StripLaunch&, int, cudaStream_t);
+cudaError_t two_step_launch_f16(int, const StripLaunch&, int, cudaStream_t);
+cudaError_t two_step_launch(int precision, int scheme, const StripLaunch& L, int grid,
+                            cudaStream_t s) {
+  if (precision == kFP32) return two_step_launch_f32(scheme, L, grid, s);
+  if (precision == kBF16Dev) return two_step_launch_bf16(scheme, L, grid, s);
+  if (precision == kFP16Dev) return two_step_launch_f16(scheme, L, grid, s);
+  return cudaErrorNotSupported;
+}
 cudaError_t set_state_launch(int precision, void* dst, float* rd, int nx, int ny, int pitch,
                              size_t plane, const double* rho, const double* ux, const double* uy,
                              const double* f_in, const EosCheck& chk, cudaStream_t s) {
@@ -436,10 +446,12 @@ cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t
       const int s = c->cur, d = 1 - c->cur;
       plan.many.src = c->f[s];
       plan.many.dst = c->f[d];
+      plan.many.rho_src = c->rho[s];
+      plan.many.rho_dst = c->rho[d];
       e = plan.kind == kTileRuns
               ? tile_steps_launch(scheme, plan.many, steps, plan.many_grid, plan.many_threads,
                                   stream)
-              : two_step_launch(scheme, plan.many, plan.many_grid, stream);
+              : two_step_launch(c->p.precision, scheme, plan.many, plan.many_grid, stream);
       if (e == cudaSuccess) c->cur = d;
     }
     if (e != cudaSuccess) return e;

@@ -88,18 +88,21 @@ inline StripGeometry strip_geometry(int nx, int ny, int variant, long long resid
 constexpr int kTwoStepCols = 56;   // columns of a strip
 constexpr int kTwoStepWarps = 12;  // resident warps per SM
 
-// Whether steps of a whole nx x ny FP32 lattice may go two per launch: AUTO
-// variant and band height (a requested kernel or height runs as requested),
-// a lattice large enough to gain, 32-bit byte offsets within a plane, and a
-// covolume for which every density inside the domain of psi (b rho / 4 < 1)
-// has a normal reciprocal.
+// Whether steps of a whole nx x ny lattice may go two per launch: FP32, or
+// 16-bit storage with even nx (its columns are copied in pairs), AUTO variant
+// and band height (a requested kernel or height runs as requested), a lattice
+// large enough to gain, 32-bit byte offsets within a plane, and a covolume for
+// which every density inside the domain of psi (b rho / 4 < 1) has a normal
+// reciprocal.
 constexpr long long kTwoStepMinCells = 176LL * 176;
 constexpr long long kTwoStepMaxCells = 1LL << 30;
 inline bool two_step_applies(int requested, int precision, int nx, int ny,
                              int band_rows_override, double b) {
   const long long cells = (long long)nx * ny;
-  return requested == LBM_VARIANT_AUTO && band_rows_override == 0 && precision == LBM_FP32 &&
-         cells >= kTwoStepMinCells && cells <= kTwoStepMaxCells && b > 1e-12 && b < 1e12;
+  const bool dev = precision == LBM_BF16DEV || precision == LBM_FP16DEV;
+  return requested == LBM_VARIANT_AUTO && band_rows_override == 0 &&
+         (precision == LBM_FP32 || (dev && nx % 2 == 0)) && cells >= kTwoStepMinCells &&
+         cells <= kTwoStepMaxCells && b > 1e-12 && b < 1e12;
 }
 
 // Strips of 56 columns and the band height that ends first.  A band of n rows

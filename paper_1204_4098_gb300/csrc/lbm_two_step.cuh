@@ -1,4 +1,4 @@
-// Two time steps in one pass over the lattice (FP32 storage).
+// Two time steps in one pass over the lattice (FP32 and 16-bit storage).
 //
 // The one-step kernels move 72 B per cell update and run at 0.93 of the copy
 // bandwidth on large lattices: they cannot get faster without moving less.
@@ -37,6 +37,12 @@
 // (147k MLUPS, DRAM at 0.77 of the measured copy bandwidth, FMA pipes 60 %
 // busy, 158 registers, 12 warps per SM).  13 to 16 warps per SM (128
 // registers, spilling) 119-122; rows of step 1 kept in registers 141 (spills).
+//
+// 16-bit storage gains from the instructions that two separate steps repeat
+// (the row copies, the halo's psi) and from the bare divisions: it was bound
+// by issue, not by memory (BF16, us per step, one-step -> two-step: 4096^2 186 ->
+// 133, 2048^2 51.1 -> 37.0, 1024^2 16.6 -> 12.4, 512^2 7.4 -> 5.8, 200^2 4.2 ->
+// 3.5; FP16 the same).
 #pragma once
 
 #include "lbm_geometry.h"
@@ -51,9 +57,18 @@ constexpr int kTwoStages = 3;                // rows in shared memory: one read,
 constexpr int kTwoThreads = 32;              // one warp per CTA
 constexpr int kTwoMinBlocks = 12;            // CTAs per SM (168 registers at most)
 
-// One row of a warp in shared memory: the 9 planes' pairs, lane-major.
+// Shared memory of a warp, lane-major.  A fetched row: the 9 planes' pairs, for
+// deviation storage also the density pair of the row after the pulled one (the
+// two before it stay in registers).  q: step 2's last two pulled rows.
+template <class S>
 struct TwoRow {
-  float2 d[kQ][32];
+  typename Vec2<typename S::T>::type d[kQ][32];
+  float2 rr[S::kDev ? 32 : 1];
+};
+template <class S>
+struct TwoSmem {
+  TwoRow<S> row[kTwoStages];
+  float2 q[2][kQ][32];
 };
 
 // psi of a row: the x neighbours only enter the force (Eq. 3) as their
@@ -100,12 +115,20 @@ __device__ __forceinline__ F2 psi_normal(F2 rho, const Phys<float>& P, bool& ok)
 //             columns each half-warp takes a band of its own.
 enum TwoLayout { kFlatEven, kFlatOdd, kPadOdd, kRing };
 
-// Two steps of one strip x band item.  st: the warp's kTwoStages + 2 rows of
-// shared memory.  kNormal: returns false as soon as a value fails
-// psi_normal's check; the item then has to be run again with kNormal = false.
-template <int SCHEME, int LAYOUT, bool kNormal>
-__device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int strip, int band,
-                                              int lane, TwoRow* st) {
+// Two steps of one strip x band item.  kNormal: returns false as soon as a
+// value fails psi_normal's check; the item then has to be run again with
+// kNormal = false.  Deviation storage (kFlatEven only) rounds the populations
+// between the two steps to what the one-step kernel would store and read
+// back, in registers.
+template <class S, int SCHEME, int LAYOUT, bool kNormal>
+__device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, int band, int lane,
+                                              TwoSmem<S>& sm) {
+  using T = typename S::T;
+  using V = typename Vec2<T>::type;
+  static_assert(std::is_same<typename S::C, float>::value && (!S::kDev || LAYOUT == kFlatEven),
+                "FP32 arithmetic; 16-bit columns are copied in aligned pairs");
+  constexpr unsigned kBytes = sizeof(T);
+  TwoRow<S>* const st = sm.row;
   constexpr bool kNeedPsi = SCHEME != kNoForce;
   constexpr bool kOneByOne = LAYOUT == kFlatOdd || LAYOUT == kPadOdd;  // row copies of 4 bytes
   const unsigned FULL = 0xffffffffu;
@@ -156,10 +179,10 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
   // 2^30 elements, so 32 bits hold them).
   auto wrap_row = [ny](int y) { return ((y % ny) + ny) % ny; };
   int nrow = wrap_row(y0 - 2);  // the row after the next pulled one
-  unsigned om = (unsigned(wrap_row(y0 - 4)) * pitch + unsigned(ca)) * 4u;
-  unsigned oz = (unsigned(wrap_row(y0 - 3)) * pitch + unsigned(ca)) * 4u;
-  auto fetch = [&](TwoRow& R) {
-    const unsigned op = (unsigned(nrow) * pitch + unsigned(ca)) * 4u;
+  unsigned om = (unsigned(wrap_row(y0 - 4)) * pitch + unsigned(ca)) * kBytes;
+  unsigned oz = (unsigned(wrap_row(y0 - 3)) * pitch + unsigned(ca)) * kBytes;
+  auto fetch = [&](TwoRow<S>& R) {
+    const unsigned op = (unsigned(nrow) * pitch + unsigned(ca)) * kBytes;
 #pragma unroll
     for (int a = 0; a < kQ; ++a) {
       const unsigned o = ey_of(a) == 0 ? oz : (ey_of(a) == 1 ? om : op);
@@ -168,9 +191,11 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
         cp_async<4>(&R.d[a][lane].x, p);
         cp_async<4>(&R.d[a][lane].y, p + 4 * (cb - ca));
       } else {
-        cp_async<8>(&R.d[a][lane], p);
+        cp_async<sizeof(V)>(&R.d[a][lane], p);
       }
     }
+    if constexpr (S::kDev)
+      cp_async<8>(&R.rr[lane], reinterpret_cast<const char*>(A.rho_src) + 2u * op);
     cp_async_commit();
     om = oz;
     oz = op;
@@ -189,9 +214,39 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
     if (ex == 1) return F2(left(v.y()), v.x());
     return F2(v.y(), right(v.x()));
   };
-  auto assemble = [&](const TwoRow& R, F2 (&P)[kQ]) {
+  // deviation storage: density pairs of the two rows before the next R.rr
+  F2 ring0 = F2(0.f), ring1 = F2(0.f);
+  if constexpr (S::kDev) {
+    const char* const r = reinterpret_cast<const char*>(A.rho_src);
+    ring0 = F2(__ldg(reinterpret_cast<const float2*>(r + 2u * om)));
+    ring1 = F2(__ldg(reinterpret_cast<const float2*>(r + 2u * oz)));
+  }
+  auto assemble = [&](const TwoRow<S>& R, F2 (&P)[kQ]) {
+    if constexpr (S::kDev) {
+      const F2 rr[3] = {ring0, ring1, F2(R.rr[lane])};  // source rows r - 1, r, r + 1
 #pragma unroll
-    for (int a = 0; a < kQ; ++a) P[a] = pull_x(a, F2(R.d[a][lane]));
+      for (int a = 0; a < kQ; ++a)
+        P[a] = pull_x(a, S::decode2(mul_rn(F2(w_of<float>(a)), rr[1 - ey_of(a)]), R.d[a][lane]));
+      ring0 = rr[1];
+      ring1 = rr[2];
+    } else {
+#pragma unroll
+      for (int a = 0; a < kQ; ++a) P[a] = pull_x(a, F2(R.d[a][lane]));
+    }
+  };
+  // deviation storage: the 16-bit deviations of post-collision populations f
+  // of density r, and the density that absorbs their rounding
+  auto encode = [&](const F2 (&f)[kQ], F2 r, V (&v)[kQ]) {
+    F2 res = r;
+    if constexpr (S::kDev) {
+#pragma unroll
+      for (int a = 0; a < kQ; ++a) {
+        const F2 d = fma_rn(F2(-w_of<float>(a)), r, f[a]);
+        v[a] = S::from_c2(d.x(), d.y());
+        res = S::sub_from(res, v[a]);
+      }
+    }
+    return res;
   };
   auto rho_of = [](const F2 (&P)[kQ]) {
     F2 r = P[0];
@@ -236,7 +291,6 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
   constexpr int D = kTwoStages - 1;  // rows in flight
 #pragma unroll
   for (int k = 0; k < D; ++k) fetch(st[k]);  // n_rows >= 7
-  TwoRow* const qrow = st + kTwoStages;  // step 2's last two pulled rows
 
   // In iteration k the pulled row r = y0 - 3 + k arrives.  Step 1 has its
   // pulled row r - 1 (P0, rho0) and the psi of rows r - 2 (m1) and r - 1 (z1).
@@ -254,14 +308,14 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
 #pragma unroll
   for (int k = 0; k < 3; ++k) d0[k] = dn[k] = dnn[k] = zero;
 
-  unsigned out = (unsigned(y0) * pitch + unsigned(xo)) * 4u;
+  unsigned out = (unsigned(y0) * pitch + unsigned(xo)) * kBytes;
   int sg = 0, sf = D % kTwoStages;  // stages of row r and of row r + D
   bool go = true;
 #pragma unroll 2
   for (int k = 0; k <= n_rows && go; ++k) {
     // step 2: psi of row r - 3, output row r - 4 (the first rows of the march
     // run on values that no later row uses)
-    TwoRow& slot = qrow[k & 1];
+    float2(&slot)[kQ][32] = sm.q[k & 1];
     {
       const bool use = valid2 && k >= 5;
       PsiRow p2 = none;
@@ -273,18 +327,23 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
         rho_check(qrhoB, use);
       }
 #pragma unroll
-      for (int a = 0; a < kQ; ++a) Q0[a] = F2(slot.d[a][lane]);
+      for (int a = 0; a < kQ; ++a) Q0[a] = F2(slot[a][lane]);
       collide<SCHEME, kNormal>(Q0, qrhoA, Gx, Gy, z2.c, A.P);
       if (store_a && k >= 7 && (LAYOUT != kRing || k - 7 < y1 - y0)) {
         // (kPadOdd: columns 0, 1 and 2 are copied to nx .. nx + 2; column nx is
         // also the second cell of the lane that holds the last column)
         const bool copies = LAYOUT == kPadOdd && xo < 4;
         const int goff = xo == 0 ? nx + 1 : nx;
+        V v[kQ];
+        const F2 res = encode(Q0, qrhoA, v);
+        if constexpr (S::kDev)
+          *reinterpret_cast<float2*>(reinterpret_cast<char*>(A.rho_dst) + 2u * out) = res.v;
 #pragma unroll
         for (int a = 0; a < kQ; ++a) {
-          float* const at =
-              reinterpret_cast<float*>(reinterpret_cast<char*>(A.dst + a * A.plane) + out);
-          if constexpr (LAYOUT == kFlatOdd) {
+          T* const at = reinterpret_cast<T*>(reinterpret_cast<char*>(A.dst + a * A.plane) + out);
+          if constexpr (S::kDev) {
+            *reinterpret_cast<V*>(at) = v[a];
+          } else if constexpr (LAYOUT == kFlatOdd) {
             at[0] = Q0[a].x();
             if (store_b) at[1] = Q0[a].y();
           } else {
@@ -293,7 +352,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
           }
         }
       }
-      if (k >= 7) out += pitch * 4u;
+      if (k >= 7) out += pitch * kBytes;
       m2 = z2;
       z2 = p2;
     }
@@ -315,6 +374,13 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
       rho_check(rho1, valid1 && k < n_rows);
     }
     collide<SCHEME, kNormal>(P0, rho0, Fx, Fy, z1.c, A.P);  // row r - 1
+    if constexpr (S::kDev) {
+      V v[kQ];
+      const F2 res = encode(P0, rho0, v);
+#pragma unroll
+      for (int a = 0; a < kQ; ++a)
+        P0[a] = S::decode2(mul_rn(F2(w_of<float>(a)), res), v[a]);
+    }
     // step 2's pulled row r - 2 is complete
     F2 Q1[kQ];
     Q1[0] = d0[0];
@@ -337,7 +403,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
     qrhoA = qrhoB;
     qrhoB = rho_of(Q1);
 #pragma unroll
-    for (int a = 0; a < kQ; ++a) slot.d[a][lane] = Q1[a].v;
+    for (int a = 0; a < kQ; ++a) slot[a][lane] = Q1[a].v;
     m1 = z1;
     z1 = p1;
     rho0 = rho1;
@@ -352,21 +418,21 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<StoreF32>& A, int 
 }
 
 // The item again with the full divisions and domain checks (rare).
-template <int SCHEME, int LAYOUT>
-__device__ __noinline__ void strip_run_two_general(const StripArgs<StoreF32>& A, int strip,
-                                                   int band, int lane, TwoRow* st) {
-  strip_run_two<SCHEME, LAYOUT, false>(A, strip, band, lane, st);
+template <class S, int SCHEME, int LAYOUT>
+__device__ __noinline__ void strip_run_two_general(const StripArgs<S>& A, int strip, int band,
+                                                   int lane, TwoSmem<S>& sm) {
+  strip_run_two<S, SCHEME, LAYOUT, false>(A, strip, band, lane, sm);
 }
 
-template <int SCHEME, int LAYOUT>
+template <class S, int SCHEME, int LAYOUT>
 __global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
-two_step_kernel(const __grid_constant__ StripArgs<StoreF32> A) {
-  __shared__ TwoRow rows[kTwoStages + 2];
+two_step_kernel(const __grid_constant__ StripArgs<S> A) {
+  __shared__ TwoSmem<S> sm;
   const int lane = threadIdx.x;
   const int strip = blockIdx.x % A.n_strips;  // strips of kTwoCols columns
   const int band = blockIdx.x / A.n_strips;
-  if (!strip_run_two<SCHEME, LAYOUT, true>(A, strip, band, lane, rows))
-    strip_run_two_general<SCHEME, LAYOUT>(A, strip, band, lane, rows);
+  if (!strip_run_two<S, SCHEME, LAYOUT, true>(A, strip, band, lane, sm))
+    strip_run_two_general<S, SCHEME, LAYOUT>(A, strip, band, lane, sm);
 }
 
 }  // namespace lbm

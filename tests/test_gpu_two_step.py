@@ -19,8 +19,8 @@ def field(nx, ny, seed):
     return rho, rng.uniform(-0.02, 0.02, (ny, nx)), rng.uniform(-0.02, 0.02, (ny, nx))
 
 
-def populations(nx, ny, state, steps, scheme, variant):
-    with lbm.Lattice(nx, ny, T) as lat:
+def populations(nx, ny, state, steps, scheme, variant, precision=lbm.FP32):
+    with lbm.Lattice(nx, ny, T, precision=precision) as lat:
         lat.set_variant(variant)
         lat.set_mrt_rates(0.8, 1.1, 1.3)
         lat.init_density(*state)
@@ -28,9 +28,9 @@ def populations(nx, ny, state, steps, scheme, variant):
         return st, lat.populations()
 
 
-def check(nx, ny, state, steps, scheme):
-    st_a, auto = populations(nx, ny, state, steps, scheme, lbm.VARIANT_AUTO)
-    st_r, ref = populations(nx, ny, state, steps, scheme, lbm.VARIANT_REGISTER)
+def check(nx, ny, state, steps, scheme, precision=lbm.FP32):
+    st_a, auto = populations(nx, ny, state, steps, scheme, lbm.VARIANT_AUTO, precision)
+    st_r, ref = populations(nx, ny, state, steps, scheme, lbm.VARIANT_REGISTER, precision)
     assert st_a == st_r
     return auto, ref
 
@@ -44,6 +44,17 @@ def check(nx, ny, state, steps, scheme):
 @pytest.mark.parametrize("steps", [2, 5])
 def test_sizes(nx, ny, steps):
     auto, ref = check(nx, ny, field(nx, ny, nx + ny), steps, lbm.IMPROVED)
+    assert np.array_equal(auto, ref)
+
+
+# 16-bit storage: the rounding between the two steps of a launch, every scheme
+@pytest.mark.parametrize("precision", [lbm.BF16DEV, lbm.FP16DEV])
+@pytest.mark.parametrize("nx,ny,scheme", [(200, 190, s) for s in SCHEMES] + [
+    (2, 15500, lbm.IMPROVED), (56, 600, lbm.IMPROVED), (58, 601, lbm.SC), (112, 300, lbm.EDM),
+    (640, 333, lbm.IMPROVED), (31000, 1, lbm.IMPROVED), (15500, 2, lbm.SC),
+    (641, 333, lbm.IMPROVED)])  # (odd nx: one step per launch)
+def test_16_bit_storage(precision, nx, ny, scheme):
+    auto, ref = check(nx, ny, field(nx, ny, nx + ny), 21, scheme, precision)
     assert np.array_equal(auto, ref)
 
 

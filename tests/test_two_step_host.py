@@ -84,7 +84,7 @@ def test_tiles_cover_the_lattice_in_one_wave(H):
         assert 2 * (threads // 32) >= rows + 16 and threads <= 768
 
 
-def test_only_automatic_fp32_lattices_take_two_steps(H):
+def test_which_lattices_take_two_steps(H):
     H.applies.argtypes = [ctypes.c_int] * 5 + [ctypes.c_double]
     assert H.applies(0, 0, 200, 200, 0, 4.0)
     assert not H.applies(0, 0, 100, 100, 0, 4.0)       # too small
@@ -93,8 +93,10 @@ def test_only_automatic_fp32_lattices_take_two_steps(H):
     assert not H.applies(0, 0, 200, 200, 0, 1e-13)     # subnormal reciprocals possible
     for variant in (1, 2, 3):
         assert not H.applies(variant, 0, 4096, 4096, 0, 4.0)
-    for precision in (1, 2, 3):
-        assert not H.applies(0, precision, 4096, 4096, 0, 4.0)
+    assert not H.applies(0, 1, 4096, 4096, 0, 4.0)     # FP64
+    for precision in (2, 3):  # 16-bit columns go in aligned pairs
+        assert H.applies(0, precision, 4096, 4096, 0, 4.0)
+        assert not H.applies(0, precision, 4095, 4096, 0, 4.0)
 
 
 @pytest.mark.parametrize("rows", [4, 7, 33, 500])
