@@ -331,8 +331,11 @@ lbm_status geometry(lbm_ctx* c, int scheme, int mode, StripLaunch& L, int& grid,
   if (bps < 1) bps = 1;
   const int warps_per_cta = kStripCtaThreads / 32;
   const long long resident = (long long)c->sm_count * bps * warps_per_cta;
-  const StripGeometry g = strip_geometry(c->p.nx, rows < 0 ? c->p.ny : rows, variant, resident,
-                                         warps_per_cta, c->band_rows_override);
+  const int ny = rows < 0 ? c->p.ny : rows;
+  const StripGeometry g =
+      c->p.precision == LBM_FP64 && variant == LBM_VARIANT_REGISTER && c->band_rows_override == 0
+          ? fp64_geometry(c->p.nx, ny, c->sm_count, warps_per_cta)
+          : strip_geometry(c->p.nx, ny, variant, resident, warps_per_cta, c->band_rows_override);
   L.n_strips = g.n_strips;
   L.band_rows = g.band_rows;
   L.n_bands = g.n_bands;

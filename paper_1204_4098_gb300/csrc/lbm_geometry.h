@@ -82,6 +82,32 @@ inline StripGeometry strip_geometry(int nx, int ny, int variant, long long resid
   return g;
 }
 
+// Bands of the FP64 one-column kernel.  The FP64 pipe bounds it whatever the
+// number of warps (one warp per scheduler already saturates it), so the launch
+// takes as long as the SM with most work: with w = 1, 2 or 3 warps per
+// scheduler, w (80 rows + 41 (rows + 2)) FP64 instructions, the second term
+// being the density and psi of a band's rows and of the two around it.  Few
+// tall bands win (512^2: 14 rows, 1 warp) until they no longer divide the
+// lattice evenly (8192^2: 7 bands of 1171 rows, 3 warps).
+inline StripGeometry fp64_geometry(int nx, int ny, int sm_count, int warps_per_cta) {
+  StripGeometry g;
+  g.n_strips = (nx + 31) / 32;
+  double best = 0.0;
+  for (int w = 1; w <= 3; ++w) {
+    const long long bands = std::min<long long>(
+        ny, std::max<long long>(1, (long long)sm_count * warps_per_cta * w / g.n_strips));
+    const int rows = int((ny + bands - 1) / bands);
+    const double t = w * (80.0 * rows + 41.0 * (rows + 2));
+    if (w == 1 || t < best) {
+      best = t;
+      g.band_rows = rows;
+    }
+  }
+  g.n_bands = (ny + g.band_rows - 1) / g.band_rows;
+  g.grid = int(((long long)g.n_strips * g.n_bands + warps_per_cta - 1) / warps_per_cta);
+  return g;
+}
+
 // ---------------------------------------------------------------------------
 // two steps per launch (lbm_two_step.cuh)
 // ---------------------------------------------------------------------------

@@ -33,6 +33,7 @@
 namespace lbm {
 
 constexpr int kStripWarpsPerCta = 4;
+constexpr int kFp64Ctas = 3;  // resident CTAs per SM of the FP64 one-column kernel
 constexpr int kStripThreads = kStripWarpsPerCta * 32;
 // Resident CTAs per SM the register allocation must allow (occupancy target).
 #ifndef LBM_STRIP_MIN_BLOCKS
@@ -112,6 +113,11 @@ __device__ __forceinline__ void strip_run(const StripArgs<S>& A, int strip, int 
   const int hsx = ((hcol - hex) % nx + nx) % nx;
   const bool hlane = ha < kQ;
   const int hbase = lane & 16;
+  // FP64: psi of the halo columns is evaluated for 16 rows at a time, a row
+  // and side per lane, instead of once per row by every lane: the FP64 pipe
+  // bounds these kernels (2 lanes a clock and SM), and the halo's density and
+  // psi are a fifth of a row's FP64 instructions.
+  constexpr bool kHaloRows = std::is_same<C, double>::value && kNeedPsi;
 
   bool bad = false;
 
@@ -129,7 +135,7 @@ __device__ __forceinline__ void strip_run(const StripArgs<S>& A, int strip, int 
     P[6] = pull_one<S, kCoherent>(A, 6, rm + cp);
     P[7] = pull_one<S, kCoherent>(A, 7, rp + cp);
     P[8] = pull_one<S, kCoherent>(A, 8, rp + cm);
-    if constexpr (kNeedPsi) {
+    if constexpr (kNeedPsi && !kHaloRows) {
       int hy = y - hey;  // |hey| <= 1 and 0 <= y < ny: one conditional wrap
       hy = hy < 0 ? hy + ny : (hy >= ny ? hy - ny : hy);
       h = hlane ? pull_one<S, kCoherent>(A, ha, hy * pitch + hsx) : C(0);
@@ -150,15 +156,42 @@ __device__ __forceinline__ void strip_run(const StripArgs<S>& A, int strip, int 
     return psi_of_rho(r, A.P, bad);
   };
 
+  // kHaloRows: psi of the halo column of rows y0 - 1 + k .. + 15 (lane & 15),
+  // rows up to y1 only (further ones may be ghost rows of no meaning)
+  C hrows = C(0);
+  auto halo_rows = [&](int k) {
+    const int y = y0 - 1 + k + (lane & 15);
+    if (y > y1) return;
+    const int cw = hcol == 0 ? nx - 1 : hcol - 1, ce = hcol == nx - 1 ? 0 : hcol + 1;
+    const int yz = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+    const int ym = yz == 0 ? ny - 1 : yz - 1, yp = yz == ny - 1 ? 0 : yz + 1;
+    C r = C(0);
+#pragma unroll
+    for (int a = 0; a < kQ; ++a) {
+      const int row = ey_of(a) == 0 ? yz : (ey_of(a) == 1 ? ym : yp);
+      const int col = ex_of(a) == 0 ? hcol : (ex_of(a) == 1 ? cw : ce);
+      const C v = pull_one<S, kCoherent>(A, a, row * pitch + col);
+      r = a == 0 ? v : add_rn(r, v);
+    }
+    hrows = psi_of_rho(r, A.P, bad);
+  };
+
   // psi ring: rows y-1 (m), y (z), y+1 (p); W / C / E = columns x-1, x, x+1
   C Wm = 0, Cm = 0, Em = 0, Wz = 0, Cz = 0, Ez = 0;
   C rho0;
 
-  auto psi_row = [&](const C (&P)[kQ], C h, C& Wv, C& Cv, C& Ev, C& rho_out) {
+  // (k: the row is y0 - 1 + k)
+  auto psi_row = [&](const C (&P)[kQ], C h, int k, C& Wv, C& Cv, C& Ev, C& rho_out) {
     rho_out = rho_of(P);
     if constexpr (kNeedPsi) {
       Cv = psi_of_rho(rho_out, A.P, bad);
-      const C hp = halo_psi(h);
+      C hp;
+      if constexpr (kHaloRows) {
+        if ((k & 15) == 0) halo_rows(k);  // warp-uniform
+        hp = __shfl_sync(FULL, hrows, hbase + (k & 15));
+      } else {
+        hp = halo_psi(h);
+      }
       Wv = __shfl_up_sync(FULL, Cv, 1);
       Ev = __shfl_down_sync(FULL, Cv, 1);
       if (lane == 0) Wv = hp;
@@ -174,7 +207,7 @@ __device__ __forceinline__ void strip_run(const StripArgs<S>& A, int strip, int 
                  C& hload) {
     if (y + 2 <= y1) load_row(y + 2 >= ny ? y + 2 - ny : y + 2, Pload, hload);
     C Wp = 0, Cp = 0, Ep = 0, rho1;
-    psi_row(Pnext, hnext, Wp, Cp, Ep, rho1);
+    psi_row(Pnext, hnext, y - y0 + 2, Wp, Cp, Ep, rho1);
 
     C Fx = C(0), Fy = C(0);
     if constexpr (kNeedPsi) {
@@ -234,8 +267,8 @@ __device__ __forceinline__ void strip_run(const StripArgs<S>& A, int strip, int 
     load_row(y0 == 0 ? ny - 1 : y0 - 1, PC, hC);
     load_row(y0, PA, hA);
     load_row(y0 + 1 == ny ? 0 : y0 + 1, PB, hB);
-    psi_row(PC, hC, Wm, Cm, Em, rdummy);
-    psi_row(PA, hA, Wz, Cz, Ez, rho0);
+    psi_row(PC, hC, 0, Wm, Cm, Em, rdummy);
+    psi_row(PA, hA, 1, Wz, Cz, Ez, rho0);
   }
 #if LBM_STRIP_UNROLL3
   int y = y0;
@@ -261,8 +294,11 @@ __device__ __forceinline__ void strip_run(const StripArgs<S>& A, int strip, int 
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(A.status, kStatusDiverged);
 }
 
+// FP64 runs one to three CTAs per SM (fp64_geometry): no spills.
 template <class S, int SCHEME, int MODE>
-__global__ void __launch_bounds__(kStripThreads, LBM_STRIP_MIN_BLOCKS)
+__global__ void __launch_bounds__(kStripThreads, std::is_same<S, StoreF64>::value
+                                                     ? kFp64Ctas
+                                                     : LBM_STRIP_MIN_BLOCKS)
 strip_kernel(const StripArgs<S> A) {
   const int lane = threadIdx.x & 31;
   const int gwarp = (blockIdx.x * kStripThreads + threadIdx.x) >> 5;
