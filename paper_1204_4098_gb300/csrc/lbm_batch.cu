@@ -243,11 +243,12 @@ batch_balanced_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
 // Against the work list it halves the traffic and the launches, keeps 12
 // warps per SM in flight whatever the item lengths, and gives lattices of up
 // to 64 even columns whole rows (the work list's 64-column strips leave half
-// of a 32-column lattice's lanes idle).  Measured, us per step, best work-list
-// or balanced mode -> this: 96 slabs of 32 columns 31.3 -> 11.4 (95k MLUPS),
-// 600 of them 148 -> 44.2, 48 mixed slabs (4.7 M cells) 79 -> 48.1, 128 mixed
-// slabs 179 -> 104 (110k MLUPS), 2 slabs 14.2 -> 6.1.  Bound by the latency
-// and issue of its instructions, like two_step_kernel.
+// of a 32-column lattice's lanes idle).  The lattices are split into several
+// chains of launches that run side by side (two_step_graph).  Measured, us
+// per step, best work-list or balanced mode -> this: 96 slabs of 32 columns
+// 31.3 -> 9.2 (117k MLUPS), 600 of them 148 -> 38.4, 48 mixed slabs (4.7 M cells)
+// 79 -> 39.1 (121k MLUPS), 128 mixed slabs 179 -> 98, 6 slabs 17.6 -> 7.9.  Bound
+// by the latency and issue of its instructions, like two_step_kernel.
 template <int SCHEME, int LAYOUT>
 __device__ __noinline__ void batch_two_general(const StripArgs<StoreF32>& A, int strip, int lane,
                                                TwoSmem<StoreF32>& sm) {
@@ -270,21 +271,25 @@ __device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int
     batch_two_general<kAnyForced, LAYOUT>(shared, strip, lane, sm);
 }
 
+// (One kernel per layout: with the bodies of all layouts in one, registers
+// spill and mixed sweeps lose 6-12 %.)
+template <int LAYOUT>
 __global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
 batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict__ items,
-                      const int* __restrict__ n_items, const float* src, float* dst,
+                      const int2* __restrict__ chain, const float* src, float* dst,
                       unsigned* inst_status) {
   __shared__ TwoSmem<StoreF32> sm;
   __shared__ StripArgs<StoreF32> shared;
   const int lane = threadIdx.x;
-  if (int(blockIdx.x) >= *n_items) return;
-  const int4 it = items[blockIdx.x];  // instance, strip, first row, end row
+  const int2 range = *chain;  // first item, number of items
+  if (int(blockIdx.x) >= range.y) return;
+  const int4 it = items[range.x + blockIdx.x];  // instance, strip, first row, end row
   const int i = it.x;
   // An instance that has left the domain of psi has its verdict; its state is
   // of no further use and is not advanced.
   if (inst_status[i] & kStatusDiverged) return;
   const BatchInst& I = inst[i];
-  StripArgs<StoreF32> A;  // (field by field: a copy of the whole record spills)
+  StripArgs<StoreF32> A;
   A.src = src + I.off;
   A.dst = dst + I.off;
   A.status = inst_status + i;
@@ -296,17 +301,23 @@ batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
   A.y_begin = it.z;
   A.y_end = it.w;
   A.band_rows = it.w - it.z;
-  const int strip = it.y;
-  if (A.nx <= 64 && A.nx % 2 == 0) {
-    if (A.nx <= 32) A.band_rows = (A.band_rows + 1) / 2;
-    batch_two_item<kRing>(A, A.P.scheme, strip, lane, sm, shared);
-  } else if (A.nx % 2 == 0) {
-    batch_two_item<kFlatEven>(A, A.P.scheme, strip, lane, sm, shared);
-  } else {
-    if (A.pitch == A.nx)  // nx = 1
-      batch_two_item<kFlatOdd>(A, A.P.scheme, strip, lane, sm, shared);
-    else
-      batch_two_item<kPadOdd>(A, A.P.scheme, strip, lane, sm, shared);
+  if (LAYOUT == kRing && A.nx <= 32) A.band_rows = (A.band_rows + 1) / 2;  // a band per half-warp
+  batch_two_item<LAYOUT>(A, A.P.scheme, it.y, lane, sm, shared);
+}
+
+// The copies of columns 0 .. 2 behind the rows of odd lattices, which the
+// two-step kernel does not keep and the one-step kernels read: before the
+// last steps of a window that go one by one.  A CTA per active instance.
+__global__ void __launch_bounds__(kReduceCta)
+batch_copies_kernel(const BatchInst* __restrict__ inst, const int* __restrict__ active,
+                    const int* __restrict__ n_active, float* buf) {
+  if (int(blockIdx.x) >= *n_active) return;
+  const BatchInst I = inst[active[blockIdx.x]];
+  if (I.pitch == I.nx) return;
+  float* const f = buf + I.off;
+  for (int k = threadIdx.x; k < kQ * I.ny * 3; k += kReduceCta) {
+    float* const row = f + size_t(k / 3) * I.pitch;  // planes are whole rows
+    row[I.nx + k % 3] = row[k % 3 % I.nx];
   }
 }
 
@@ -600,6 +611,14 @@ __global__ void to_float_kernel(const double* in, float* out, size_t n) {
 
 using namespace lbm;
 
+// Chains of a two-step window: as many as wanted, and one more for each layout
+// that rounding leaves without.  (48 lattices of even width, us per step: 43.5
+// with one chain, 38.8 with 2, 36.0 with 3, 35.3 with 6, 35.5 with 12.)
+constexpr int kTwoChainsWanted = 6;
+constexpr int kTwoMaxChains = kTwoChainsWanted + kTwoBatchLayouts;
+constexpr int kTwoChunk = 50;       // launches per chain in a captured chunk (even)
+constexpr size_t kMaxGraphs = 64;   // captured graphs kept by a batch
+
 struct lbm_batch {
   lbm_batch_params p{};
   int count = 0;
@@ -629,11 +648,15 @@ struct lbm_batch {
   int4* h_bal_items = nullptr;
   int* h_bal_begin = nullptr;
   int bal_cap = 0;               // items per class table
-  int4* d_two_items = nullptr;   // two-step windows: items and their number
-  int* d_two_count = nullptr;
+  // two-step windows: the items of all chains, and per chain its first item
+  // and their number; streams and events of the chains after the first
+  int4* d_two_items = nullptr;
+  int2* d_two_chain = nullptr;
   int4* h_two_items = nullptr;
-  int* h_two_count = nullptr;
-  int two_cap = 0;
+  int2* h_two_chain = nullptr;
+  std::vector<std::pair<int, int>> two_chain;  // (layout, grid)
+  cudaStream_t two_side[kTwoMaxChains - 1] = {};
+  cudaEvent_t two_join[kTwoMaxChains - 1] = {};
   int* h_active = nullptr;
   int* h_prefix = nullptr;
   int* h_cta_begin = nullptr;
@@ -651,9 +674,9 @@ struct lbm_batch {
   unsigned* d_sync = nullptr;    // grid barrier: arrivals, generation, error
   cudaStream_t side = nullptr;   // second branch of the window graph
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  // window graphs by (mode, grid of the two-step kernel, grid of the two-column
-  // kernel, grid of the one-column kernel); a grid of 0 leaves a kernel out
-  std::map<std::tuple<int, int, int, int>, cudaGraphExec_t> graphs;
+  // graphs by mode and grids of the two-column and the one-column kernel (0
+  // leaves a kernel out), or by layout and grid of every two-step chain
+  std::map<std::vector<int>, cudaGraphExec_t> graphs;
   int class_items[2] = {0, 0};  // work-list items of the active instances per class
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   bool initialized = false;
@@ -720,6 +743,7 @@ std::vector<TwoLattice> two_lattices(const lbm_batch* b) {
   std::vector<TwoLattice> lat;
   lat.reserve(b->active.size());
   for (int i : b->active) lat.push_back(TwoLattice{i, b->desc[i].nx, b->desc[i].ny});
+  two_layouts(lat);
   return lat;
 }
 
@@ -764,15 +788,22 @@ lbm_status upload_tables(lbm_batch* b, int mode, int rows) {
   LBM_BCUDA(b, cudaMemcpyAsync(b->d_cta_list, b->h_cta_list, std::max(pos, 1) * sizeof(int),
                                cudaMemcpyHostToDevice, b->stream));
   if (mode == kBatchTwoStep) {
-    std::vector<TwoItem> items;
-    two_items(two_lattices(b), rows, items);
-    const int n = int(items.size());
-    *b->h_two_count = n;
     static_assert(sizeof(TwoItem) == sizeof(int4), "an item is one 16-byte load");
-    std::memcpy(b->h_two_items, items.data(), n * sizeof(TwoItem));
-    LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_items, b->h_two_items, n * sizeof(int4),
+    const std::vector<TwoChain> chains = two_chains(two_lattices(b), kTwoChainsWanted);
+    std::vector<TwoItem> items;
+    int total = 0, c = 0;
+    b->two_chain.clear();
+    for (const TwoChain& chain : chains) {
+      two_items(chain.lat, rows, items);
+      const int n = int(items.size());
+      std::memcpy(b->h_two_items + total, items.data(), n * sizeof(TwoItem));
+      b->h_two_chain[c++] = make_int2(total, n);
+      b->two_chain.push_back({chain.layout, two_item_grid(n)});
+      total += n;
+    }
+    LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_items, b->h_two_items, total * sizeof(int4),
                                  cudaMemcpyHostToDevice, b->stream));
-    LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_count, b->h_two_count, sizeof(int),
+    LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_chain, b->h_two_chain, c * sizeof(int2),
                                  cudaMemcpyHostToDevice, b->stream));
   }
   if (mode == LBM_BATCH_BALANCED)
@@ -803,27 +834,60 @@ int class_grid(const lbm_batch* b, int mode, int cls) {
   return worklist_grid(b->class_items[cls], kWorklistThreads / 32, b->wl_grid[cls]);
 }
 
+// Launch s of chain c of a two-step window.
+void two_step_chain(lbm_batch* b, int c, int s, cudaStream_t q) {
+  const int layout = b->two_chain[c].first, grid = b->two_chain[c].second;
+  const auto kernel = layout == kTwoBatchPairs  ? batch_two_step_kernel<kFlatEven>
+                      : layout == kTwoBatchRing ? batch_two_step_kernel<kRing>
+                                                : batch_two_step_kernel<kAnyWidth>;
+  kernel<<<grid, kTwoThreads, 0, q>>>(b->d_inst, b->d_two_items, b->d_two_chain + c,
+                                      b->buf[s & 1], b->buf[(s + 1) & 1], b->d_status);
+}
+
+void window_reduce(lbm_batch* b) {
+  batch_window_reduce<<<b->count, kReduceCta, 0, b->stream>>>(
+      b->d_inst, b->d_active, b->d_n_active + 1, b->buf[0], b->snap, b->rowmean, b->d_out,
+      float(b->p.tol));
+}
+
+// End the capture on the batch's stream and keep the graph under `key`.
+lbm_status keep_graph(lbm_batch* b, const std::vector<int>& key, cudaGraphExec_t* out) {
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamEndCapture(b->stream, &g);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return bfail(b, LBM_E_CUDA, std::string("capture: ") + cudaGetErrorString(e));
+  }
+  cudaGraphExec_t exec = nullptr;
+  e = cudaGraphInstantiate(&exec, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return bfail(b, LBM_E_CUDA, std::string("instantiate: ") + cudaGetErrorString(e));
+  }
+  if (b->graphs.size() >= kMaxGraphs) {  // (none is running: every window is waited for)
+    for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
+    b->graphs.clear();
+  }
+  b->graphs[key] = exec;
+  *out = exec;
+  return LBM_OK;
+}
+
 // One window as a CUDA graph, captured once per (mode, class grids) and
 // cached: the kernels read the active set and geometry from device memory,
 // so the graph stays valid as instances leave.
 lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
   const bool coop = mode == LBM_BATCH_COOPERATIVE;
   const int W = b->p.window;
-  // Two-step windows: an even number of two-step launches, so that the state
-  // ends in buf[0]; the two steps left over where W / 2 is odd go one by one.
-  const bool two = mode == kBatchTwoStep;
-  const int two_launches = two ? W / 4 * 2 : 0;
-  const int two_grid = two ? two_item_grid(*b->h_two_count) : 0;
-  const bool singles = !two || W % 4 != 0;
-  const int g0 = coop ? b->coop_grid : (singles ? class_grid(b, mode, 0) : 0);
-  const int g1 = coop || !singles ? 0 : class_grid(b, mode, 1);
-  const auto key = std::make_tuple(mode, two_grid, g0, g1);
+  const int g0 = coop ? b->coop_grid : class_grid(b, mode, 0);
+  const int g1 = coop ? 0 : class_grid(b, mode, 1);
+  const std::vector<int> key{mode, g0, g1};
   const auto it = b->graphs.find(key);
   if (it != b->graphs.end()) {
     *out = it->second;
     return LBM_OK;
   }
-  cudaGraph_t g = nullptr;
   LBM_BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   const int span = b->pers_grid_max + 1;
   // with both classes active they run as two branches of the graph, joined
@@ -867,12 +931,8 @@ lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
       cudaGetLastError();
       return bfail(b, LBM_E_CUDA, std::string("cooperative launch: ") + cudaGetErrorString(le));
     }
-  } else if (mode == LBM_BATCH_WORKLIST || two) {
-    for (int s = 0; s < two_launches; ++s)
-      batch_two_step_kernel<<<two_grid, kTwoThreads, 0, b->stream>>>(
-          b->d_inst, b->d_two_items, b->d_two_count, b->buf[s & 1], b->buf[(s + 1) & 1],
-          b->d_status);
-    for (int s = 2 * two_launches; s < W; ++s) {
+  } else if (mode == LBM_BATCH_WORKLIST) {
+    for (int s = 0; s < W; ++s) {
       fork();
       if (g0 > 0)
         batch_worklist_kernel<true><<<g0, kWorklistThreads, 0, b->stream>>>(
@@ -924,23 +984,65 @@ lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
           b->d_status);
     join();
   }
-  batch_window_reduce<<<b->count, kReduceCta, 0, b->stream>>>(
-      b->d_inst, b->d_active, b->d_n_active + 1, b->buf[0], b->snap, b->rowmean, b->d_out,
-      float(b->p.tol));
-  cudaError_t e = cudaStreamEndCapture(b->stream, &g);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return bfail(b, LBM_E_CUDA, std::string("capture: ") + cudaGetErrorString(e));
+  window_reduce(b);
+  return keep_graph(b, key, out);
+}
+
+// The chunk of launches that a two-step window replays: kTwoChunk launches of
+// every chain, side by side.  The chains advance different instances, so one
+// fills the SMs while another's launch ends and the next begins.
+lbm_status two_step_graph(lbm_batch* b, cudaGraphExec_t* out) {
+  std::vector<int> key{kBatchTwoStep};
+  for (const auto& c : b->two_chain) key.insert(key.end(), {c.first, c.second});
+  const auto it = b->graphs.find(key);
+  if (it != b->graphs.end()) {
+    *out = it->second;
+    return LBM_OK;
   }
-  cudaGraphExec_t exec = nullptr;
-  e = cudaGraphInstantiate(&exec, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return bfail(b, LBM_E_CUDA, std::string("instantiate: ") + cudaGetErrorString(e));
+  LBM_BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+  const int chains = int(b->two_chain.size());
+  cudaEventRecord(b->ev_fork, b->stream);
+  for (int c = 0; c < chains; ++c) {
+    const cudaStream_t q = c == 0 ? b->stream : b->two_side[c - 1];
+    if (c > 0) cudaStreamWaitEvent(q, b->ev_fork, 0);
+    for (int s = 0; s < kTwoChunk; ++s) two_step_chain(b, c, s, q);
+    if (c > 0) cudaEventRecord(b->two_join[c - 1], q);
   }
-  b->graphs[key] = exec;
-  *out = exec;
+  for (int c = 1; c < chains; ++c) cudaStreamWaitEvent(b->stream, b->two_join[c - 1], 0);
+  return keep_graph(b, key, out);
+}
+
+// Queue a two-step window: chunks of kTwoChunk launches, what is left of an
+// even number of launches (the state ends in buf[0]), the last two steps one
+// by one where W / 2 is odd, and the reduction.
+lbm_status two_step_window(lbm_batch* b) {
+  const int W = b->p.window;
+  int left = W / 4 * 2;
+  if (left >= kTwoChunk) {
+    cudaGraphExec_t g = nullptr;
+    const lbm_status st = two_step_graph(b, &g);
+    if (st != LBM_OK) return st;
+    for (; left >= kTwoChunk; left -= kTwoChunk) LBM_BCUDA(b, cudaGraphLaunch(g, b->stream));
+  }
+  for (int c = 0; c < int(b->two_chain.size()); ++c)
+    for (int s = 0; s < left; ++s) two_step_chain(b, c, s, b->stream);
+  if (W % 4 != 0) {
+    batch_copies_kernel<<<b->count, kReduceCta, 0, b->stream>>>(b->d_inst, b->d_active,
+                                                                b->d_n_active + 1, b->buf[0]);
+    const int g0 = class_grid(b, LBM_BATCH_WORKLIST, 0), g1 = class_grid(b, LBM_BATCH_WORKLIST, 1);
+    for (int s = 0; s < 2; ++s) {
+      if (g0 > 0)
+        batch_worklist_kernel<true><<<g0, kWorklistThreads, 0, b->stream>>>(
+            b->d_inst, b->d_active, b->d_prefix, b->d_n_active, b->buf[s], b->buf[1 - s],
+            b->d_status);
+      if (g1 > 0)
+        batch_worklist_kernel<false><<<g1, kWorklistThreads, 0, b->stream>>>(
+            b->d_inst, b->d_active, b->d_prefix, b->d_n_active, b->buf[s], b->buf[1 - s],
+            b->d_status);
+    }
+  }
+  window_reduce(b);
+  LBM_BCUDA(b, cudaGetLastError());
   return LBM_OK;
 }
 
@@ -1061,7 +1163,7 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
     d.nx = s.nx;
     d.ny = s.ny;
     d.pair = (s.nx % 2 == 0 || s.nx >= 3) && p->variant != LBM_VARIANT_REGISTER;
-    d.pitch = d.pair && s.nx % 2 ? s.nx + 3 : s.nx;
+    d.pitch = s.nx % 2 && p->variant != LBM_VARIANT_REGISTER ? s.nx + 3 : s.nx;
     d.n_strips = d.pair ? (s.nx + 63) / 64 : (s.nx + 31) / 32;
     d.scheme = s.scheme;
     d.row_off = roff;
@@ -1147,15 +1249,19 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
   }
   {
     long long items = 0;
-    for (const BatchInst& d : b->desc)
-      items += (long long)two_item_strips(d.nx) * two_item_bands(d.nx, d.ny, kTwoMinRows);
-    b->two_cap = int(items);
-    ok &= cudaMalloc(&b->d_two_items, size_t(b->two_cap) * sizeof(int4)) == cudaSuccess;
-    ok &= cudaMalloc(&b->d_two_count, sizeof(int)) == cudaSuccess;
+    for (const BatchInst& d : b->desc) {  // (no layout has more items than this one)
+      const TwoLattice t{0, d.nx, d.ny, kTwoBatchAny};
+      items += (long long)two_item_strips(t) * two_item_bands(t, kTwoMinRows);
+    }
+    ok &= cudaMalloc(&b->d_two_items, items * sizeof(int4)) == cudaSuccess;
+    ok &= cudaMalloc(&b->d_two_chain, kTwoMaxChains * sizeof(int2)) == cudaSuccess;
+    ok &= cudaMallocHost(&b->h_two_items, items * sizeof(int4)) == cudaSuccess;
+    ok &= cudaMallocHost(&b->h_two_chain, kTwoMaxChains * sizeof(int2)) == cudaSuccess;
+    for (int c = 0; c + 1 < kTwoMaxChains; ++c)
+      ok &= cudaStreamCreateWithFlags(&b->two_side[c], cudaStreamNonBlocking) == cudaSuccess &&
+            cudaEventCreateWithFlags(&b->two_join[c], cudaEventDisableTiming) == cudaSuccess;
   }
   if (!ok) return bail(LBM_E_NOMEM, "cudaMalloc");
-  ok &= cudaMallocHost(&b->h_two_items, size_t(b->two_cap) * sizeof(int4)) == cudaSuccess;
-  ok &= cudaMallocHost(&b->h_two_count, sizeof(int)) == cudaSuccess;
   ok &= cudaMallocHost(&b->h_active, count * sizeof(int)) == cudaSuccess;
   ok &= cudaMallocHost(&b->h_prefix, (count + 3) * sizeof(int)) == cudaSuccess;
   ok &= cudaMallocHost(&b->h_cta_begin, 2 * (b->pers_grid_max + 1) * sizeof(int)) ==
@@ -1231,9 +1337,13 @@ lbm_status lbm_batch_destroy(lbm_batch* b) {
   cudaFree(b->d_bal_items);
   cudaFree(b->d_bal_begin);
   cudaFree(b->d_two_items);
-  cudaFree(b->d_two_count);
+  cudaFree(b->d_two_chain);
   if (b->h_two_items) cudaFreeHost(b->h_two_items);
-  if (b->h_two_count) cudaFreeHost(b->h_two_count);
+  if (b->h_two_chain) cudaFreeHost(b->h_two_chain);
+  for (int c = 0; c + 1 < kTwoMaxChains; ++c) {
+    if (b->two_side[c]) cudaStreamDestroy(b->two_side[c]);
+    if (b->two_join[c]) cudaEventDestroy(b->two_join[c]);
+  }
   if (b->h_bal_items) cudaFreeHost(b->h_bal_items);
   if (b->h_bal_begin) cudaFreeHost(b->h_bal_begin);
   if (b->h_active) cudaFreeHost(b->h_active);
@@ -1379,7 +1489,7 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     lbm_status st = upload_tables(b, mode, rows);
     if (st != LBM_OK) return st;
     cudaGraphExec_t g = nullptr;
-    st = window_graph(b, mode, &g);
+    if (mode != kBatchTwoStep) st = window_graph(b, mode, &g);
     if (st != LBM_OK && mode == LBM_BATCH_COOPERATIVE && b->p.mode == LBM_BATCH_AUTO) {
       // cooperative windows unavailable here: drop them and use the work list
       b->coop_grid = 0;
@@ -1390,7 +1500,12 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     if (st != LBM_OK) return st;
     const size_t cells = active_cells(b);
     LBM_BCUDA(b, cudaEventRecord(b->ev0, b->stream));
-    LBM_BCUDA(b, cudaGraphLaunch(g, b->stream));
+    if (mode == kBatchTwoStep) {
+      st = two_step_window(b);
+      if (st != LBM_OK) return st;
+    } else {
+      LBM_BCUDA(b, cudaGraphLaunch(g, b->stream));
+    }
     LBM_BCUDA(b, cudaEventRecord(b->ev1, b->stream));
     // two class kernels per step (work list) or per window (persistent), one
     // kernel per two steps (two-step) or per window (cooperative), and the
@@ -1399,7 +1514,8 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
         (class_grid(b, mode, 0) > 0 ? 1 : 0) + (class_grid(b, mode, 1) > 0 ? 1 : 0);
     const unsigned long long W = b->p.window;
     const unsigned long long nl =
-        1 + (mode == kBatchTwoStep           ? W / 4 * 2 + (W % 4 ? 2 * classes : 0)
+        1 + (mode == kBatchTwoStep
+                 ? b->two_chain.size() * (W / 4 * 2) + (W % 4 ? 2 * classes + 1 : 0)
              : mode == LBM_BATCH_COOPERATIVE ? 1
              : mode == LBM_BATCH_PERSISTENT  ? classes
                                              : classes * W);

@@ -115,28 +115,57 @@ inline int balanced_schedule(const std::vector<BalColumn>& cols, int warps, int 
 struct TwoItem {
   int inst, strip, y0, y1;
 };
+// Row layouts of the two-step kernel among a batch's lattices: columns copied in
+// pairs (even nx), columns copied one by one (any nx, padded rows of odd ones),
+// whole rows in a warp (even nx <= 64).
+enum { kTwoBatchPairs = 0, kTwoBatchAny = 1, kTwoBatchRing = 2, kTwoBatchLayouts = 3 };
 struct TwoLattice {
   int inst, nx, ny;
+  int layout = kTwoBatchAny;
 };
 constexpr int kTwoItemCols = 56;  // columns of a strip
 
-// A lattice of at most 64 even columns is one strip of whole rows; up to 32
-// columns a warp takes two bands of it at once.
-inline bool two_item_ring(int nx) { return nx % 2 == 0 && nx <= 64; }
-inline int two_item_strips(int nx) {
-  return two_item_ring(nx) ? 1 : (nx + kTwoItemCols - 1) / kTwoItemCols;
+// Layouts for the lattices of a window.  Pairs are the fastest for even nx and
+// rings for narrow lattices, but several kernels side by side cost each other
+// instruction cache (24 even and 24 odd lattices, us per step: 42.1 with two
+// kernels, 40.6 with one for any nx; 36.0 if all are even): with an odd lattice
+// among them everything goes one by one, unless the narrow ones are a fifth
+// of the work or more.
+inline void two_layouts(std::vector<TwoLattice>& lat) {
+  double total = 0.0, narrow = 0.0;
+  bool odd = false;
+  for (const TwoLattice& t : lat) {
+    const double cells = double(t.nx) * t.ny;
+    total += cells;
+    if (t.nx % 2) odd = true;
+    else if (t.nx <= 64) narrow += cells;
+  }
+  for (TwoLattice& t : lat) {
+    const bool even = t.nx % 2 == 0;
+    if (even && t.nx <= 64 && (!odd || 5.0 * narrow >= total)) t.layout = kTwoBatchRing;
+    else t.layout = even && !odd ? kTwoBatchPairs : kTwoBatchAny;
+  }
+}
+
+// A ring is one strip of whole rows; up to 32 columns a warp takes two bands of
+// it at once.
+inline int two_item_strips(const TwoLattice& t) {
+  return t.layout == kTwoBatchRing ? 1 : (t.nx + kTwoItemCols - 1) / kTwoItemCols;
+}
+inline int two_item_halves(const TwoLattice& t) {
+  return t.layout == kTwoBatchRing && t.nx <= 32 ? 2 : 1;
 }
 // Items over the height of one strip for bands of `rows` rows.
-inline int two_item_bands(int nx, int ny, int rows) {
-  const int span = two_item_ring(nx) && nx <= 32 ? 2 * rows : rows;
-  return (ny + span - 1) / span;
+inline int two_item_bands(const TwoLattice& t, int rows) {
+  const int span = two_item_halves(t) * rows;
+  return (t.ny + span - 1) / span;
 }
 
 // Items for bands of about `rows` rows (each strip cut evenly), longest first.
 inline void two_items(const std::vector<TwoLattice>& lat, int rows, std::vector<TwoItem>& out) {
   out.clear();
   for (const TwoLattice& t : lat) {
-    const int n = two_item_bands(t.nx, t.ny, rows), strips = two_item_strips(t.nx);
+    const int n = two_item_bands(t, rows), strips = two_item_strips(t);
     for (int b = 0; b < n; ++b)
       for (int s = 0; s < strips; ++s)
         out.push_back(TwoItem{t.inst, s, int((long long)t.ny * b / n),
@@ -147,16 +176,54 @@ inline void two_items(const std::vector<TwoLattice>& lat, int rows, std::vector<
   });
 }
 
-// CTAs launched for `items` items: rounded up in steps of an eighth of the
-// leading power of two, so that a shrinking active set needs few graphs.
+// The lattices of a window as independent chains of launches, each of one
+// layout: about `wanted` in all, shared among the layouts by their cells (one
+// at least), the lattices of a layout spread over its chains by cells.
+struct TwoChain {
+  int layout;
+  std::vector<TwoLattice> lat;
+};
+inline std::vector<TwoChain> two_chains(const std::vector<TwoLattice>& all, int wanted) {
+  const auto cells = [](const TwoLattice& t) { return double(t.nx) * t.ny; };
+  double total = 0.0;
+  for (const TwoLattice& t : all) total += cells(t);
+  std::vector<TwoChain> out;
+  for (int layout = 0; layout < kTwoBatchLayouts; ++layout) {
+    std::vector<TwoLattice> mine;
+    double sum = 0.0;
+    for (const TwoLattice& t : all)
+      if (t.layout == layout) {
+        mine.push_back(t);
+        sum += cells(t);
+      }
+    if (mine.empty()) continue;
+    const int n = std::max(1, std::min(int(wanted * sum / total + 0.5), int(mine.size())));
+    std::stable_sort(mine.begin(), mine.end(), [&](const TwoLattice& x, const TwoLattice& y) {
+      return cells(x) > cells(y);
+    });
+    std::vector<double> load(n, 0.0);
+    const size_t first = out.size();
+    out.resize(first + n, TwoChain{layout, {}});
+    for (const TwoLattice& t : mine) {  // largest first, onto the least loaded
+      const int c = int(std::min_element(load.begin(), load.end()) - load.begin());
+      out[first + c].lat.push_back(t);
+      load[c] += cells(t);
+    }
+  }
+  return out;
+}
+
+// CTAs launched for `items` items: rounded up in steps of a quarter of the
+// leading power of two, so that a shrinking active set needs few graphs (a
+// CTA without an item costs its launch, well under a microsecond for all).
 inline int two_item_grid(int items) {
   int step = 64;
-  while (step * 16 <= items) step <<= 1;
+  while (step * 8 <= items) step <<= 1;
   return (items + step - 1) / step * step;
 }
 
 // Band height of a two-step launch over the active lattices, to start the
-// tuning from.  An item of n rows runs n + 7 iterations, of about 0.70, 1.10
+// tuning from.  An item of n rows costs about n + 3 iterations, of about 0.70, 1.10
 // or 1.45 us with 1, 2 or 3 warps per scheduler.  All items resident: the
 // launch ends with its longest; more items than resident warps: with the
 // work, plus the last items' share.
@@ -169,9 +236,8 @@ inline int two_item_rows(const std::vector<TwoLattice>& lat, int sm_count) {
                    80, 92, 106, 122, 140, 161, 185, 213, 256}) {
     double items = 0.0, work = 0.0, longest = 0.0;
     for (const TwoLattice& t : lat) {
-      const int n = two_item_bands(t.nx, t.ny, rows), strips = two_item_strips(t.nx);
-      const int halves = two_item_ring(t.nx) && t.nx <= 32 ? 2 : 1;
-      const double len = std::ceil(std::ceil(double(t.ny) / n) / halves) + 7.0;
+      const int n = two_item_bands(t, rows), strips = two_item_strips(t);
+      const double len = std::ceil(std::ceil(double(t.ny) / n) / two_item_halves(t)) + 3.0;
       items += double(n) * strips;
       work += double(n) * strips * len;
       longest = std::max(longest, len);

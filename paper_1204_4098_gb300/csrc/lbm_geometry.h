@@ -132,23 +132,23 @@ inline bool two_step_applies(int requested, int precision, int nx, int ny,
 }
 
 // Strips of 56 columns and the band height that ends first.  A band of n rows
-// runs n + 7 iterations; with 4, 8 or 12 warps per SM (1, 2 or 3 per
+// costs about n + 4 iterations; with 4, 8 or 12 warps per SM (1, 2 or 3 per
 // scheduler; numbers between leave one scheduler with more than the others
-// and end no earlier) an iteration takes 0.60, 0.94 and 1.32 us (1024^2,
-// improved scheme), so short bands of many warps pay only while the rows
-// dominate: 512^2 takes 4 warps per SM (5.2 us per step against 5.9 with 7 and 6.9
-// with 12), 1024^2 8 (10.9; 11.7 with 4, 11.9 with 12), 2048^2 12 (31.9; 32.2).
+// and end no earlier) an iteration takes 0.60, 0.92 and 1.30 us (improved
+// scheme), so short bands of many warps pay only while the rows dominate.
+// us per step with 4 / 8 / 12 warps: 512^2 4.78 / 4.99 / 5.37, 768^2 7.30 /
+// 6.79 / 7.30, 1024^2 11.1 / 9.87 / 10.5, 2048^2 38.9 / 31.3 / 30.5.
 inline StripGeometry two_step_geometry(int nx, int ny, int sm_count) {
   StripGeometry g;
   g.n_strips = (nx + kTwoStepCols - 1) / kTwoStepCols;
-  const double cost[3] = {0.60, 0.94, 1.32};
+  const double cost[3] = {0.60, 0.92, 1.30};
   double best = 0.0;
   g.band_rows = ny;
   for (int k = 0; k < 3; ++k) {
     const long long resident = (long long)sm_count * kTwoStepWarps * (k + 1) / 3;
     const long long bands = std::min<long long>(std::max<long long>(1, resident / g.n_strips), ny);
     const int rows = int((ny + bands - 1) / bands);
-    const double t = (rows + 7) * cost[k];
+    const double t = (rows + 4) * cost[k];
     if (k == 0 || t < best) {
       best = t;
       g.band_rows = rows;

@@ -26,19 +26,32 @@ int applies(int variant, int precision, int nx, int ny, int rows, double b) {
 static std::vector<lbm::TwoLattice> lattices(int n, const int* sizes) {
   std::vector<lbm::TwoLattice> v;
   for (int i = 0; i < n; ++i) v.push_back(lbm::TwoLattice{i, sizes[2 * i], sizes[2 * i + 1]});
+  lbm::two_layouts(v);
   return v;
 }
-int items(int n, const int* sizes, int rows, int* out, int cap) {
-  std::vector<lbm::TwoItem> v;
-  lbm::two_items(lattices(n, sizes), rows, v);
-  for (int k = 0; k < int(v.size()) && k < cap; ++k) {
-    out[4 * k] = v[k].inst; out[4 * k + 1] = v[k].strip;
-    out[4 * k + 2] = v[k].y0; out[4 * k + 3] = v[k].y1;
+// 6 ints per item: instance, strip, rows, chain, layout
+int items(int n, const int* sizes, int rows, int wanted, int* out, int cap) {
+  int m = 0, c = 0;
+  for (const lbm::TwoChain& chain : lbm::two_chains(lattices(n, sizes), wanted)) {
+    std::vector<lbm::TwoItem> v;
+    lbm::two_items(chain.lat, rows, v);
+    for (const lbm::TwoItem& t : v) {
+      if (m < cap) {
+        const int row[6] = {t.inst, t.strip, t.y0, t.y1, c, chain.layout};
+        for (int k = 0; k < 6; ++k) out[6 * m + k] = row[k];
+      }
+      ++m;
+    }
+    ++c;
   }
-  return int(v.size());
+  return m;
 }
-int bands(int nx, int ny, int rows) { return lbm::two_item_bands(nx, ny, rows); }
-int strips(int nx) { return lbm::two_item_strips(nx); }
+int bands(int nx, int ny, int rows) {
+  return lbm::two_item_bands(lbm::TwoLattice{0, nx, ny, lbm::kTwoBatchAny}, rows);
+}
+int strips(int nx) {
+  return lbm::two_item_strips(lbm::TwoLattice{0, nx, 1, lbm::kTwoBatchAny});
+}
 int grid(int n) { return lbm::two_item_grid(n); }
 int rows(int n, const int* sizes) { return lbm::two_item_rows(lattices(n, sizes), 152); }
 }
@@ -99,24 +112,43 @@ def test_which_lattices_take_two_steps(H):
         assert not H.applies(0, precision, 4095, 4096, 0, 4.0)
 
 
+MIXED = [(2, 9), (32, 320), (33, 7), (64, 1), (65, 100), (512, 300), (1, 5)]
+EVEN = [(2, 9), (32, 320), (64, 30), (66, 100), (512, 300)]
+NARROW = [(32, 320)] * 9 + [(33, 30), (1, 5)]
+
+
 @pytest.mark.parametrize("rows", [4, 7, 33, 500])
-def test_batch_items_cover_every_row_once_longest_first(H, rows):
+@pytest.mark.parametrize("first,odd", [(MIXED, True), (EVEN, False), (NARROW, True)])
+def test_batch_items_cover_every_row_once_longest_first(H, rows, first, odd):
     rng = np.random.default_rng(rows)
-    sizes = [(2, 9), (32, 320), (33, 7), (64, 1), (65, 100), (512, 300), (1, 5)] + \
-        [tuple(int(v) for v in rng.integers(1, 400, 2)) for _ in range(30)]
+    sizes = first + [tuple(int(v) for v in rng.integers(1, 30, 2) * (1 if odd else 2))
+                     for _ in range(20)]
     flat = (ctypes.c_int * (2 * len(sizes)))(*[v for s in sizes for v in s])
     cap = sum(H.strips(nx) * H.bands(nx, ny, 4) for nx, ny in sizes)  # as allocated
-    out = (ctypes.c_int * (4 * cap))()
-    n = H.items(len(sizes), flat, rows, out, cap)
+    out = (ctypes.c_int * (6 * cap))()
+    n = H.items(len(sizes), flat, rows, 3, out, cap)
     assert n <= cap
-    got = np.array(out[:4 * n]).reshape(n, 4)
-    lengths = got[:, 3] - got[:, 2]
-    assert np.all(lengths[:-1] >= lengths[1:]) and lengths[-1] >= 1
+    got = np.array(out[:6 * n]).reshape(n, 6)
+    chains = got[:, 4].max() + 1
+    assert 1 <= chains <= 3 + 3
+    for c in range(chains):  # one layout each, longest items first
+        mine = got[got[:, 4] == c]
+        lengths = mine[:, 3] - mine[:, 2]
+        assert len(set(mine[:, 5])) == 1
+        assert np.all(lengths[:-1] >= lengths[1:]) and lengths[-1] >= 1
     for i, (nx, ny) in enumerate(sizes):
-        for s in range(H.strips(nx)):
-            mine = got[(got[:, 0] == i) & (got[:, 1] == s)]
-            covered = np.concatenate([np.arange(a, b) for a, b in mine[:, 2:]])
+        mine = got[got[:, 0] == i]
+        assert len(set(mine[:, 4])) == 1  # an instance belongs to one chain
+        layout = mine[0, 5]
+        if layout == 0:
+            assert nx % 2 == 0
+        elif layout == 2:
+            assert nx % 2 == 0 and nx <= 64
+        for s in range(1 if layout == 2 else (nx + 55) // 56):
+            rows_of = mine[mine[:, 1] == s]
+            covered = np.concatenate([np.arange(a, b) for a, b in rows_of[:, 2:4]])
             assert sorted(covered) == list(range(ny))
+        assert mine[:, 1].max() == (0 if layout == 2 else (nx + 55) // 56 - 1)
     assert 4 <= H.rows(len(sizes), flat) <= 256
 
 
@@ -124,6 +156,6 @@ def test_grids_round_up_in_few_steps(H):
     seen = set()
     for n in range(1, 20000):
         g = H.grid(n)
-        assert n <= g <= max(n + 63, int(1.125 * n) + 1)
+        assert n <= g <= max(n + 63, int(1.25 * n) + 1)
         seen.add(g)
     assert len(seen) < 100
