@@ -182,11 +182,12 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
  * on the context stream: one per step, or, with the AUTO variant and band
  * height, one per up to four steps on small FP32 lattices (up to about 270^2
  * cells) and one per two steps on larger ones and for 16-bit storage with even
- * nx (an odd last step goes alone); on lattices of at most 2048^2 cells runs of 16 steps go through a
- * CUDA graph of these kernels, captured on first use for the current buffer
- * and launch arguments and kept until the context is destroyed (bit-identical
- * to single launches); while the caller captures the context stream into a
- * graph of its own, lbm_step_async records the launches one by one instead.  The call then waits for the kernels and
+ * nx (an odd last step goes alone); on lattices of at most 2048^2 cells runs
+ * of 16 steps, and of 64 in runs of at least 128, go through a CUDA graph of
+ * these kernels, captured on first use for the current buffer and launch
+ * arguments and kept until the context is destroyed (bit-identical to single
+ * launches); while the caller captures the context stream into a graph of its
+ * own, lbm_step_async records the launches one by one instead.  The call then waits for the kernels and
  * reads the device status word once (so lbm_step itself cannot be
  * captured).  LBM_E_DIVERGED if psi became undefined in any step (the state
  * is then unspecified but the context stays usable and destroyable);

@@ -234,13 +234,14 @@ struct lbm_ctx {
   int ny_buf = 0;
   int row0 = 0;
   cudaEvent_t packed = nullptr;  // overlapped band step: boundary rows packed
-  // Step graphs of small lattices (queue_steps): one per buffer parity, with
-  // the launch arguments of its first step.
+  // Step graphs of small lattices (queue_steps): of kGraphSteps and of
+  // kLongGraphSteps steps, one per buffer parity, with the launch arguments of
+  // the first step.
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     StripLaunch L{};
     int scheme = -1, variant = -1, grid = 0;
-  } graph[2];
+  } graph[2][2];
   cudaStream_t cap_stream = nullptr;  // private stream the graphs are captured on
   // lbm_get_moments on large lattices: row chunks copied on copy_stream while
   // the next chunk is computed; obs_ev[k] marks chunk k computed, obs_ev[last]
@@ -397,7 +398,15 @@ lbm_status launch_rows(lbm_ctx* c, int scheme, StripLaunch L, int r0, int r1, in
 // them with shorter gaps (~4 us per step there, a few per cent faster up to
 // 2048^2).  From 4096^2 on the step's own time hides the gap.
 constexpr int kGraphSteps = 16;
-static_assert(kGraphSteps % 4 == 0 && kGraphSteps / kTileSteps % 2 == 0,
+// A replay itself costs 2 us or so of the GPU's time between its last kernel
+// and the next replay's first, which is felt with 4 launches of 4 us in it:
+// runs of at least kLongGraphRun steps go in graphs of kLongGraphSteps (64^2:
+// 1.28 -> 1.12 us per step, 200^2 1.92 -> 1.70, 1024^2 9.87 -> 9.75; four
+// times as long again gains another 1 %).
+constexpr int kLongGraphSteps = 64;
+constexpr int kLongGraphRun = 2 * kLongGraphSteps;
+static_assert(kGraphSteps / kTileSteps % 2 == 0 && kGraphSteps % kTileSteps == 0 &&
+                  kLongGraphSteps % kGraphSteps == 0,
               "a graph is an even number of launches of each kind");
 constexpr size_t kGraphMaxCells = size_t(2048) * 2048;
 
@@ -477,13 +486,13 @@ bool same_launch(const StripLaunch& x, const StripLaunch& y) {
          x.s_q == y.s_q;
 }
 
-// The cached graph of kGraphSteps steps from the current buffer, captured
+// The cached graph of `steps` steps from the current buffer, captured
 // again when any kernel argument, the scheme, the kernel variant or the grid
 // changed; nullptr when capture is unavailable (the caller then launches
 // step by step).  With two or kTileSteps steps per launch the number of
 // launches is even too, so a replay leaves the state in the same buffer.
-cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan) {
-  lbm_ctx::StepGraph& g = c->graph[c->cur];
+cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan, int steps) {
+  lbm_ctx::StepGraph& g = c->graph[steps == kLongGraphSteps][c->cur];
   const bool single = plan.kind == kSingleSteps;
   const int variant = single ? pick_variant(c, kStepMode) : -plan.kind;
   const int grid = single ? plan.one_grid : plan.many_grid;
@@ -511,7 +520,7 @@ cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan) {
   cudaGraph_t graph = nullptr;
   bool ok = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) ==
             cudaSuccess;
-  ok = ok && run_plan(c, scheme, scratch, kGraphSteps, c->cap_stream, &launches) == cudaSuccess;
+  ok = ok && run_plan(c, scheme, scratch, steps, c->cap_stream, &launches) == cudaSuccess;
   c->cur = cur0;  // capturing ran nothing
   const bool ended = cudaStreamEndCapture(c->cap_stream, &graph) == cudaSuccess;
   cudaGraphExec_t exec = nullptr;
@@ -576,12 +585,15 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
     capturing = cudaStreamCaptureStatusActive;
   }
   if (graphs && capturing == cudaStreamCaptureStatusNone) {
-    const cudaGraphExec_t g = step_graph(c, scheme, plan);
-    if (g)
-      for (; k + kGraphSteps <= n; k += kGraphSteps) {
+    for (const int steps : {kLongGraphSteps, kGraphSteps}) {
+      if (n - k < (steps == kLongGraphSteps ? kLongGraphRun : kGraphSteps)) continue;
+      const cudaGraphExec_t g = step_graph(c, scheme, plan, steps);
+      if (!g) break;
+      for (; k + steps <= n; k += steps) {
         LBM_CUDA(c, cudaGraphLaunch(g, c->stream));  // the state returns to c->cur
-        launches += kGraphSteps / next_launch(plan, kGraphSteps);
+        launches += steps / next_launch(plan, steps);
       }
+    }
   }
   const cudaError_t e = run_plan(c, scheme, plan, n - k, c->stream, &launches);
   if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
@@ -780,8 +792,9 @@ lbm_status lbm_destroy(lbm_ctx* c) {
   cudaFree(c->d_tmp);
   cudaFree(c->d_pop);
   if (c->packed) cudaEventDestroy(c->packed);
-  for (auto& g : c->graph)
-    if (g.exec) cudaGraphExecDestroy(g.exec);
+  for (auto& length : c->graph)
+    for (auto& g : length)
+      if (g.exec) cudaGraphExecDestroy(g.exec);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   for (cudaEvent_t e : c->obs_ev)
     if (e) cudaEventDestroy(e);

@@ -77,6 +77,25 @@ def test_schemes_and_step_graphs(scheme, nx, ny):
     assert np.array_equal(auto, ref)
 
 
+@pytest.mark.parametrize("nx,ny,precision", [(97, 60, lbm.FP32), (601, 301, lbm.FP32),
+                                             (200, 190, lbm.BF16DEV), (60, 50, lbm.FP64)])
+def test_long_runs_in_step_graphs(nx, ny, precision):
+    # graphs of 64 and of 16 steps from either buffer, and what is left
+    out = []
+    for variant in (lbm.VARIANT_AUTO, lbm.VARIANT_REGISTER):
+        with lbm.Lattice(nx, ny, T, precision=precision) as lat:
+            lat.set_variant(variant)
+            lat.init_density(*field(nx, ny, 7))
+            for n in (1, 151, 128, 3, 127, 64):
+                if variant == lbm.VARIANT_AUTO:
+                    lat.step(n, lbm.IMPROVED, 0.8, 0.1)
+                else:
+                    for _ in range(n):
+                        lat.step(1, lbm.IMPROVED, 0.8, 0.1)
+            out.append(lat.populations())
+    assert np.array_equal(*out)
+
+
 @pytest.mark.parametrize("rows", [slice(None), slice(100, 140)])
 @pytest.mark.parametrize("scheme", [lbm.IMPROVED, lbm.NOFORCE])
 @pytest.mark.parametrize("nx,ny", [(190, 240), (590, 240)])
