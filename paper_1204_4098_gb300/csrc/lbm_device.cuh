@@ -187,6 +187,55 @@ __device__ __forceinline__ V quot_one(V b, C) {  // 1 / b
   else return recip(b);
 }
 
+// FP64 value of an FP32 number, from its bits (integer operations: FP64
+// conversions share the 2 lanes a clock and SM of the FP64 pipe).
+__device__ __forceinline__ double widen_normal(float v) {
+  const unsigned u = __float_as_uint(v);
+  return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                          int(u << 29));
+}
+
+// Density and actual velocity (j + F / 2) / rho of a cell as FP64 values, the
+// quotients rounded to FP64.  The general form takes ~27 slots of the FP64
+// pipe a cell, which bounded the read-back kernel (2048^2: 190 us, against 37
+// of memory traffic; 80 us with this one, the read-back of 1024^2 with its
+// copies 205 -> 178 us).  Here the reciprocal starts from the FP32 one:
+// e = 1 - rho inv (one rounding of a number of ~24 bits) gives R = inv (1 +
+// e), 1 / rho up to e^2 ~ 2^-46, and n R plus its remainder (n - n R rho) R
+// is n / rho up to 2^-92 before its one rounding: the division's value (the
+// residual correction of Markstein, IBM J. Res. Dev. 34, 1990).  One FP64
+// operation for R and three for each quotient.  Operands outside the range
+// where every intermediate is normal take the division.
+__device__ __forceinline__ void actual_velocity(double jx, double jy, double rho, double Fx,
+                                                double Fy, double& out_rho, double& out_vx,
+                                                double& out_vy) {
+  out_rho = rho;
+  out_vx = (jx + 0.5 * Fx) / rho;
+  out_vy = (jy + 0.5 * Fy) / rho;
+}
+__device__ __forceinline__ void actual_velocity(float jx, float jy, float rho, float Fx, float Fy,
+                                                double& out_rho, double& out_vx,
+                                                double& out_vy) {
+  constexpr float kLeast = 0x1p-60f, kMost = 0x1p60f;
+  auto plain = [](float v) { return fabsf(v) < kMost && (fabsf(v) > kLeast || v == 0.f); };
+  if (rho > kLeast && rho < kMost && plain(jx) && plain(jy) && plain(Fx) && plain(Fy)) {
+    const float inv = rcp_normal(rho), e = __fmaf_rn(-rho, inv, 1.f);
+    const double r = widen_normal(rho), i = widen_normal(inv), d = widen_normal(e);
+    const double R = __fma_rn(i, d, i);  // (e = 0 widens to 2^-127: R = inv)
+    auto widen = [](float v) { return v == 0.f ? 0.0 : widen_normal(v); };
+    auto quotient = [&](float j, float F) {
+      const double n = __fma_rn(0.5, widen(F), widen(j)), q = __dmul_rn(n, R);
+      return __fma_rn(__fma_rn(-q, r, n), R, q);
+    };
+    out_rho = r;
+    out_vx = quotient(jx, Fx);
+    out_vy = quotient(jy, Fy);
+  } else {
+    actual_velocity(double(jx), double(jy), double(rho), double(Fx), double(Fy), out_rho, out_vx,
+                    out_vy);
+  }
+}
+
 // psi of Eq. 8 with the Carnahan-Starling p_EOS of Eq. 23.  Flags (and
 // returns 0 for) densities outside the domain of psi: rho <= 0, eta >= 1,
 // a negative or non-finite radicand.  psi_radicand holds the arithmetic
@@ -237,6 +286,21 @@ __device__ __forceinline__ Pair<C> psi_of_rho(Pair<C> rho, const Phys<C>& P, boo
   psi_radicand(rho, P, eta, om, arg);
   return Pair<C>(psi_finish(rho.x(), eta.x(), arg.x(), bad),
                  psi_finish(rho.y(), eta.y(), arg.y(), bad));
+}
+
+// Flags a given density outside the domain of psi.  The check itself takes
+// ~23 FP64 operations; a density whose FP32 radicand lies above 1e-3 of its
+// terms' magnitude, where FP32 with eta < 0.9 is good to ~1e-5 of it, is
+// inside, so the FP64 form runs only near the domain's edges.
+__device__ __forceinline__ void check_domain(double rho, const Phys<double>& P,
+                                             const Phys<float>& F, bool& bad) {
+  const float r = float(rho), eta = F.b4 * r, om = 1.f - eta;
+  const float t = r * F.RT * fmaf(eta, fmaf(eta, om, 1.f), 1.f) / (om * om * om);
+  const float u = F.a * r * r, third = r * (1.f / 3.f);
+  const float arg = F.two_over_G * ((t - u) - third);
+  const float terms = fabsf(F.two_over_G) * (fabsf(t) + u + third);
+  const bool inside = r > 1e-30f && eta < 0.9f && arg > 1e-3f * terms && terms < 1e25f;
+  if (!inside) (void)psi_of_rho(rho, P, bad);
 }
 
 // ---------------------------------------------------------------------------

@@ -193,8 +193,22 @@ cudaError_t set_state_t(void* dst, float* rho_dst, int nx, int ny, int pitch, si
   P.a = chk.a;
   P.b4 = chk.b4;
   P.two_over_G = chk.two_over_G;
+  Phys<float> F{};
+  F.RT = float(chk.RT);
+  F.a = float(chk.a);
+  F.b4 = float(chk.b4);
+  F.two_over_G = float(chk.two_over_G);
+  if constexpr (!S::kDev) {
+    if (!f_in && pitch == nx) {
+      const unsigned rows = kPushThreads / 32, bands = (unsigned(ny) + rows - 1) / rows;
+      const dim3 grid((unsigned(nx) + 31) / 32, bands < 65535u ? bands : 65535u);
+      push_state_kernel<S><<<grid, kPushThreads, 0, s>>>(static_cast<typename S::T*>(dst), nx, ny,
+                                                        plane, rho, ux, uy, P, F, chk.status);
+      return cudaGetLastError();
+    }
+  }
   set_state_kernel<S><<<grid_for(plane, 256), 256, 0, s>>>(
-      static_cast<typename S::T*>(dst), rho_dst, nx, ny, pitch, plane, rho, ux, uy, f_in, P,
+      static_cast<typename S::T*>(dst), rho_dst, nx, ny, pitch, plane, rho, ux, uy, f_in, P, F,
       chk.status);
   return cudaGetLastError();
 }
