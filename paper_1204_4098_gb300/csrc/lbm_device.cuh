@@ -217,7 +217,8 @@ __device__ __forceinline__ void actual_velocity(float jx, float jy, float rho, f
                                                 double& out_rho, double& out_vx,
                                                 double& out_vy) {
   constexpr float kLeast = 0x1p-60f, kMost = 0x1p60f;
-  auto plain = [](float v) { return fabsf(v) < kMost && (fabsf(v) > kLeast || v == 0.f); };
+  // (a NaN fails its comparison)
+  const auto plain = [](float v) { return fabsf(v) < kMost && (fabsf(v) > kLeast || v == 0.f); };
   if (rho > kLeast && rho < kMost && plain(jx) && plain(jy) && plain(Fx) && plain(Fy)) {
     const float inv = rcp_normal(rho), e = __fmaf_rn(-rho, inv, 1.f);
     const double r = widen_normal(rho), i = widen_normal(inv), d = widen_normal(e);
@@ -231,8 +232,11 @@ __device__ __forceinline__ void actual_velocity(float jx, float jy, float rho, f
     out_vx = quotient(jx, Fx);
     out_vy = quotient(jy, Fy);
   } else {
-    actual_velocity(double(jx), double(jy), double(rho), double(Fx), double(Fy), out_rho, out_vx,
-                    out_vy);
+    out_rho = double(rho);
+#pragma unroll 1  // one division's code and registers
+    for (int k = 0; k < 2; ++k)
+      (k ? out_vy : out_vx) =
+          (double(k ? jy : jx) + 0.5 * double(k ? Fy : Fx)) / double(rho);
   }
 }
 
