@@ -180,10 +180,11 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
 /* Advance n >= 0 time steps with the given scheme and relaxation time
  * tau > 1/2 (sigma is read by LBM_SCHEME_IMPROVED only).  Kernels are queued
  * on the context stream: one per step, or, with the AUTO variant and band
- * height, one per up to four steps on small FP32 lattices (up to about 270^2
- * cells) and one per two steps on larger ones and for 16-bit storage with even
+ * height, one per up to four steps on small FP32 lattices (four up to about
+ * 270^2 cells, three or two up to about 370^2) and one per two steps on larger ones and for 16-bit storage with even
  * nx (an odd last step goes alone); on lattices of at most 2048^2 cells runs
- * of 16 steps, and of 64 in runs of at least 128, go through a CUDA graph of
+ * of 16 steps, and of 64 in runs of at least 128 (of 4 and 16 launches where a
+ * launch takes several steps of a small lattice), go through a CUDA graph of
  * these kernels, captured on first use for the current buffer and launch
  * arguments and kept until the context is destroyed (bit-identical to single
  * launches); while the caller captures the context stream into a graph of its

@@ -234,9 +234,8 @@ struct lbm_ctx {
   int ny_buf = 0;
   int row0 = 0;
   cudaEvent_t packed = nullptr;  // overlapped band step: boundary rows packed
-  // Step graphs of small lattices (queue_steps): of kGraphSteps and of
-  // kLongGraphSteps steps, one per buffer parity, with the launch arguments of
-  // the first step.
+  // Step graphs of small lattices (queue_steps), a short and a long one per
+  // buffer parity, with the launch arguments of the first step.
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     StripLaunch L{};
@@ -391,22 +390,24 @@ lbm_status launch_rows(lbm_ctx* c, int scheme, StripLaunch L, int r0, int r1, in
   return LBM_OK;
 }
 
-// Steps per captured step graph (even: a replay leaves the state in the same
-// buffer) and the lattice size up to which steps go through graphs.  With
-// one launch per step a small lattice (64^2 to 256^2) takes a flat ~6.2 us
-// per step however little it computes; a graph of the same kernels replays
-// them with shorter gaps (~4 us per step there, a few per cent faster up to
-// 2048^2).  From 4096^2 on the step's own time hides the gap.
+// Steps per captured step graph (an even number of launches: a replay leaves
+// the state in the same buffer) and the lattice size up to which steps go
+// through graphs.  With one launch per step a small lattice (64^2 to 256^2)
+// takes a flat ~6.2 us per step however little it computes; a graph of the
+// same kernels replays them with shorter gaps (~4 us per step there, a few
+// per cent faster up to 2048^2).  From 4096^2 on the step's own time hides the
+// gap.
 constexpr int kGraphSteps = 16;
 // A replay itself costs 2 us or so of the GPU's time between its last kernel
 // and the next replay's first, which is felt with 4 launches of 4 us in it:
-// runs of at least kLongGraphRun steps go in graphs of kLongGraphSteps (64^2:
-// 1.28 -> 1.12 us per step, 200^2 1.92 -> 1.70, 1024^2 9.87 -> 9.75; four
-// times as long again gains another 1 %).
+// runs of at least twice as many steps go in graphs of 64 (64^2: 1.28 -> 1.12
+// us per step, 200^2 1.92 -> 1.70, 1024^2 9.87 -> 9.75; four times as long
+// again gains another 1 %).
 constexpr int kLongGraphSteps = 64;
-constexpr int kLongGraphRun = 2 * kLongGraphSteps;
-static_assert(kGraphSteps / kTileSteps % 2 == 0 && kGraphSteps % kTileSteps == 0 &&
-                  kLongGraphSteps % kGraphSteps == 0,
+// Graphs of tile launches: 4 launches and 16, however many steps each takes.
+constexpr int kGraphTiles = 4, kLongGraphTiles = 16;
+static_assert(kGraphTiles % 2 == 0 && kLongGraphTiles % 2 == 0 && kGraphSteps % 4 == 0 &&
+                  kLongGraphSteps % 4 == 0,
               "a graph is an even number of launches of each kind");
 constexpr size_t kGraphMaxCells = size_t(2048) * 2048;
 
@@ -429,19 +430,25 @@ cudaError_t launch_step(lbm_ctx* c, int scheme, StripLaunch& L, int grid, cudaSt
 }
 
 // The launches of a run of steps: `one` step each, and where the lattice takes
-// them `many`: up to kTileSteps on tiles, or two.
+// them `many`: up to tile_steps on tiles, or two.
 enum { kSingleSteps = 0, kTwoSteps = 1, kTileRuns = 2 };
 struct StepPlan {
   StripLaunch one;
   int one_grid = 0;
   int kind = kSingleSteps;
   StripLaunch many;
-  int many_grid = 0, many_threads = 0;
+  int many_grid = 0, many_threads = 0, tile_steps = 0;
 };
+
+// Steps of the shorter and of the longer step graph.
+int graph_steps(const StepPlan& plan, bool longer) {
+  if (plan.kind == kTileRuns) return plan.tile_steps * (longer ? kLongGraphTiles : kGraphTiles);
+  return longer ? kLongGraphSteps : kGraphSteps;
+}
 
 // Steps of the next launch when n are left.
 int next_launch(const StepPlan& plan, int n) {
-  if (plan.kind == kTileRuns) return std::min(n, kTileSteps);
+  if (plan.kind == kTileRuns) return std::min(n, plan.tile_steps);
   return plan.kind == kTwoSteps && n >= 2 ? 2 : 1;
 }
 
@@ -461,8 +468,8 @@ cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t
       plan.many.rho_src = c->rho[s];
       plan.many.rho_dst = c->rho[d];
       e = plan.kind == kTileRuns
-              ? tile_steps_launch(scheme, plan.many, steps, plan.many_grid, plan.many_threads,
-                                  stream)
+              ? tile_steps_launch(scheme, plan.many, steps, plan.tile_steps, plan.many_grid,
+                                  plan.many_threads, stream)
               : two_step_launch(c->p.precision, scheme, plan.many, plan.many_grid, stream);
       if (e == cudaSuccess) c->cur = d;
     }
@@ -486,13 +493,13 @@ bool same_launch(const StripLaunch& x, const StripLaunch& y) {
          x.s_q == y.s_q;
 }
 
-// The cached graph of `steps` steps from the current buffer, captured
-// again when any kernel argument, the scheme, the kernel variant or the grid
+// The cached graph (the shorter or the longer one) of steps from the current
+// buffer, captured again when any kernel argument, the scheme, the kernel variant or the grid
 // changed; nullptr when capture is unavailable (the caller then launches
-// step by step).  With two or kTileSteps steps per launch the number of
-// launches is even too, so a replay leaves the state in the same buffer.
-cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan, int steps) {
-  lbm_ctx::StepGraph& g = c->graph[steps == kLongGraphSteps][c->cur];
+// step by step).  The number of launches is even, so a replay leaves the
+// state in the same buffer.
+cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan, bool longer) {
+  lbm_ctx::StepGraph& g = c->graph[longer][c->cur];
   const bool single = plan.kind == kSingleSteps;
   const int variant = single ? pick_variant(c, kStepMode) : -plan.kind;
   const int grid = single ? plan.one_grid : plan.many_grid;
@@ -520,7 +527,8 @@ cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan, int ste
   cudaGraph_t graph = nullptr;
   bool ok = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) ==
             cudaSuccess;
-  ok = ok && run_plan(c, scheme, scratch, steps, c->cap_stream, &launches) == cudaSuccess;
+  ok = ok && run_plan(c, scheme, scratch, graph_steps(plan, longer), c->cap_stream,
+                      &launches) == cudaSuccess;
   c->cur = cur0;  // capturing ran nothing
   const bool ended = cudaStreamEndCapture(c->cap_stream, &graph) == cudaSuccess;
   cudaGraphExec_t exec = nullptr;
@@ -563,6 +571,7 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
       plan.many.band_rows = t.rows;
       plan.many_grid = t.grid;
       plan.many_threads = t.threads;
+      plan.tile_steps = t.steps;
     } else if (two_step_applies(c->variant, c->p.precision, c->p.nx, c->p.ny,
                                 c->band_rows_override, c->p.b)) {
       const StripGeometry g = two_step_geometry(c->p.nx, c->p.ny, c->sm_count);
@@ -577,17 +586,18 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
   int k = 0, launches = 0;
   // (not while the caller captures the context stream into a graph of its
   // own: the steps are then recorded one launch at a time)
-  const bool graphs =
-      !c->band && n >= kGraphSteps && size_t(c->p.nx) * c->p.ny <= kGraphMaxCells;
+  const bool graphs = !c->band && n >= graph_steps(plan, false) &&
+                      size_t(c->p.nx) * c->p.ny <= kGraphMaxCells;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   if (graphs && cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) {
     cudaGetLastError();  // treated as capturing: plain launches
     capturing = cudaStreamCaptureStatusActive;
   }
   if (graphs && capturing == cudaStreamCaptureStatusNone) {
-    for (const int steps : {kLongGraphSteps, kGraphSteps}) {
-      if (n - k < (steps == kLongGraphSteps ? kLongGraphRun : kGraphSteps)) continue;
-      const cudaGraphExec_t g = step_graph(c, scheme, plan, steps);
+    for (const bool longer : {true, false}) {
+      const int steps = graph_steps(plan, longer);
+      if (n - k < (longer ? 2 * steps : steps)) continue;
+      const cudaGraphExec_t g = step_graph(c, scheme, plan, longer);
       if (!g) break;
       for (; k + steps <= n; k += steps) {
         LBM_CUDA(c, cudaGraphLaunch(g, c->stream));  // the state returns to c->cur

@@ -160,43 +160,45 @@ inline StripGeometry two_step_geometry(int nx, int ny, int sm_count) {
 }
 
 // ---------------------------------------------------------------------------
-// four steps per launch on tiles (lbm_tile_steps.cuh)
+// several steps per launch on tiles (lbm_tile_steps.cuh)
 // ---------------------------------------------------------------------------
-constexpr int kTileSteps = 4;
-constexpr int kTileHalo = 2 * kTileSteps;      // cells around a tile that its steps reach
-constexpr int kTileCols = 32 - 2 * kTileHalo;  // columns a tile owns
-constexpr int kTileMaxWarps = 24;              // two rows each
+constexpr int kTileMinSteps = 2, kTileMaxSteps = 4;  // steps per launch
+constexpr int kTileMaxWarps = 24;                    // two rows each
 
 struct TileGeometry {
   int n_cols;   // tiles side by side
   int rows;     // rows a tile owns; 0: the lattice does not take tiles
   int grid;     // tiles
   int threads;  // per CTA
+  int steps;    // steps of a launch
 };
 
 // Tiles for a lattice that they cover in one wave, one CTA per SM: as many
-// rows of tiles as there are SMs for, at most 32 lattice rows each (48 with
-// the halo).  Up to there tiles are the fastest at every size (128^2: 1.41 us
-// per step with 152 tiles of 7 rows, 1.66 with 72 of 15); where a second wave
-// starts they only tie with two-step launches (300^2: 3.20 against 3.58).
-// The same requirements on variant, storage, band height and covolume as
-// two_step_applies.
+// rows of tiles as there are SMs for, at most 48 lattice rows each with the
+// halo of two cells per step.  Up to there tiles are the fastest at every size
+// (128^2: 1.41 us per step with 152 tiles of 7 rows, 1.66 with 72 of 15; a
+// second wave only ties with two-step launches: 300^2 with four steps 3.02).
+// Fewer steps leave more columns and rows to a tile, so a lattice takes the
+// most steps that fit, us per step with 4 / 3 / 2 and of the two-step strips:
+// 64^2 1.10 / 1.29 / 1.42, 128^2 1.26 / 1.42 / 1.55, 200^2 1.71 / 1.72 / 1.93,
+// 256^2 2.12 / 2.06 / 2.12, 300^2 - / 2.40 / 2.57 / 3.02.  (Five steps gain 3 %
+// at 16^2 and 1 % at 64^2 and lose from 96^2 on.)  The same requirements on
+// variant, storage, band height and covolume as two_step_applies.
 inline TileGeometry tile_geometry(int requested, int precision, int nx, int ny,
                                   int band_rows_override, double b, int sm_count) {
-  TileGeometry g{0, 0, 0, 0};
+  const TileGeometry none{0, 0, 0, 0, 0};
   if (requested != LBM_VARIANT_AUTO || band_rows_override != 0 || precision != LBM_FP32 ||
       !(b > 1e-12 && b < 1e12))
-    return g;
-  const int cols = nx / kTileCols + (nx % kTileCols != 0);
-  if (cols > sm_count) return g;
-  const int tile_rows = std::min(ny, sm_count / cols);
-  const int rows = (ny - 1) / tile_rows + 1;
-  if (rows + 2 * kTileHalo > 2 * kTileMaxWarps) return g;
-  g.n_cols = cols;
-  g.rows = rows;
-  g.grid = cols * ((ny - 1) / rows + 1);
-  g.threads = 32 * ((rows + 2 * kTileHalo + 1) / 2);
-  return g;
+    return none;
+  for (int steps = kTileMaxSteps; steps >= kTileMinSteps; --steps) {
+    const int halo = 2 * steps, cols = (nx - 1) / (32 - 2 * halo) + 1;
+    if (cols > sm_count) continue;
+    const int tile_rows = std::min(ny, sm_count / cols), rows = (ny - 1) / tile_rows + 1;
+    if (rows + 2 * halo > 2 * kTileMaxWarps) continue;
+    return TileGeometry{cols, rows, cols * ((ny - 1) / rows + 1),
+                        32 * ((rows + 2 * halo + 1) / 2), steps};
+  }
+  return none;
 }
 
 }  // namespace lbm

@@ -1,14 +1,15 @@
-// Four time steps per launch for small lattices (FP32 storage).
+// Two to four time steps per launch for small lattices (FP32 storage).
 //
-// A lattice of up to ~270^2 cells is spread thinly over the GPU: its step is
+// A lattice of up to ~370^2 cells is spread thinly over the GPU: its step is
 // a chain of latencies (launch, load, one or two rows of arithmetic, store)
 // that leaves nearly every issue slot empty, and no band height shortens it.
-// Here a CTA takes a tile of 16 columns and a few rows together with the 8
+// Here a CTA takes a tile of a few rows and 16 columns together with the 8
 // cells around it that four steps reach (two per step: the pull and the psi
-// stencil), and runs the four steps in shared memory between one load and one
+// stencil), and runs the steps in shared memory between one load and one
 // store.  Neighbouring CTAs compute the overlap again -- about twice the work
 // of the lattice -- on SMs that would otherwise wait; nothing is exchanged
-// between them.
+// between them.  A lattice too large for tiles of four steps takes three or
+// two, with 20 or 24 columns (tile_geometry).
 //
 // A warp owns two rows of the tile, a lane one column: every population pulled
 // is one conflict-free shared load, the two rows are one packed pair of the
@@ -22,11 +23,13 @@
 // again with the full forms.
 //
 // Measured, us per step in step graphs (improved scheme), best other kernel ->
-// this: 32^2 2.69 -> 1.28, 64^2 2.69 -> 1.15, 128^2 2.76 -> 1.41, 200^2 3.20 ->
-// 1.79, 256^2 3.46 -> 2.18; 280^2 would need two waves of tiles (3.46 -> 3.20) and
-// larger lattices gain nothing.  Of the 4.6 us of a 64^2 launch the four steps
-// take about 1.4, the rest is the launch, the load and the store; programmatic
-// dependent launch changed nothing.
+// this: 32^2 2.69 -> 1.06, 64^2 2.69 -> 1.10, 128^2 2.76 -> 1.26, 200^2 3.20 ->
+// 1.71, 256^2 3.46 -> 2.12 with four steps, 300^2 3.02 -> 2.41 with three, 360^2
+// 3.53 -> 3.08 with two.  A launch takes about 1.8 us + 0.24 us and 0.03 us per
+// active row for every step + 0.03 us per row loaded: at 64^2 a third of its 4.4
+// us is the launch itself, the rest mostly one warp's serial row of arithmetic.
+// Tried without gain: one row per warp, programmatic dependent launch (64^2:
+// 1.34), five steps (64^2 1.09, 96^2 1.10 -> 1.19).
 #pragma once
 
 #include "lbm_geometry.h"
@@ -34,7 +37,7 @@
 
 namespace lbm {
 
-// (kTileSteps, kTileHalo, kTileCols, kTileMaxWarps: lbm_geometry.h)
+// (kTileMaxWarps: lbm_geometry.h)
 constexpr int kTilePlanes = kQ + 1;  // populations and psi
 
 // psi of a pair whose elements may be out of use (kNormal: ok says whether
@@ -50,23 +53,23 @@ __device__ __forceinline__ F2 psi_normal_masked(F2 rho, const Phys<float>& P, bo
 }
 
 // The tile whose first owned cell is (x0, y0), `rows` owned rows; f: shared
-// memory, kTilePlanes planes of H x 32 floats, H = 2 warps >= rows + 16;
-// 1 <= steps <= kTileSteps.
+// memory, kTilePlanes planes of H x 32 floats, H = 2 warps >= rows + 2 halo;
+// 1 <= steps <= halo / 2.
 // Returns (to every thread of the CTA) whether every check held.
 template <int SCHEME, bool kNormal>
-__device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps, int x0, int y0,
-                                         int rows, float* f) {
+__device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps, int halo,
+                                         int x0, int y0, int rows, float* f) {
   constexpr bool kNeedPsi = SCHEME != kNoForce;
   const unsigned FULL = 0xffffffffu;
   const int nx = A.nx, ny = A.ny;
   const int x = threadIdx.x & 31, r = 2 * (threadIdx.x >> 5);  // this lane's column, first row
   const int H = 2 * (blockDim.x >> 5), plane = 32 * H;
   float* const psi = f + kQ * plane;
-  // load: rows y0 - 8 .. , columns x0 - 8 .. x0 + 23, wrapped
+  // load: rows y0 - halo .. , the 32 columns from x0 - halo, wrapped
   {
-    int c = (x0 - kTileHalo + x) % nx;
+    int c = (x0 - halo + x) % nx;
     c = c < 0 ? c + nx : c;
-    int ya = (y0 - kTileHalo + r) % ny;
+    int ya = (y0 - halo + r) % ny;
     ya = ya < 0 ? ya + ny : ya;
     const int yb = ya + 1 == ny ? 0 : ya + 1;
 #pragma unroll
@@ -148,12 +151,12 @@ __device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps
           f[a * plane + rp + x] = P[a].y();
         }
       } else {
-        const int xg = x0 - kTileHalo + x, ya = y0 - kTileHalo + r;
-        // (after fewer than kTileSteps steps the halo holds results too: the
+        const int xg = x0 - halo + x, ya = y0 - halo + r;
+        // (after fewer than halo / 2 steps the halo holds results too: the
         // owned cells only)
-        const bool own = x >= kTileHalo && x < kTileHalo + kTileCols && xg < nx && r >= kTileHalo;
-        const bool sa = own && r < kTileHalo + rows && ya < ny;
-        const bool sb = own && r + 1 < kTileHalo + rows && ya + 1 < ny;
+        const bool own = x >= halo && x < 32 - halo && xg < nx && r >= halo;
+        const bool sa = own && r < halo + rows && ya < ny;
+        const bool sb = own && r + 1 < halo + rows && ya + 1 < ny;
         float* const dst = A.dst + size_t(ya) * nx + xg;
 #pragma unroll
         for (int a = 0; a < kQ; ++a) {
@@ -172,20 +175,20 @@ __device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps
 }
 
 template <int SCHEME>
-__device__ __noinline__ void run_tile_general(const StripArgs<StoreF32>& A, int steps, int x0,
-                                              int y0, int rows, float* f) {
-  run_tile<SCHEME, false>(A, steps, x0, y0, rows, f);
+__device__ __noinline__ void run_tile_general(const StripArgs<StoreF32>& A, int steps, int halo,
+                                              int x0, int y0, int rows, float* f) {
+  run_tile<SCHEME, false>(A, steps, halo, x0, y0, rows, f);
 }
 
 // CTA b: tile (b % A.n_strips, b / A.n_strips) of A.band_rows rows.
 template <int SCHEME>
 __global__ void __launch_bounds__(32 * kTileMaxWarps, 1)
-tile_steps_kernel(const __grid_constant__ StripArgs<StoreF32> A, int steps) {
+tile_steps_kernel(const __grid_constant__ StripArgs<StoreF32> A, int steps, int halo) {
   extern __shared__ __align__(16) float tile[];
-  const int x0 = int(blockIdx.x % A.n_strips) * kTileCols;
+  const int x0 = int(blockIdx.x % A.n_strips) * (32 - 2 * halo);
   const int y0 = int(blockIdx.x / A.n_strips) * A.band_rows;
-  if (!run_tile<SCHEME, true>(A, steps, x0, y0, A.band_rows, tile))
-    run_tile_general<SCHEME>(A, steps, x0, y0, A.band_rows, tile);
+  if (!run_tile<SCHEME, true>(A, steps, halo, x0, y0, A.band_rows, tile))
+    run_tile_general<SCHEME>(A, steps, halo, x0, y0, A.band_rows, tile);
 }
 
 }  // namespace lbm

@@ -59,10 +59,12 @@ def test_16_bit_storage(precision, nx, ny, scheme):
 
 
 # tiles: one cell to the largest lattice they cover in a wave, widths around
-# the 16 columns of a tile, odd and even rows per tile, a ragged last tile
+# the 16, 20 and 24 columns of a tile (of 4, 3 and 2 steps), odd and even rows
+# per tile, a ragged last tile
 @pytest.mark.parametrize("nx,ny", [
     (1, 1), (2, 9), (1, 152), (15, 33), (16, 16), (17, 5), (32, 32), (40, 36), (33, 47), (64, 64),
-    (100, 3), (3, 100), (2432, 1), (2417, 32), (120, 128), (270, 250), (48, 1600), (257, 101)])
+    (100, 3), (3, 100), (2432, 1), (2417, 32), (120, 128), (270, 250), (48, 1600), (257, 101),
+    (300, 300), (299, 331), (2441, 31), (3039, 36), (360, 360), (361, 341), (3647, 40), (1, 5000)])
 @pytest.mark.parametrize("steps", [2, 3, 4, 9])
 def test_tiles(nx, ny, steps):
     auto, ref = check(nx, ny, field(nx, ny, nx + ny), steps, lbm.IMPROVED)
@@ -70,14 +72,16 @@ def test_tiles(nx, ny, steps):
 
 
 @pytest.mark.parametrize("scheme", SCHEMES)
-@pytest.mark.parametrize("nx,ny", [(200, 190), (97, 60), (600, 300), (601, 301)])
+@pytest.mark.parametrize("nx,ny", [(200, 190), (97, 60), (310, 290), (340, 370), (600, 300),
+                                   (601, 301)])
 def test_schemes_and_step_graphs(scheme, nx, ny):
     # 35 steps: two replays of a graph of 16 and what is left
     auto, ref = check(nx, ny, field(nx, ny, 5), 35, scheme)
     assert np.array_equal(auto, ref)
 
 
-@pytest.mark.parametrize("nx,ny,precision", [(97, 60, lbm.FP32), (601, 301, lbm.FP32),
+@pytest.mark.parametrize("nx,ny,precision", [(97, 60, lbm.FP32), (310, 290, lbm.FP32),
+                                             (340, 370, lbm.FP32), (601, 301, lbm.FP32),
                                              (200, 190, lbm.BF16DEV), (60, 50, lbm.FP64)])
 def test_long_runs_in_step_graphs(nx, ny, precision):
     # graphs of 64 and of 16 steps from either buffer, and what is left

@@ -18,7 +18,7 @@ void geometry(int nx, int ny, int* out) {
 }
 void tiles(int nx, int ny, int* out) {
   const lbm::TileGeometry g = lbm::tile_geometry(0, 0, nx, ny, 0, 4.0, 152);
-  out[0] = g.n_cols; out[1] = g.rows; out[2] = g.grid; out[3] = g.threads;
+  out[0] = g.n_cols; out[1] = g.rows; out[2] = g.grid; out[3] = g.threads; out[4] = g.steps;
 }
 int applies(int variant, int precision, int nx, int ny, int rows, double b) {
   return lbm::two_step_applies(variant, precision, nx, ny, rows, b);
@@ -84,17 +84,24 @@ def test_bands_cover_the_rows_in_one_wave(H):
 
 def test_tiles_cover_the_lattice_in_one_wave(H):
     rng = np.random.default_rng(1)
-    for nx, ny in [(1, 1), (2432, 1), (2433, 1), (1, 4864), (1, 4865)] + \
+    def rows_of(steps, nx, ny):  # of the tiles when all start in one wave, else 0
+        cols = -(-nx // (32 - 4 * steps))
+        rows = -(-ny // (152 // cols)) if cols <= 152 else 48
+        return rows if rows + 4 * steps <= 48 else 0
+
+    for nx, ny in [(1, 1), (2432, 1), (2433, 1), (3648, 1), (3649, 1), (1, 4864), (1, 6080),
+                   (1, 6081), (2 ** 31 - 1, 1), (1, 2 ** 31 - 1)] + \
             [tuple(int(2 ** v) for v in rng.uniform(0, 12, 2)) for _ in range(300)]:
-        out = (ctypes.c_int * 4)()
+        out = (ctypes.c_int * 5)()
         H.tiles(nx, ny, out)
-        cols, rows, grid, threads = out
-        if rows == 0:  # too large for one wave of tiles of at most 32 rows
-            assert (nx + 15) // 16 > 152 or -(-ny // (152 // ((nx + 15) // 16))) > 32
+        cols, rows, grid, threads, steps = out
+        if rows == 0:
+            assert not any(rows_of(t, nx, ny) for t in (2, 3, 4))
             continue
-        assert cols == (nx + 15) // 16 and grid % cols == 0 and grid <= 152
+        assert 2 <= steps <= 4 and not any(rows_of(t, nx, ny) for t in range(steps + 1, 5))
+        assert cols == -(-nx // (32 - 4 * steps)) and grid % cols == 0 and grid <= 152
         assert grid // cols * rows >= ny > (grid // cols - 1) * rows
-        assert 2 * (threads // 32) >= rows + 16 and threads <= 768
+        assert 2 * (threads // 32) >= rows + 4 * steps and threads <= 768
 
 
 def test_which_lattices_take_two_steps(H):
