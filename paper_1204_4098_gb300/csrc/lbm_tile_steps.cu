@@ -10,7 +10,7 @@ namespace {
 template <int SCHEME>
 cudaError_t launch(const StripLaunch& L, int steps, int most, int grid, int threads,
                    cudaStream_t s) {
-  const int smem = kTilePlanes * 2 * threads * int(sizeof(float));
+  const int smem = (kQ * kTilePlane + 2 * threads) * int(sizeof(float));
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(
         tile_steps_kernel<SCHEME>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -23,10 +23,10 @@
 // again with the full forms.
 //
 // Measured, us per step in step graphs (improved scheme), best other kernel ->
-// this: 32^2 2.69 -> 1.06, 64^2 2.69 -> 1.10, 128^2 2.76 -> 1.26, 200^2 3.20 ->
-// 1.71, 256^2 3.46 -> 2.12 with four steps, 300^2 3.02 -> 2.41 with three, 360^2
-// 3.53 -> 3.08 with two.  A launch takes about 1.8 us + 0.24 us and 0.03 us per
-// active row for every step + 0.03 us per row loaded: at 64^2 a third of its 4.4
+// this: 32^2 2.69 -> 1.03, 64^2 2.69 -> 1.07, 128^2 2.76 -> 1.23, 200^2 3.20 ->
+// 1.68, 256^2 3.46 -> 2.09 with four steps, 300^2 3.02 -> 2.32 with three, 360^2
+// 3.53 -> 2.95 with two.  A launch takes about 1.8 us + 0.24 us and 0.03 us per
+// active row for every step + 0.03 us per row loaded: at 64^2 a third of its 4.3
 // us is the launch itself, the rest mostly one warp's serial row of arithmetic.
 // Tried without gain: one row per warp, programmatic dependent launch (64^2:
 // 1.34), five steps (64^2 1.09, 96^2 1.10 -> 1.19).
@@ -39,6 +39,11 @@ namespace lbm {
 
 // (kTileMaxWarps: lbm_geometry.h)
 constexpr int kTilePlanes = kQ + 1;  // populations and psi
+// floats between the planes in shared memory: those of the tallest tile, so
+// that every address of a cell is one of a few registers plus a constant (64^2
+// 1.10 -> 1.07 us per step, 200^2 1.71 -> 1.68, MRT 1.87 -> 1.80, against planes
+// of H rows)
+constexpr int kTilePlane = 2 * 32 * kTileMaxWarps;
 
 // psi of a pair whose elements may be out of use (kNormal: ok says whether
 // the used ones hold, see psi_normal).
@@ -53,8 +58,8 @@ __device__ __forceinline__ F2 psi_normal_masked(F2 rho, const Phys<float>& P, bo
 }
 
 // The tile whose first owned cell is (x0, y0), `rows` owned rows; f: shared
-// memory, kTilePlanes planes of H x 32 floats, H = 2 warps >= rows + 2 halo;
-// 1 <= steps <= halo / 2.
+// memory, kQ planes of populations and one of psi, H x 32 floats each, H = 2
+// warps >= rows + 2 halo; 1 <= steps <= halo / 2.
 // Returns (to every thread of the CTA) whether every check held.
 template <int SCHEME, bool kNormal>
 __device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps, int halo,
@@ -63,7 +68,8 @@ __device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps
   const unsigned FULL = 0xffffffffu;
   const int nx = A.nx, ny = A.ny;
   const int x = threadIdx.x & 31, r = 2 * (threadIdx.x >> 5);  // this lane's column, first row
-  const int H = 2 * (blockDim.x >> 5), plane = 32 * H;
+  const int H = 2 * (blockDim.x >> 5);
+  constexpr int plane = kTilePlane;
   float* const psi = f + kQ * plane;
   // load: rows y0 - halo .. , the 32 columns from x0 - halo, wrapped
   {
