@@ -102,9 +102,10 @@ MEASURED_TRAFFIC = {
     ("c6698b519fa83361", "fp32", 8192, "pair"): 4.6972e9,
     ("c6698b519fa83361", "fp32", 8192, "two_step"): 4.7692e9,
     # the same step kernels after changes to the read-back and initial-state
-    # kernels: 616.8 + 554.9 MB (one step), 630.8 + 559.3 (two), x4 cells
-    ("c97eb076ff990075", "fp32", 8192, "pair"): 4.6870e9,
-    ("c97eb076ff990075", "fp32", 8192, "two_step"): 4.7602e9,
+    # kernels and to FP64's divisions: 616.8 + 554.8 MB (one step), 630.7 +
+    # 559.2 (two), x4 cells
+    ("cd76c253203ad670", "fp32", 8192, "pair"): 4.6865e9,
+    ("cd76c253203ad670", "fp32", 8192, "two_step"): 4.7595e9,
 }
 
 

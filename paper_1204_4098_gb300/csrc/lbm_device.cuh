@@ -136,14 +136,7 @@ struct Phys {
 // approximations (MUFU.RCP / MUFU.RSQ, ~1 ulp), which are deterministic, so
 // the owner and the halo copy of psi stay bit-identical.
 __device__ __forceinline__ float fast_div(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fast_div(double a, double b) { return __ddiv_rn(a, b); }
 __device__ __forceinline__ float fast_sqrt_pos(float a) { return a * rsqrtf(a); }
-__device__ __forceinline__ double fast_sqrt_pos(double a) { return __dsqrt_rn(a); }
-
-template <class C>
-__device__ __forceinline__ Pair<C> fast_div(Pair<C> a, Pair<C> b) {
-  return Pair<C>(fast_div(a.x(), b.x()), fast_div(a.y(), b.y()));
-}
 
 // The same reciprocal and root for operands known to be normal, with normal
 // results: without the handling of subnormal and huge operands around it,
@@ -159,15 +152,65 @@ __device__ __forceinline__ float rsqrt_normal(float a) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
   return r;
 }
-// 1 / b, the value of fast_div(1, b) (FP64: one correctly rounded reciprocal
-// instead of a division, 3 fewer FP64 instructions)
+
+// FP64 value of a normal FP32 number and back (positive, cut to 24 bits), by
+// integer operations on the bits: FP64 conversions share the 2 lanes a clock
+// and SM of the FP64 pipe.
+__device__ __forceinline__ double widen_normal(float v) {
+  const unsigned u = __float_as_uint(v);
+  return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                          int(u << 29));
+}
+__device__ __forceinline__ float narrow_normal(double v) {
+  return __uint_as_float(__funnelshift_l(unsigned(__double2loint(v)),
+                                         unsigned(__double2hiint(v)) - 0x38000000u, 3));
+}
+
+// FP64 quotient, reciprocal and root of positive numbers from 2^-100 to 2^100,
+// started from the FP32 approximations, which run beside the FP64 pipe: the
+// reciprocal i of the cut divisor gives e = 1 - b i, |e| < 2^-22, and R = i (1 +
+// e), 1 / b up to e^2; a quotient, a reciprocal and a root then get their
+// remainder's correction (Markstein, IBM J. Res. Dev. 34, 1990; Goldschmidt's
+// root).  Before the last rounding the values are good to 2^-85 or better: on
+// 1.9e10 random operands all three gave the IEEE operations' bits (with
+// mantissas of 28 leading ones, whose reciprocals are nearly ties, one
+// reciprocal in 10^5 was the neighbour).  5, 4 and 6 FP64 operations take 5 % off the FP64 step (SC 512^2 72.6 -> 69.3 us, 1024^2 272 ->
+// 258, improved 337 -> 317).  Other operands take the IEEE operations.
+__device__ __forceinline__ bool middling(double v) {
+  constexpr unsigned kLow = (1023u - 100u) << 20, kHigh = (1023u + 100u) << 20;
+  return unsigned(__double2hiint(v)) - kLow < kHigh - kLow;
+}
+__device__ __forceinline__ double fast_div(double a, double b) {
+  if (!(middling(a) && middling(b))) return __ddiv_rn(a, b);
+  const double i = widen_normal(rcp_normal(narrow_normal(b)));
+  const double R = __fma_rn(i, __fma_rn(-b, i, 1.0), i), q = __dmul_rn(a, R);
+  return __fma_rn(__fma_rn(-q, b, a), R, q);
+}
+__device__ __forceinline__ double fast_sqrt_pos(double a) {
+  if (!middling(a)) return __dsqrt_rn(a);
+  const float y = rsqrt_normal(narrow_normal(a));
+  const double g0 = __dmul_rn(a, widen_normal(y)), h0 = widen_normal(0.5f * y);
+  const double r = __fma_rn(-g0, h0, 0.5);
+  const double g = __fma_rn(g0, r, g0), h = __fma_rn(h0, r, h0);
+  return __fma_rn(__fma_rn(-g, g, a), h, g);
+}
+template <class C>
+__device__ __forceinline__ Pair<C> fast_div(Pair<C> a, Pair<C> b) {
+  return Pair<C>(fast_div(a.x(), b.x()), fast_div(a.y(), b.y()));
+}
+// 1 / b, the value of fast_div(1, b)
 template <class V>
 __device__ __forceinline__ V recip(V b) { return fast_div(V(1), b); }
 template <>
-__device__ __forceinline__ double recip(double b) { return __drcp_rn(b); }
+__device__ __forceinline__ double recip(double b) {
+  if (!middling(b)) return __drcp_rn(b);
+  const double i = widen_normal(rcp_normal(narrow_normal(b)));
+  const double R = __fma_rn(i, __fma_rn(-b, i, 1.0), i);
+  return __fma_rn(R, __fma_rn(-b, R, 1.0), R);
+}
 template <>
 __device__ __forceinline__ Pair<double> recip(Pair<double> b) {
-  return Pair<double>(__drcp_rn(b.x()), __drcp_rn(b.y()));
+  return Pair<double>(recip(b.x()), recip(b.y()));
 }
 
 // a / b; kNormal: b and 1 / b are normal numbers (FP32)
@@ -185,14 +228,6 @@ template <bool kNormal, class V, class C>
 __device__ __forceinline__ V quot_one(V b, C) {  // 1 / b
   if constexpr (kNormal) return quot<true>(V(C(1)), b);
   else return recip(b);
-}
-
-// FP64 value of an FP32 number, from its bits (integer operations: FP64
-// conversions share the 2 lanes a clock and SM of the FP64 pipe).
-__device__ __forceinline__ double widen_normal(float v) {
-  const unsigned u = __float_as_uint(v);
-  return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
-                          int(u << 29));
 }
 
 // Density and actual velocity (j + F / 2) / rho of a cell as FP64 values, the

@@ -4,6 +4,7 @@ in FP64 on the host."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_1204_4098_gb300 import lbm
 
 pytestmark = pytest.mark.gpu
@@ -87,3 +88,22 @@ def test_velocities_are_the_rounded_quotients(nx, scale):
         want = [rho.astype(np.float64)] + [j.astype(np.float64) / rho for j in (jx, jy)]
     for got, w in zip(out, want):
         assert np.array_equal(got, w, equal_nan=True)
+
+
+@pytest.mark.parametrize("scale", [1e-32, 1e-30, 0.1])  # 2^-100 = 7.9e-31: below it, above it
+@pytest.mark.parametrize("scheme", [lbm.SC, lbm.IMPROVED, lbm.MRT])
+def test_fp64_steps_at_densities_of_any_scale(scheme, scale):
+    nx, ny = 37, 21
+    rho = scale * np.random.default_rng(3).uniform(0.95, 1.05, (ny, nx))
+    with lbm.Lattice(nx, ny, 0.85, precision=lbm.FP64) as lat:
+        lat.init_density(rho)
+        lat.step(2, scheme, 0.9, 0.1)
+        got = lat.observe()
+    ref = oracle.Lattice(nx, ny, 0.85)
+    ref.init_density(rho)
+    rc, _ = ref.step(2, scheme, 0.9, 0.1)
+    assert rc == 0
+    # two steps of ~100 roundings each, errors grown tenfold at most by differences
+    tol = 2 * 100 * 10 * 2.0 ** -53
+    for g, w, unit in zip(got, ref.observe(), (scale, 1.0, 1.0)):
+        assert np.max(np.abs(g - w)) <= tol * unit
