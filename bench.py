@@ -106,6 +106,10 @@ MEASURED_TRAFFIC = {
     # 559.2 (two), x4 cells
     ("cd76c253203ad670", "fp32", 8192, "pair"): 4.6865e9,
     ("cd76c253203ad670", "fp32", 8192, "two_step"): 4.7595e9,
+    # the two-step kernel with the arriving row read first and predicated row
+    # copies: 616.8 + 554.9 MB (one step), 630.7 + 558.8 (two), x4 cells
+    ("c9ce772ed26597b5", "fp32", 8192, "pair"): 4.6868e9,
+    ("c9ce772ed26597b5", "fp32", 8192, "two_step"): 4.7581e9,
 }
 
 

@@ -246,22 +246,27 @@ batch_balanced_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
 // of a 32-column lattice's lanes idle).  The lattices are split into several
 // chains of launches that run side by side (two_step_graph).  Measured, us
 // per step, best work-list or balanced mode -> this: 96 slabs of 32 columns
-// 31.3 -> 9.2 (117k MLUPS), 600 of them 148 -> 38.4, 48 mixed slabs (4.7 M cells)
-// 79 -> 39.1 (121k MLUPS), 128 mixed slabs 179 -> 98, 6 slabs 17.6 -> 7.9.  Bound
+// 31.3 -> 9.1 (118k MLUPS), 600 of them 148 -> 37.8, 48 mixed slabs (4.7 M cells)
+// 79 -> 38.8 (122k MLUPS), 128 mixed slabs 179 -> 97.8, 6 slabs 17.6 -> 7.8.  Bound
 // by the latency and issue of its instructions, like two_step_kernel.
 template <int SCHEME, int LAYOUT>
 __device__ __noinline__ void batch_two_general(const StripArgs<StoreF32>& A, int strip, int lane,
                                                TwoSmem<StoreF32>& sm) {
   if constexpr (SCHEME == kNoForce)
-    if (strip_run_two<StoreF32, kNoForce, LAYOUT, true>(A, strip, 0, lane, sm)) return;
-  strip_run_two<StoreF32, SCHEME, LAYOUT, false>(A, strip, 0, lane, sm);
+    if (strip_run_two<StoreF32, kNoForce, LAYOUT, true, 0>(A, strip, 0, lane, sm)) return;
+  strip_run_two<StoreF32, SCHEME, LAYOUT, false, 0>(A, strip, 0, lane, sm);
 }
 
 template <int LAYOUT>
 __device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int scheme, int strip,
                                                int lane, TwoSmem<StoreF32>& sm,
                                                StripArgs<StoreF32>& shared) {
-  if (scheme != kNoForce && strip_run_two<StoreF32, kBlend, LAYOUT, true>(A, strip, 0, lane, sm))
+  // (two_form's choices spill here; even slabs 35.4 -> 34.9 us per step, odd 39.7
+  // -> 39.5, slabs of 32 columns 9.23 -> 9.13 against neither)
+  constexpr int kForm =
+      LAYOUT == kFlatEven ? kFetchIf : (LAYOUT == kRing ? kEarlyRow : kStoreIf | kFetchIf);
+  if (scheme != kNoForce &&
+      strip_run_two<StoreF32, kBlend, LAYOUT, true, kForm>(A, strip, 0, lane, sm))
     return;
   if (lane == 0) shared = A;
   __syncwarp();
@@ -274,7 +279,7 @@ __device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int
 // (One kernel per layout: with the bodies of all layouts in one, registers
 // spill and mixed sweeps lose 6-12 %.)
 template <int LAYOUT>
-__global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
+__global__ void __launch_bounds__(kTwoThreads, kTwoManyCtas)
 batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict__ items,
                       const int2* __restrict__ chain, const float* src, float* dst,
                       unsigned* inst_status) {

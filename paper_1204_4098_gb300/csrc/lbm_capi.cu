@@ -145,14 +145,14 @@ cudaError_t strip_tma_occupancy(int precision, int scheme, int* b) {
   if (precision != kFP32) return cudaErrorNotSupported;
   return strip_tma_occupancy_f32(scheme, b);
 }
-cudaError_t two_step_launch_f32(int, const StripLaunch&, int, cudaStream_t);
-cudaError_t two_step_launch_bf16(int, const StripLaunch&, int, cudaStream_t);
-cudaError_t two_step_launch_f16(int, const StripLaunch&, int, cudaStream_t);
-cudaError_t two_step_launch(int precision, int scheme, const StripLaunch& L, int grid,
+cudaError_t two_step_launch_f32(int, const StripLaunch&, int, bool, cudaStream_t);
+cudaError_t two_step_launch_bf16(int, const StripLaunch&, int, bool, cudaStream_t);
+cudaError_t two_step_launch_f16(int, const StripLaunch&, int, bool, cudaStream_t);
+cudaError_t two_step_launch(int precision, int scheme, const StripLaunch& L, int grid, bool few,
                             cudaStream_t s) {
-  if (precision == kFP32) return two_step_launch_f32(scheme, L, grid, s);
-  if (precision == kBF16Dev) return two_step_launch_bf16(scheme, L, grid, s);
-  if (precision == kFP16Dev) return two_step_launch_f16(scheme, L, grid, s);
+  if (precision == kFP32) return two_step_launch_f32(scheme, L, grid, few, s);
+  if (precision == kBF16Dev) return two_step_launch_bf16(scheme, L, grid, few, s);
+  if (precision == kFP16Dev) return two_step_launch_f16(scheme, L, grid, few, s);
   return cudaErrorNotSupported;
 }
 cudaError_t set_state_launch(int precision, void* dst, float* rd, int nx, int ny, int pitch,
@@ -470,7 +470,8 @@ cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t
       e = plan.kind == kTileRuns
               ? tile_steps_launch(scheme, plan.many, steps, plan.tile_steps, plan.many_grid,
                                   plan.many_threads, stream)
-              : two_step_launch(c->p.precision, scheme, plan.many, plan.many_grid, stream);
+              : two_step_launch(c->p.precision, scheme, plan.many, plan.many_grid,
+                                plan.many_grid <= c->sm_count * kTwoStepFewWarps, stream);
       if (e == cudaSuccess) c->cur = d;
     }
     if (e != cudaSuccess) return e;

@@ -113,6 +113,7 @@ inline StripGeometry fp64_geometry(int nx, int ny, int sm_count, int warps_per_c
 // ---------------------------------------------------------------------------
 constexpr int kTwoStepCols = 56;   // columns of a strip
 constexpr int kTwoStepWarps = 12;  // resident warps per SM
+constexpr int kTwoStepFewWarps = 8;  // of launches that have no use for more
 
 // Whether steps of a whole nx x ny lattice may go two per launch: FP32, or
 // 16-bit storage with even nx (its columns are copied in pairs), AUTO variant
@@ -134,14 +135,16 @@ inline bool two_step_applies(int requested, int precision, int nx, int ny,
 // Strips of 56 columns and the band height that ends first.  A band of n rows
 // costs about n + 4 iterations; with 4, 8 or 12 warps per SM (1, 2 or 3 per
 // scheduler; numbers between leave one scheduler with more than the others
-// and end no earlier) an iteration takes 0.60, 0.92 and 1.30 us (improved
-// scheme), so short bands of many warps pay only while the rows dominate.
-// us per step with 4 / 8 / 12 warps: 512^2 4.78 / 4.99 / 5.37, 768^2 7.30 /
-// 6.79 / 7.30, 1024^2 11.1 / 9.87 / 10.5, 2048^2 38.9 / 31.3 / 30.5.
+// and end no earlier) an iteration takes 0.58, 0.89 and 1.285 us (improved
+// scheme, the first two in the kernel for few CTAs), so short bands of many
+// warps pay only while the rows dominate.  us per step with 4 / 8 / 12 warps,
+// one kernel: 512^2 4.78 / 4.99 / 5.37, 768^2 7.30 / 6.79 / 7.30, 1024^2 11.1 /
+// 9.87 / 10.5, 2048^2 38.9 / 31.3 / 30.5; now 512^2 4.30, 768^2 6.37, 1024^2 9.37,
+// 2048^2 30.0.
 inline StripGeometry two_step_geometry(int nx, int ny, int sm_count) {
   StripGeometry g;
   g.n_strips = (nx + kTwoStepCols - 1) / kTwoStepCols;
-  const double cost[3] = {0.60, 0.92, 1.30};
+  const double cost[3] = {0.58, 0.89, 1.285};
   double best = 0.0;
   g.band_rows = ny;
   for (int k = 0; k < 3; ++k) {
@@ -179,7 +182,8 @@ struct TileGeometry {
 // (128^2: 1.41 us per step with 152 tiles of 7 rows, 1.66 with 72 of 15; a
 // second wave only ties with two-step launches: 300^2 with four steps 3.02).
 // Fewer steps leave more columns and rows to a tile, so a lattice takes the
-// most steps that fit, us per step with 4 / 3 / 2 and of the two-step strips:
+// most steps that fit, us per step with 4 / 3 / 2 and of the two-step strips
+// (300^2):
 // 64^2 1.10 / 1.29 / 1.42, 128^2 1.26 / 1.42 / 1.55, 200^2 1.71 / 1.72 / 1.93,
 // 256^2 2.12 / 2.06 / 2.12, 300^2 - / 2.40 / 2.57 / 3.02.  (Five steps gain 3 %
 // at 16^2 and 1 % at 64^2 and lose from 96^2 on.)  The same requirements on

@@ -59,7 +59,9 @@ cudaError_t strip_tma_launch(int precision, int scheme, const StripLaunch& L, in
 cudaError_t strip_tma_occupancy(int precision, int scheme, int* blocks_per_sm);
 // Two steps from L.src to L.dst in one launch (FP32, or 16-bit storage with
 // even nx; at most kTwoStepMaxCells cells; L as two_step_geometry sets it).
-cudaError_t two_step_launch(int precision, int scheme, const StripLaunch& L, int grid, cudaStream_t s);
+// few: at most kTwoStepFewWarps CTAs per SM.
+cudaError_t two_step_launch(int precision, int scheme, const StripLaunch& L, int grid, bool few,
+                            cudaStream_t s);
 // 1 .. `most` steps from L.src to L.dst in one launch (FP32 storage; most,
 // grid, threads, L.n_strips and L.band_rows as tile_geometry gives them).
 cudaError_t tile_steps_launch(int scheme, const StripLaunch& L, int steps, int most, int grid,

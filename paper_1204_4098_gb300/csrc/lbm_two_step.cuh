@@ -34,16 +34,19 @@
 //
 // Measured on the way (improved scheme, 4096^2, us per step; one-step kernel
 // 197.5): first version 141; unrolled by two 134; bare divisions and roots
-// 128; no branches 123; step 2 one row behind 118; one warp per CTA 114
-// (147k MLUPS, DRAM at 0.77 of the measured copy bandwidth, FMA pipes 60 %
-// busy, 158 registers, 12 warps per SM).  13 to 16 warps per SM (128
-// registers, spilling) 119-122; rows of step 1 kept in registers 141 (spills).
+// 128; no branches 123; step 2 one row behind 118; one warp per CTA 114; the
+// arriving row read first and predicated copies 112.2 (149k MLUPS, DRAM at
+// 0.78 of the measured copy bandwidth, FMA pipes 60 % busy, 12 warps per SM).
+// 13 to 16 warps per SM (128 registers, spilling) 119-122; rows of step 1 kept
+// in registers 141 (spills).  Small launches, whose SMs get 4 or 8 warps, are
+// latency bound and take a kernel with 255 registers and more overlap
+// (two_form): 512^2 4.65 -> 4.30, 1024^2 9.75 -> 9.37.
 //
 // 16-bit storage gains from the instructions that two separate steps repeat
 // (the row copies, the halo's psi) and from the bare divisions: it was bound
 // by issue, not by memory (BF16, us per step, one-step -> two-step: 4096^2 186 ->
-// 133, 2048^2 51.1 -> 37.0, 1024^2 16.6 -> 12.4, 512^2 7.4 -> 5.8, 200^2 4.2 ->
-// 3.5; FP16 the same).
+// 129, 2048^2 51.1 -> 34.4, 1024^2 16.6 -> 10.8, 512^2 7.4 -> 5.1, 256^2 4.2 ->
+// 3.4; FP16 the same).
 #pragma once
 
 #include "lbm_geometry.h"
@@ -56,7 +59,9 @@ constexpr int kTwoCols = kTwoStepCols;   // columns a strip owns
 static_assert(kTwoCols + 2 * kTwoHalo == 64, "a warp loads two columns per lane");
 constexpr int kTwoStages = 3;                // rows in shared memory: one read, two in flight
 constexpr int kTwoThreads = 32;              // one warp per CTA
-constexpr int kTwoMinBlocks = 12;            // CTAs per SM (168 registers at most)
+// CTAs per SM: 12 (168 registers at most), or for launches that bring no more
+// than 8 to an SM, 8 (255 registers)
+constexpr int kTwoManyCtas = kTwoStepWarps, kTwoFewCtas = kTwoStepFewWarps;
 
 // Shared memory of a warp, lane-major.  A fetched row: the 9 planes' pairs, for
 // deviation storage also the density pair of the row after the pulled one (the
@@ -104,6 +109,48 @@ __device__ __forceinline__ F2 psi_normal(F2 rho, const Phys<float>& P, bool& ok)
   return F2(mul_rn(arg.x(), rsqrt_normal(arg.x())), mul_rn(arg.y(), rsqrt_normal(arg.y())));
 }
 
+// Forms of the march, the order and the branches the compiler gets to schedule
+// an iteration in; the values are the same.  kEarlyRow: the row that arrives is
+// taken from shared memory before step 2's work, not after it; kStoreIf,
+// kFetchIf: the stores and the row copies are predicated instead of branched
+// around, so that step 2 and step 1 share a block of instructions.  More
+// overlap takes registers, so what pays differs, us per step with neither / the
+// form taken: even nx, 12 CTAs per SM: 512^2 4.65 / 4.49, 1024^2 9.71 / 9.61,
+// 4096^2 113.1 / 112.3, MRT 2048^2 32.6 / 31.6; 8 CTAs per SM: 512^2 4.62 / 4.27,
+// 1024^2 9.72 / 9.38, BF16 1024^2 10.90 / 10.71; odd nx: 1023x1025 11.31 / 10.97
+// with 8.  All three with 12 CTAs spill (4096^2 114.0).
+enum TwoForm { kEarlyRow = 1, kStoreIf = 2, kFetchIf = 4 };
+__host__ __device__ constexpr int two_form(bool dev, int scheme, bool odd, int ctas) {
+  if (ctas == kTwoFewCtas)
+    return dev ? kEarlyRow | kStoreIf | kFetchIf
+               : (scheme == kMRT ? kEarlyRow | kFetchIf : kEarlyRow | kStoreIf);
+  return odd ? kStoreIf : kEarlyRow | kFetchIf;
+}
+
+__device__ __forceinline__ void store_if(bool p, void* at, float v) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.global.f32 [%0], %1;\n}" ::"l"(at),
+               "f"(v), "r"(unsigned(p)));
+}
+__device__ __forceinline__ void store_if(bool p, void* at, float2 v) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q st.global.v2.f32 [%0], {%1, %2};\n}" ::"l"(at),
+               "f"(v.x), "f"(v.y), "r"(unsigned(p)));
+}
+template <class V>
+__device__ __forceinline__ void store_if(bool p, void* at, V v) {  // 32 bits
+  static_assert(sizeof(V) == 4, "");
+  unsigned u;
+  __builtin_memcpy(&u, &v, 4);
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.global.b32 [%0], %1;\n}" ::"l"(at),
+               "r"(u), "r"(unsigned(p)));
+}
+// (no bytes are read where `p` does not hold; the destination gets zeros)
+template <int N>
+__device__ __forceinline__ void cp_async_if(bool p, void* smem, const void* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(
+                   unsigned(__cvta_generic_to_shared(smem))),
+               "l"(g), "n"(N), "r"(p ? N : 0));
+}
+
 // Row layouts.
 //  kFlatEven  even nx = pitch: a lane's two columns are one aligned pair;
 //  kFlatOdd   odd nx = pitch: columns copied and stored one by one;
@@ -120,7 +167,7 @@ enum TwoLayout { kFlatEven, kFlatOdd, kAnyWidth, kRing };
 // kNormal = false.  Deviation storage (kFlatEven only) rounds the populations
 // between the two steps to what the one-step kernel would store and read
 // back, in registers.
-template <class S, int SCHEME, int LAYOUT, bool kNormal>
+template <class S, int SCHEME, int LAYOUT, bool kNormal, int FORM>
 __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, int band, int lane,
                                               TwoSmem<S>& sm) {
   using T = typename S::T;
@@ -180,7 +227,11 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
   int nrow = wrap_row(y0 - 2);  // the row after the next pulled one
   unsigned om = (unsigned(wrap_row(y0 - 4)) * pitch + unsigned(ca)) * kBytes;
   unsigned oz = (unsigned(wrap_row(y0 - 3)) * pitch + unsigned(ca)) * kBytes;
-  auto fetch = [&](TwoRow<S>& R) {
+  auto copy = [](bool p, void* to, const char* from, auto bytes) {
+    if constexpr ((FORM & kFetchIf) != 0) cp_async_if<bytes()>(p, to, from);
+    else cp_async<bytes()>(to, from);
+  };
+  auto fetch = [&](TwoRow<S>& R, bool p) {
     const unsigned op = (unsigned(nrow) * pitch + unsigned(ca)) * kBytes;
     auto source = [&](int a) {
       const unsigned o = ey_of(a) == 0 ? oz : (ey_of(a) == 1 ? om : op);
@@ -189,14 +240,15 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
 #pragma unroll
     for (int a = 0; a < kQ; ++a) {
       if constexpr (LAYOUT == kFlatOdd || LAYOUT == kAnyWidth) {
-        cp_async<4>(&R.d[a][lane].x, source(a));
-        cp_async<4>(&R.d[a][lane].y, source(a) + 4 * (cb - ca));
+        copy(p, &R.d[a][lane].x, source(a), std::integral_constant<int, 4>());
+        copy(p, &R.d[a][lane].y, source(a) + 4 * (cb - ca), std::integral_constant<int, 4>());
       } else {
-        cp_async<sizeof(V)>(&R.d[a][lane], source(a));
+        copy(p, &R.d[a][lane], source(a), std::integral_constant<int, int(sizeof(V))>());
       }
     }
     if constexpr (S::kDev)
-      cp_async<8>(&R.rr[lane], reinterpret_cast<const char*>(A.rho_src) + 2u * op);
+      copy(p, &R.rr[lane], reinterpret_cast<const char*>(A.rho_src) + 2u * op,
+           std::integral_constant<int, 8>());
     cp_async_commit();
     om = oz;
     oz = op;
@@ -291,7 +343,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
 
   constexpr int D = kTwoStages - 1;  // rows in flight
 #pragma unroll
-  for (int k = 0; k < D; ++k) fetch(st[k]);  // n_rows >= 7
+  for (int k = 0; k < D; ++k) fetch(st[k], true);  // n_rows >= 7
 
   // In iteration k the pulled row r = y0 - 3 + k arrives.  Step 1 has its
   // pulled row r - 1 (P0, rho0) and the psi of rows r - 2 (m1) and r - 1 (z1).
@@ -325,36 +377,48 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
 #pragma unroll
     for (int a = 0; a < kQ; ++a) Q0[a] = F2(sm.q[k & 1][a][lane]);
     collide<SCHEME, kNormal>(Q0, qrhoA, Gx, Gy, z2.c, A.P);
-    if (store_a && (LAYOUT != kRing || k - 7 < y1 - y0)) {
+    const bool store = store_a && (LAYOUT != kRing || k - 7 < y1 - y0);
+    auto put = [&](auto to) {
       V v[kQ];
       const F2 res = encode(Q0, qrhoA, v);
-      if constexpr (S::kDev)
-        *reinterpret_cast<float2*>(reinterpret_cast<char*>(A.rho_dst) + 2u * out) = res.v;
+      if constexpr (S::kDev) to(store, reinterpret_cast<char*>(A.rho_dst) + 2u * out, res.v);
 #pragma unroll
       for (int a = 0; a < kQ; ++a) {
-        T* const at = reinterpret_cast<T*>(reinterpret_cast<char*>(A.dst + a * A.plane) + out);
+        char* const at = reinterpret_cast<char*>(A.dst + a * A.plane) + out;
         if constexpr (S::kDev) {
-          *reinterpret_cast<V*>(at) = v[a];
+          to(store, at, v[a]);
         } else if constexpr (LAYOUT == kFlatOdd) {
-          at[0] = Q0[a].x();
-          if (store_b) at[1] = Q0[a].y();
+          to(store, at, Q0[a].x());
+          to(store && store_b, at + kBytes, Q0[a].y());
         } else {
-          *reinterpret_cast<float2*>(at) = Q0[a].v;
+          to(store, at, Q0[a].v);
         }
       }
+    };
+    if constexpr ((FORM & kStoreIf) != 0) {
+      put([](bool p, void* at, auto v) { store_if(p, at, v); });
+    } else if (store) {
+      put([](bool p, void* at, auto v) {
+        if (p) *reinterpret_cast<decltype(v)*>(at) = v;
+      });
     }
     out += pitch * kBytes;
   };
-  // Step 1 of iteration k: row r arrives, and (`full`) row r - 1 is advanced,
-  // which completes step 2's pulled row r - 2.
-  auto step1 = [&](int k, bool full) {
+  // Step 1 of iteration k: row r arrives ...
+  F2 P1[kQ];
+  auto arrive = [&](int k) {
     cp_async_wait<D - 1>();
-    F2 P1[kQ];
     assemble(st[sg], P1);
     sg = sg == kTwoStages - 1 ? 0 : sg + 1;
-    if (k + D < n_rows) fetch(st[sf]);  // into the stage read in iteration k - 1
-    else cp_async_commit();             // an empty group keeps the count per row
+    // (into the stage read in iteration k - 1; an empty group keeps the count)
+    if constexpr ((FORM & kFetchIf) != 0) fetch(st[sf], k + D < n_rows);
+    else if (k + D < n_rows) fetch(st[sf], true);
+    else cp_async_commit();
     sf = sf == kTwoStages - 1 ? 0 : sf + 1;
+  };
+  // ... and (`full`) row r - 1 is advanced, which completes step 2's pulled row
+  // r - 2.
+  auto step1 = [&](int k, bool full) {
     const F2 rho1 = rho_of(P1);
     PsiRow p1 = none;
     if constexpr (kNeedPsi) p1 = psi_row(rho1, valid1);
@@ -407,13 +471,16 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
   // y0 - 3, its collision from row y0 - 2, psi of step 2 from row y0 - 1.
 #pragma unroll 1
   for (int k = 0; k < 7 && go; ++k) {
+    arrive(k);
     if (k >= 5) step2_psi();
     step1(k, k >= 2);
   }
 #pragma unroll 2
   for (int k = 7; k < n_rows && go; ++k) {
+    if constexpr ((FORM & kEarlyRow) != 0) arrive(k);
     step2_psi();
     step2_row(k);
+    if constexpr ((FORM & kEarlyRow) == 0) arrive(k);
     step1(k, true);
   }
   if (go) {
@@ -431,17 +498,18 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
 template <class S, int SCHEME, int LAYOUT>
 __device__ __noinline__ void strip_run_two_general(const StripArgs<S>& A, int strip, int band,
                                                    int lane, TwoSmem<S>& sm) {
-  strip_run_two<S, SCHEME, LAYOUT, false>(A, strip, band, lane, sm);
+  strip_run_two<S, SCHEME, LAYOUT, false, 0>(A, strip, band, lane, sm);
 }
 
-template <class S, int SCHEME, int LAYOUT>
-__global__ void __launch_bounds__(kTwoThreads, kTwoMinBlocks)
+template <class S, int SCHEME, int LAYOUT, int CTAS>
+__global__ void __launch_bounds__(kTwoThreads, CTAS)
 two_step_kernel(const __grid_constant__ StripArgs<S> A) {
   __shared__ TwoSmem<S> sm;
+  constexpr int kForm = two_form(S::kDev, SCHEME, LAYOUT == kFlatOdd, CTAS);
   const int lane = threadIdx.x;
   const int strip = blockIdx.x % A.n_strips;  // strips of kTwoCols columns
   const int band = blockIdx.x / A.n_strips;
-  if (!strip_run_two<S, SCHEME, LAYOUT, true>(A, strip, band, lane, sm))
+  if (!strip_run_two<S, SCHEME, LAYOUT, true, kForm>(A, strip, band, lane, sm))
     strip_run_two_general<S, SCHEME, LAYOUT>(A, strip, band, lane, sm);
 }
 

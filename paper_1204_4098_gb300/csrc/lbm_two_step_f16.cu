@@ -3,8 +3,9 @@
 
 namespace lbm {
 
-cudaError_t two_step_launch_f16(int scheme, const StripLaunch& L, int grid, cudaStream_t s) {
-  return two_step_launch_t<StoreF16, kFlatEven>(scheme, L, grid, s);
+cudaError_t two_step_launch_f16(int scheme, const StripLaunch& L, int grid, bool few,
+                                cudaStream_t s) {
+  return two_step_launch_t<StoreF16, kFlatEven>(scheme, L, grid, few, s);
 }
 
 }  // namespace lbm

@@ -47,6 +47,15 @@ def test_sizes(nx, ny, steps):
     assert np.array_equal(auto, ref)
 
 
+# both kernels of each layout: launches of up to 8 warps per SM and of more
+@pytest.mark.parametrize("nx,ny", [(900, 800), (901, 800), (2000, 1900), (2001, 1900)])
+@pytest.mark.parametrize("scheme,precision", [(s, lbm.FP32) for s in SCHEMES] +
+                         [(lbm.IMPROVED, lbm.BF16DEV), (lbm.MRT, lbm.FP16DEV)])
+def test_few_and_many_warps(nx, ny, scheme, precision):
+    auto, ref = check(nx, ny, field(nx, ny, 11), 3, scheme, precision)
+    assert np.array_equal(auto, ref)
+
+
 # 16-bit storage: the rounding between the two steps of a launch, every scheme
 @pytest.mark.parametrize("precision", [lbm.BF16DEV, lbm.FP16DEV])
 @pytest.mark.parametrize("nx,ny,scheme", [(200, 190, s) for s in SCHEMES] + [
