@@ -57,7 +57,7 @@ constexpr int kCols = kHid / kClusterCtas;             // hidden columns a CTA o
 constexpr int kPad = kHid + 4;  // padded row: 16-byte aligned, rows 4 banks apart
 
 struct TrainSmem {
-  float W1[kIn * kHid], b1[kHid], W2[kHid * kPad], b2[kHid], W3[kHid * kOut], b3[kOut + 1];
+  float W1[kIn * kHid], b1[kHid], W2[kHid * kPad], b2[kHid], W3t[kOut * kHid], b3[kOut + 1];
   float H1[kMaxBatch * kPad];       // every sample
   float H2[kCtaSamples * kPad];     // this CTA's samples
   float DZ2[kCtaSamples * kPad];
@@ -81,7 +81,7 @@ __device__ __forceinline__ int weight_slot(int p) {
   if (p < kOffW2) return ob1 + (p - kOffB1);
   if (p < kOffB2) return o2 + (p - kOffW2) / kHid * kPad + (p - kOffW2) % kHid;
   if (p < kOffW3) return ob2 + (p - kOffB2);
-  if (p < kOffB3) return o3 + (p - kOffW3);
+  if (p < kOffB3) return o3 + (p - kOffW3) % kOut * kHid + (p - kOffW3) / kOut;  // transposed
   return ob3 + (p - kOffB3);
 }
 
@@ -129,27 +129,37 @@ mlp_train_kernel(float* params, float* adam_m, float* adam_v, const float* __res
   const int steps = mode == 0 ? epochs * per_epoch : 1;
 
   // a minibatch's rows travel in registers (thread b: sample b) from the end
-  // of the minibatch before
+  // of the minibatch before, their indices from one minibatch earlier still
+  // (a row's address waits for its index)
   float4 xin = make_float4(0.f, 0.f, 0.f, 0.f);
   float tin[kOut] = {0.f, 0.f, 0.f};
+  int next = 0;  // this thread's sample of the minibatch that load_rows takes
+  auto load_index = [&](int st) {
+    if (mode != 0 || st >= steps || tid >= kMaxBatch) return;
+    const int e = st / per_epoch, k0 = (st % per_epoch) * batch;
+    if (tid < min(batch, n - k0)) next = order[size_t(e) * n + k0 + tid];
+  };
   auto load_rows = [&](int st) {
     if (st >= steps || tid >= kMaxBatch) return;
-    const int e = st / per_epoch, k0 = (st % per_epoch) * batch;
+    const int k0 = (st % per_epoch) * batch;
     const int nb = mode == 0 ? min(batch, n - k0) : n;
     if (tid >= nb) return;
-    const int idx = mode == 0 ? order[size_t(e) * n + k0 + tid] : tid;
+    const int idx = mode == 0 ? next : tid;
     xin = reinterpret_cast<const float4*>(X)[idx];
     if (tid / kCtaSamples == rank)
 #pragma unroll
       for (int k = 0; k < kOut; ++k) tin[k] = Y[size_t(idx) * kOut + k];
   };
+  load_index(0);
   load_rows(0);
+  load_index(1);
   cluster.sync();  // every CTA of the cluster runs: its shared memory may be written
 
   for (int st = 0; st < steps; ++st) {
     const int k0 = (st % per_epoch) * batch;
     const int nb = mode == 0 ? min(batch, n - k0) : n;
     const int first = kCtaSamples * rank;                      // this CTA's samples
+    const float scale = 2.f / float(nb * kOut);
     const int mine = max(0, min(kCtaSamples, nb - first));
     if (tid < nb) reinterpret_cast<float4*>(s.X)[tid] = xin;
     if (tid >= first && tid < first + mine)
@@ -216,12 +226,12 @@ mlp_train_kernel(float* params, float* adam_m, float* adam_v, const float* __res
 #pragma unroll
       for (int j = 0; j < kHid; j += 4) {
         const float4 h = *reinterpret_cast<const float4*>(&s.H2[b * kPad + j]);
-        y = fmaf(h.x, s.W3[j * kOut + kk], y);
-        y = fmaf(h.y, s.W3[(j + 1) * kOut + kk], y);
-        y = fmaf(h.z, s.W3[(j + 2) * kOut + kk], y);
-        y = fmaf(h.w, s.W3[(j + 3) * kOut + kk], y);
+        const float4 w = *reinterpret_cast<const float4*>(&s.W3t[kk * kHid + j]);
+        y = fmaf(h.x, w.x, y);
+        y = fmaf(h.y, w.y, y);
+        y = fmaf(h.z, w.z, y);
+        y = fmaf(h.w, w.w, y);
       }
-      const float scale = 2.f / float(nb * kOut);
       const float d = y - s.T[b * 4 + kk];
       const float d1 = __shfl_down_sync(0xffffffffu, d, 1), d2 = __shfl_down_sync(0xffffffffu, d, 2);
       if (b < mine) {
@@ -240,16 +250,20 @@ mlp_train_kernel(float* params, float* adam_m, float* adam_v, const float* __res
     {
       const int b = tid >> 4, j = (tid & 15) * 4;
       if (b < mine) {
-        float dz[4];
+        const float4 h4 = *reinterpret_cast<const float4*>(&s.H2[b * kPad + j]);
+        const float hv[4] = {h4.x, h4.y, h4.z, h4.w};
+        float g[4] = {0.f, 0.f, 0.f, 0.f}, dz[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          float g = 0.f;
-#pragma unroll
-          for (int k = 0; k < kOut; ++k)
-            g = fmaf(s.DY[(first + b) * 4 + k], s.W3[(j + q) * kOut + k], g);
-          const float h = s.H2[b * kPad + j + q];
-          dz[q] = g * (1.f - h * h);
+        for (int k = 0; k < kOut; ++k) {
+          const float dy = s.DY[(first + b) * 4 + k];
+          const float4 w = *reinterpret_cast<const float4*>(&s.W3t[k * kHid + j]);
+          g[0] = fmaf(dy, w.x, g[0]);
+          g[1] = fmaf(dy, w.y, g[1]);
+          g[2] = fmaf(dy, w.z, g[2]);
+          g[3] = fmaf(dy, w.w, g[3]);
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dz[q] = g[q] * (1.f - hv[q] * hv[q]);
         const float4 dv = make_float4(dz[0], dz[1], dz[2], dz[3]);
         *reinterpret_cast<float4*>(&s.DZ2[b * kPad + j]) = dv;
         *reinterpret_cast<float4*>(cluster.map_shared_rank(
@@ -293,6 +307,7 @@ mlp_train_kernel(float* params, float* adam_m, float* adam_v, const float* __res
       }
     }
     load_rows(st + 1);
+    load_index(st + 2);
     cluster.sync();  // every sample's activations and derivatives are in place
 
     // gradients of the owned parameters over the minibatch, then Adam
