@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <string>
 
@@ -49,7 +50,7 @@ constexpr int kMaxBatch = 128;                 // largest minibatch
 // of one thread going through it alone (inputs, then samples, ascending), so
 // results do not depend on the split.  One CTA of 128 threads, a sample per
 // thread and 37 parameters each in the second half, took 72 us per minibatch
-// of 128 against 7.5 us here.
+// of 128 against 7.6 us here.
 constexpr int kClusterCtas = 8;
 constexpr int kTrainThreads = 256;
 constexpr int kCtaSamples = kMaxBatch / kClusterCtas;  // 16
@@ -72,8 +73,9 @@ struct TrainSmem {
   float red[kMaxBatch / 32];
 };
 
-// Where parameter p of the flat vector lives in a CTA's copy (an offset in
-// floats from the start of TrainSmem).
+// Where parameter p of the flat vector lives in a CTA's copy of the weights (an
+// offset in floats from the start of TrainSmem and of PredictSmem, which begin
+// alike; W3 transposed for vector loads).
 __device__ __forceinline__ int weight_slot(int p) {
   constexpr int o1 = 0, ob1 = o1 + kIn * kHid, o2 = ob1 + kHid, ob2 = o2 + kHid * kPad,
                 o3 = ob2 + kHid, ob3 = o3 + kHid * kOut;
@@ -81,7 +83,7 @@ __device__ __forceinline__ int weight_slot(int p) {
   if (p < kOffW2) return ob1 + (p - kOffB1);
   if (p < kOffB2) return o2 + (p - kOffW2) / kHid * kPad + (p - kOffW2) % kHid;
   if (p < kOffW3) return ob2 + (p - kOffB2);
-  if (p < kOffB3) return o3 + (p - kOffW3) % kOut * kHid + (p - kOffW3) / kOut;  // transposed
+  if (p < kOffB3) return o3 + (p - kOffW3) % kOut * kHid + (p - kOffW3) / kOut;
   return ob3 + (p - kOffB3);
 }
 
@@ -411,11 +413,14 @@ mlp_train_kernel(float* params, float* adam_m, float* adam_v, const float* __res
 // 4096 multiply-adds deep.)  X and Y may be mapped host memory.
 constexpr int kPredictSamples = 16;
 struct PredictSmem {
-  float W1[kIn * kHid], b1[kHid], W2[kHid * kPad], b2[kHid], W3[kHid * kOut], b3[kOut + 1];
+  float W1[kIn * kHid], b1[kHid], W2[kHid * kPad], b2[kHid], W3t[kOut * kHid], b3[kOut + 1];
   float X[kPredictSamples * kIn];
   float H1[kPredictSamples * kPad];
   float H2[kPredictSamples * kPad];
 };
+static_assert(offsetof(PredictSmem, W3t) == offsetof(TrainSmem, W3t) &&
+                  offsetof(PredictSmem, b3) == offsetof(TrainSmem, b3),
+              "weight_slot serves both");
 
 __global__ void __launch_bounds__(kTrainThreads)
 mlp_predict_kernel(const float* __restrict__ params, const float* __restrict__ X, int n,
@@ -478,7 +483,14 @@ mlp_predict_kernel(const float* __restrict__ params, const float* __restrict__ X
       const int b = tid / kOut, k = tid % kOut;
       float y = s.b3[k];
 #pragma unroll
-      for (int j = 0; j < kHid; ++j) y = fmaf(s.H2[b * kPad + j], s.W3[j * kOut + k], y);
+      for (int j = 0; j < kHid; j += 4) {
+        const float4 h = *reinterpret_cast<const float4*>(&s.H2[b * kPad + j]);
+        const float4 w = *reinterpret_cast<const float4*>(&s.W3t[k * kHid + j]);
+        y = fmaf(h.x, w.x, y);
+        y = fmaf(h.y, w.y, y);
+        y = fmaf(h.z, w.z, y);
+        y = fmaf(h.w, w.w, y);
+      }
       Y[size_t(first) * kOut + tid] = y;
     }
     // (the next group's writes to X and H1 come before its own barriers, after
