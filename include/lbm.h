@@ -196,7 +196,9 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
 lbm_status lbm_step(lbm_ctx *ctx, int n, int scheme, double tau, double sigma);
 
 /* Queue n steps without waiting and without reading the status (for timing
- * and graph capture); lbm_sync_status() later waits and reports. */
+ * and graph capture); lbm_sync_status() later waits and reports.  Captured into
+ * the caller's graph, an even n leaves the state in the buffer it was in, so
+ * that the graph can be replayed any number of times. */
 lbm_status lbm_step_async(lbm_ctx *ctx, int n, int scheme, double tau,
                           double sigma);
 lbm_status lbm_sync_status(lbm_ctx *ctx);

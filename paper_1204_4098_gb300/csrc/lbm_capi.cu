@@ -481,6 +481,21 @@ cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t
   return cudaSuccess;
 }
 
+// A caller that captures an even number of steps may replay its graph any
+// number of times, if they leave the state in the buffer they found it in.
+// Launches of several steps can make the number of launches odd: the steps to
+// run one by one first so that it is odd or even as n is.
+int single_steps(const StepPlan& plan, int n) {
+  const int per = plan.kind == kTileRuns ? plan.tile_steps : 2;
+  auto launches = [&](int m) {
+    if (plan.kind == kSingleSteps) return m;
+    return plan.kind == kTileRuns ? (m + per - 1) / per : m / 2 + m % 2;
+  };
+  int s = 0;
+  while (s < n && (s + launches(n - s) - n) % 2 != 0) ++s;
+  return s;
+}
+
 // Every argument a step kernel reads, compared field by field.
 bool same_launch(const StripLaunch& x, const StripLaunch& y) {
   return x.src == y.src && x.dst == y.dst && x.rho_src == y.rho_src && x.rho_dst == y.rho_dst &&
@@ -589,10 +604,18 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
   // own: the steps are then recorded one launch at a time)
   const bool graphs = !c->band && n >= graph_steps(plan, false) &&
                       size_t(c->p.nx) * c->p.ny <= kGraphMaxCells;
+  const int single = single_steps(plan, n);
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (graphs && cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) {
+  if ((graphs || single > 0) && cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) {
     cudaGetLastError();  // treated as capturing: plain launches
     capturing = cudaStreamCaptureStatusActive;
+  }
+  if (capturing != cudaStreamCaptureStatusNone && single > 0) {
+    StepPlan ones = plan;
+    ones.kind = kSingleSteps;
+    const cudaError_t e = run_plan(c, scheme, ones, single, c->stream, &launches);
+    if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+    k = single;
   }
   if (graphs && capturing == cudaStreamCaptureStatusNone) {
     for (const bool longer : {true, false}) {

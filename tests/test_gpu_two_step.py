@@ -182,3 +182,28 @@ def test_batch_instance_that_diverges_leaves_the_others_alone():
     assert b.run(1) == 3 and alone.run(1) == 1
     assert b.result(1)["status"] == lbm.RUN_DIVERGED
     assert np.array_equal(b.density(2), alone.density(0))
+
+
+# a caller's graph of an even number of steps leaves the state in the buffer it
+# found it in, however many steps its launches take, so it can be replayed
+@pytest.mark.parametrize("nx,ny,precision", [
+    (66, 40, lbm.FP32), (310, 290, lbm.FP32), (340, 370, lbm.FP32), (600, 300, lbm.FP32),
+    (601, 301, lbm.FP32), (600, 300, lbm.BF16DEV), (60, 50, lbm.FP64)])
+@pytest.mark.parametrize("steps", [2, 4, 6, 10, 12, 18])
+def test_replays_of_captured_steps(nx, ny, precision, steps):
+    torch = pytest.importorskip("torch")
+    stream = torch.cuda.Stream()
+    with lbm.Lattice(nx, ny, T, precision=precision, stream=stream.cuda_stream) as lat:
+        lat.init_density(*field(nx, ny, 3))
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+            lat.step_async(steps, lbm.IMPROVED, 0.8, 0.1)
+        for _ in range(3):
+            graph.replay()
+        torch.cuda.synchronize()
+        got = lat.populations()
+    with lbm.Lattice(nx, ny, T, precision=precision) as lat:
+        lat.init_density(*field(nx, ny, 3))
+        lat.step(3 * steps, lbm.IMPROVED, 0.8, 0.1)
+        assert np.array_equal(got, lat.populations())
