@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include "lbm.h"
@@ -511,7 +512,10 @@ struct lbm_mlp {
   float* d_v = nullptr;
   float* d_scratch = nullptr;  // gradient / loss
   // predict: samples of a small call in mapped host memory, of a larger one on
-  // the device; kept for the next call, at most kStageMost samples
+  // the device; kept for the next call, at most kStageMost samples.  One call
+  // at a time holds them (stage_mutex); one that another thread makes meanwhile
+  // takes buffers of its own.
+  std::mutex stage_mutex;
   float* h_stage = nullptr;    // kStageSamples x (4 + 3), page-locked
   float* d_stage = nullptr;    // stage_samples x (4 + 3)
   int stage_samples = 0;
@@ -700,7 +704,8 @@ lbm_status lbm_mlp_predict(lbm_mlp* m, const float* X, int n, float* Y) {
   const size_t xb = size_t(n) * kIn * sizeof(float), yb = size_t(n) * kOut * sizeof(float);
   const int groups = (n + kPredictSamples - 1) / kPredictSamples;
   const int grid = std::min(groups, 4 * m->sm_count);
-  if (n <= kStageSamples) {
+  const std::unique_lock<std::mutex> stage(m->stage_mutex, std::try_to_lock);
+  if (n <= kStageSamples && stage) {
     // small calls: the kernel reads and writes page-locked host memory, so the
     // call is one launch and one wait (256 samples: 58 -> 22 us against two
     // allocations, two copies and one CTA per 256 samples)
@@ -720,9 +725,9 @@ lbm_status lbm_mlp_predict(lbm_mlp* m, const float* X, int n, float* Y) {
     std::memcpy(Y, hy, yb);
     return LBM_OK;
   }
-  DevBuf temp;  // beyond the staging that is kept
+  DevBuf temp;  // beyond the staging that is kept, or beside a call that holds it
   float* dx = nullptr;
-  if (n <= kStageMost) {
+  if (n <= kStageMost && stage) {
     if (m->stage_samples < n) {
       cudaFree(m->d_stage);  // (waits for the work that reads it)
       m->d_stage = nullptr;

@@ -1,5 +1,7 @@
 """Prediction and gradients of the warm-start network at the edges of their
 sample groups and staging, against the FP64 oracle."""
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 
@@ -39,3 +41,14 @@ def test_gradient_sizes(n):
                                    T.astype(np.float32))
     assert loss == pytest.approx(want_loss, rel=1e-5)
     assert np.max(np.abs(g - want)) <= 2e-5 * np.max(np.abs(want)) + 1e-8
+
+
+# several threads predicting with one network: none gets another's staging
+def test_predict_from_several_threads():
+    net = lbm.MLP(network(5))
+    jobs = [np.random.default_rng(k).uniform(-1, 1, (n, 4)).astype(np.float32)
+            for k, n in enumerate([17, 300, 4096, 5000, 1, 20000, 64, 4097] * 8)]
+    want = [net.predict(X) for X in jobs]
+    with ThreadPoolExecutor(8) as pool:
+        for got, w in zip(pool.map(net.predict, jobs), want):
+            assert np.array_equal(got, w)
