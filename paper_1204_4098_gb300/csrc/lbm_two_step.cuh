@@ -16,7 +16,9 @@
 // march (the one-step kernel's extra halo loads, shuffles and psi evaluation,
 // ~10 % of its instructions, have no counterpart); 8 of 64 columns are
 // computed twice.  At the wrong side of the strip's edge, lanes compute
-// values that nothing uses.  Rows likewise: a band of n rows pulls n + 6; the
+// values that nothing uses: of columns -4 .. 59 (0 .. 55 owned), step 1 needs
+// psi of -3 .. 58 and step 2 of -1 .. 56, one column of each outermost lane
+// (psi_row).  Rows likewise: a band of n rows pulls n + 6; the
 // first iterations run only the part of the work that their rows are for (the
 // whole work in all n + 7: 1024^2 10.9 us per step instead of 9.9).
 //
@@ -183,7 +185,10 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
   int y0, y1, n_rows;  // rows of this lane's band; pulled rows of the march
   int xo, ca, cb;      // left column of this lane; its loaded columns (wrapped)
   int from_l = 0, from_r = 0;  // kRing: lanes holding the columns beside
-  bool valid1, valid2;  // the lane's step-1 / step-2 densities are the lattice's
+  // whether columns of the lane are collided in step 1 / 2, and whether psi of
+  // its left (_l) and right (_r) column is used there
+  bool valid1, valid2;
+  bool psi1_l, psi1_r, psi2_l, psi2_r;
   bool store_a, store_b;
   if constexpr (LAYOUT == kRing) {
     const int width = nx / 2;                   // lanes of a row
@@ -199,6 +204,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
     from_l = l == 0 ? base + width - 1 : lane - 1;
     from_r = l == width - 1 ? base : lane + 1;
     valid1 = valid2 = in_row;
+    psi1_l = psi1_r = psi2_l = psi2_r = in_row;
     store_a = store_b = in_row;
     if (y0 >= y1) {  // a half-warp without a band: marches along, stores nothing
       y0 = A.y_begin;
@@ -214,6 +220,10 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
     cb = ca + 1 == nx ? 0 : ca + 1;
     valid1 = lane >= 1 && lane < 31;
     valid2 = lane >= 2 && lane < 30;
+    psi1_l = lane != 0;
+    psi1_r = lane != 31;
+    psi2_l = lane >= 2 && lane < 31;
+    psi2_r = lane >= 1 && lane < 30;
     store_a = valid2 && xo < nx;
     store_b = valid2 && xo + 1 < nx;
   }
@@ -307,16 +317,22 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
     for (int a = 1; a < kQ; ++a) r = add_rn(r, P[a]);
     return r;
   };
-  auto psi_row = [&](F2 r, bool valid) {
+  // psi of a row; use_l, use_r: whether that of the lane's left and right column
+  // is used (`some`: either).  Where one is, kNormal checks both: the other, of
+  // a density that lacks its share from beyond the strip, can only have the item
+  // run again, and masking it costs more (us per step, this / masked: 1024^2 9.29
+  // / 9.73, 4096^2 111.9 / 113.9, BF16 129.4 / 133.3).  The full form reports
+  // divergence, of the columns in use only.
+  auto psi_row = [&](F2 r, bool some, bool use_l, bool use_r) {
     PsiRow p;
     if constexpr (kNormal) {
       bool ok;
       p.c = psi_normal(r, A.P, ok);
-      fine = fine && (ok || !valid);
+      fine = fine & (ok | !some);  // (with && and || BF16 4096^2 131.1)
     } else {
-      bool f = false;
-      p.c = psi_of_rho(r, A.P, f);
-      bad |= f && valid;
+      bool fl = false, fr = false;
+      p.c = F2(psi_of_rho(r.x(), A.P, fl), psi_of_rho(r.y(), A.P, fr));
+      bad |= (fl && use_l) || (fr && use_r);
     }
     const F2 W = F2(left(p.c.y()), p.c.x());
     const F2 E = F2(p.c.y(), right(p.c.x()));
@@ -367,7 +383,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
   // Step 2 of iteration k: psi of its pulled row r - 3 ...
   PsiRow p2 = none;
   auto step2_psi = [&]() {
-    if constexpr (kNeedPsi) p2 = psi_row(qrhoB, valid2);
+    if constexpr (kNeedPsi) p2 = psi_row(qrhoB, LAYOUT == kRing ? valid2 : valid1, psi2_l, psi2_r);
     else rho_check(qrhoB, valid2);
   };
   // ... and its output row r - 4
@@ -421,7 +437,7 @@ __device__ __forceinline__ bool strip_run_two(const StripArgs<S>& A, int strip, 
   auto step1 = [&](int k, bool full) {
     const F2 rho1 = rho_of(P1);
     PsiRow p1 = none;
-    if constexpr (kNeedPsi) p1 = psi_row(rho1, valid1);
+    if constexpr (kNeedPsi) p1 = psi_row(rho1, LAYOUT != kRing || valid1, psi1_l, psi1_r);
     else rho_check(rho1, valid1);
     m2 = z2;
     z2 = p2;
