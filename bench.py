@@ -110,6 +110,10 @@ MEASURED_TRAFFIC = {
     # copies: 616.8 + 554.9 MB (one step), 630.7 + 558.8 (two), x4 cells
     ("c9ce772ed26597b5", "fp32", 8192, "pair"): 4.6868e9,
     ("c9ce772ed26597b5", "fp32", 8192, "two_step"): 4.7581e9,
+    # the two-step kernel with psi checked at every column in use: 616.8 + 554.9 MB
+    # (one step), 630.7 + 558.8 (two), x4 cells
+    ("cfed21be853ad9c9", "fp32", 8192, "pair"): 4.6868e9,
+    ("cfed21be853ad9c9", "fp32", 8192, "two_step"): 4.7578e9,
 }
 
 
