@@ -870,13 +870,17 @@ lbm_status keep_graph(lbm_batch* b, const std::vector<int>& key, cudaGraphExec_t
     cudaGetLastError();
     return bfail(b, LBM_E_CUDA, std::string("instantiate: ") + cudaGetErrorString(e));
   }
-  if (b->graphs.size() >= kMaxGraphs) {  // (none is running: every window is waited for)
-    for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
-    b->graphs.clear();
-  }
   b->graphs[key] = exec;
   *out = exec;
   return LBM_OK;
+}
+
+// Before a window takes its graphs: drop the kept ones if it could need `more`
+// than there is room for.  (None is running: every window is waited for.)
+void make_graph_room(lbm_batch* b, size_t more) {
+  if (b->graphs.size() + more <= kMaxGraphs) return;
+  for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
+  b->graphs.clear();
 }
 
 // One window as a CUDA graph, captured once per (mode, class grids) and
@@ -893,6 +897,7 @@ lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
     *out = it->second;
     return LBM_OK;
   }
+  make_graph_room(b, 1);
   LBM_BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   const int span = b->pers_grid_max + 1;
   // with both classes active they run as two branches of the graph, joined
@@ -993,11 +998,11 @@ lbm_status window_graph(lbm_batch* b, int mode, cudaGraphExec_t* out) {
   return keep_graph(b, key, out);
 }
 
-// The chunk of launches that a two-step window replays: kTwoChunk launches of
-// every chain, side by side.  The chains advance different instances, so one
-// fills the SMs while another's launch ends and the next begins.
-lbm_status two_step_graph(lbm_batch* b, cudaGraphExec_t* out) {
-  std::vector<int> key{kBatchTwoStep};
+// `launches` launches of every chain, side by side, as a graph.  The chains
+// advance different instances, so one fills the SMs while another's launch ends
+// and the next begins.
+lbm_status two_step_graph(lbm_batch* b, int launches, cudaGraphExec_t* out) {
+  std::vector<int> key{kBatchTwoStep, launches};
   for (const auto& c : b->two_chain) key.insert(key.end(), {c.first, c.second});
   const auto it = b->graphs.find(key);
   if (it != b->graphs.end()) {
@@ -1010,22 +1015,35 @@ lbm_status two_step_graph(lbm_batch* b, cudaGraphExec_t* out) {
   for (int c = 0; c < chains; ++c) {
     const cudaStream_t q = c == 0 ? b->stream : b->two_side[c - 1];
     if (c > 0) cudaStreamWaitEvent(q, b->ev_fork, 0);
-    for (int s = 0; s < kTwoChunk; ++s) two_step_chain(b, c, s, q);
+    for (int s = 0; s < launches; ++s) two_step_chain(b, c, s, q);
     if (c > 0) cudaEventRecord(b->two_join[c - 1], q);
   }
   for (int c = 1; c < chains; ++c) cudaStreamWaitEvent(b->stream, b->two_join[c - 1], 0);
   return keep_graph(b, key, out);
 }
 
-// Queue a two-step window: chunks of kTwoChunk launches (`chunk`), what is left
-// of an even number of launches (the state ends in buf[0]), the last two steps
-// one by one where W / 2 is odd, and the reduction.
-lbm_status two_step_window(lbm_batch* b, cudaGraphExec_t chunk) {
+// The launches of a chain in a two-step window: an even number, so that the
+// state ends in buf[0].  They go in chunks of kTwoChunk and a graph of what is
+// left (plain launches of one chain after the other instead, windows of 98 steps:
+// 48 mixed slabs 48.7 -> 107.7 us per step, 6 narrow ones 7.9 -> 27.4).
+struct TwoStepGraphs {
+  cudaGraphExec_t chunk = nullptr, rest = nullptr;
+};
+lbm_status two_step_graphs(lbm_batch* b, TwoStepGraphs* g) {
+  const int launches = b->p.window / 4 * 2, rest = launches % kTwoChunk;
+  make_graph_room(b, 2);
+  lbm_status st = LBM_OK;
+  if (launches >= kTwoChunk) st = two_step_graph(b, kTwoChunk, &g->chunk);
+  if (st == LBM_OK && rest > 0) st = two_step_graph(b, rest, &g->rest);
+  return st;
+}
+
+// Queue a two-step window: its graphs, the last two steps one by one where W / 2
+// is odd, and the reduction.
+lbm_status two_step_window(lbm_batch* b, const TwoStepGraphs& g) {
   const int W = b->p.window;
-  int left = W / 4 * 2;
-  for (; left >= kTwoChunk; left -= kTwoChunk) LBM_BCUDA(b, cudaGraphLaunch(chunk, b->stream));
-  for (int c = 0; c < int(b->two_chain.size()); ++c)
-    for (int s = 0; s < left; ++s) two_step_chain(b, c, s, b->stream);
+  for (int k = W / 4 * 2 / kTwoChunk; k > 0; --k) LBM_BCUDA(b, cudaGraphLaunch(g.chunk, b->stream));
+  if (g.rest) LBM_BCUDA(b, cudaGraphLaunch(g.rest, b->stream));
   if (W % 4 != 0) {
     batch_copies_kernel<<<b->count, kReduceCta, 0, b->stream>>>(b->d_inst, b->d_active,
                                                                 b->d_n_active + 1, b->buf[0]);
@@ -1490,8 +1508,9 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     if (st != LBM_OK) return st;
     cudaGraphExec_t g = nullptr;
     // (before the clock starts: a new graph takes the host milliseconds)
-    if (mode != kBatchTwoStep) st = window_graph(b, mode, &g);
-    else if (b->p.window / 4 * 2 >= kTwoChunk) st = two_step_graph(b, &g);
+    TwoStepGraphs two;
+    if (mode == kBatchTwoStep) st = two_step_graphs(b, &two);
+    else st = window_graph(b, mode, &g);
     if (st != LBM_OK && mode == LBM_BATCH_COOPERATIVE && b->p.mode == LBM_BATCH_AUTO) {
       // cooperative windows unavailable here: drop them and use the work list
       b->coop_grid = 0;
@@ -1503,7 +1522,7 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     const size_t cells = active_cells(b);
     LBM_BCUDA(b, cudaEventRecord(b->ev0, b->stream));
     if (mode == kBatchTwoStep) {
-      st = two_step_window(b, g);
+      st = two_step_window(b, two);
       if (st != LBM_OK) return st;
     } else {
       LBM_BCUDA(b, cudaGraphLaunch(g, b->stream));

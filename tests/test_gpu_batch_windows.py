@@ -39,3 +39,35 @@ def test_device_time_of_a_window_leaves_out_the_capture_of_its_graph():
         first.append(first_ms)
         later += rest
     assert min(first) < 1.5 * np.median(later)
+
+
+def test_short_windows_cost_no_more_per_step_than_a_chunk():
+    # 98 steps are 48 launches a chain and two steps one by one, 100 one chunk
+    step = {}
+    for window in (100, 98, 50):
+        b = batch(window)
+        window_ms(b, 3)
+        step[window] = np.median(window_ms(b, 9)) / window
+    # a window itself (tail, reduction, gaps) costs less than 50 steps of these
+    assert step[98] < 1.5 * step[100]
+    assert step[50] < 2.0 * step[100]
+
+
+# (launches a chain: 0, 2, 8, 10; 48 and two steps; a chunk; a chunk and 2, 24, 48)
+@pytest.mark.parametrize("window", [2, 4, 6, 16, 20, 98, 100, 102, 104, 150, 196])
+def test_windows_of_any_length(window):
+    inst = [dict(SMALL[k % 6], nx=nx, ny=ny) for k, (nx, ny) in
+            enumerate([(32, 41), (64, 33), (114, 40), (66, 19), (57, 30), (1, 21), (3, 33)])]
+    b = batch(window, inst, rows=8)
+    start = []
+    for k, d in enumerate(inst):
+        start.append(b.density(k).astype(np.float64))
+        b.init_density(k, start[k])
+    assert b.run(2) == len(inst)
+    for k, d in enumerate(inst):
+        with lbm.Lattice(d["nx"], d["ny"], T) as lat:
+            lat.set_variant(lbm.VARIANT_REGISTER)
+            lat.init_density(start[k])
+            lat.step(2 * window, d["scheme"], d["tau"], d["sigma"])
+            for got, want in zip(b.moments(k), lat.observe()):
+                assert np.array_equal(got, want), (k, d)
