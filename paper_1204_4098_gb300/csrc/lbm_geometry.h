@@ -120,7 +120,11 @@ constexpr int kTwoStepFewWarps = 8;  // of launches that have no use for more
 // and band height (a requested kernel or height runs as requested), a lattice
 // large enough to gain, 32-bit byte offsets within a plane, and a covolume for
 // which every density inside the domain of psi (b rho / 4 < 1) has a normal
-// reciprocal.
+// reciprocal.  Not 1 or 3 columns: the one-by-one copies of a row then all read
+// the same few addresses, which takes longer than the rest of the march (us per
+// step, one step per launch / two: 1 x 32000 17.4 / 51.9, 3 x 10666 8.6 / 10.6, 3
+// x 133333 60 / 76; 5 x 6400 6.9 / 6.0, 7 x 57142 28.5 / 25.8; even widths gain
+// from 2 on).
 constexpr long long kTwoStepMinCells = 176LL * 176;
 constexpr long long kTwoStepMaxCells = 1LL << 30;
 inline bool two_step_applies(int requested, int precision, int nx, int ny,
@@ -128,7 +132,8 @@ inline bool two_step_applies(int requested, int precision, int nx, int ny,
   const long long cells = (long long)nx * ny;
   const bool dev = precision == LBM_BF16DEV || precision == LBM_FP16DEV;
   return requested == LBM_VARIANT_AUTO && band_rows_override == 0 &&
-         (precision == LBM_FP32 || (dev && nx % 2 == 0)) && cells >= kTwoStepMinCells &&
+         (precision == LBM_FP32 || (dev && nx % 2 == 0)) && nx != 1 && nx != 3 &&
+         cells >= kTwoStepMinCells &&
          cells <= kTwoStepMaxCells && b > 1e-12 && b < 1e12;
 }
 
