@@ -620,7 +620,7 @@ using namespace lbm;
 // that rounding leaves without.  (48 lattices of even width, us per step: 43.5
 // with one chain, 38.8 with 2, 36.0 with 3, 35.3 with 6, 35.5 with 12.)
 constexpr int kTwoChainsWanted = 6;
-constexpr int kTwoMaxChains = kTwoChainsWanted + kTwoBatchLayouts;
+constexpr int kTwoMaxChains = kTwoChainsWanted + kTwoBatchLayouts + 1;  // (kTwoBatchSingle)
 constexpr int kTwoChunk = 50;       // launches per chain in a captured chunk (even)
 constexpr size_t kMaxGraphs = 64;   // captured graphs kept by a batch
 
@@ -659,7 +659,7 @@ struct lbm_batch {
   int2* d_two_chain = nullptr;
   int4* h_two_items = nullptr;
   int2* h_two_chain = nullptr;
-  std::vector<std::pair<int, int>> two_chain;  // (layout, grid)
+  std::vector<std::pair<int, int>> two_chain;  // (layout or kTwoBatchSingle, grid)
   cudaStream_t two_side[kTwoMaxChains - 1] = {};
   cudaEvent_t two_join[kTwoMaxChains - 1] = {};
   int* h_active = nullptr;
@@ -736,20 +736,41 @@ constexpr int kBalancedMinRows = 8;
 constexpr int kBatchTwoStep = 100;
 constexpr int kTwoMinRows = 4;  // shortest band of a two-step window
 
-// AUTO runs two-step windows, unless one column per lane was asked for or the
-// covolume is outside the range of two_step_applies.  (A window of fewer than
-// four steps has no even number of two-step launches.)
+// Lattices of one column take one step per launch in two-step windows too, as a
+// chain of their own: the march's lanes would all read the same address (96 of 1
+// x 320, us per step: 46.9 with two steps per launch, 21.8 with one).  Bands of
+// kSingleRows rows.
+constexpr int kTwoBatchSingle = kTwoBatchLayouts;
+constexpr int kSingleRows = 16;
+bool takes_two_steps(const BatchInst& d) { return d.nx > 1; }
+
+// AUTO runs two-step windows, unless one column per lane was asked for, no
+// lattice takes two steps or the covolume is outside the range of
+// two_step_applies.  (A window of fewer than four steps has no even number of
+// two-step launches.)
 bool two_step_windows(const lbm_batch* b) {
   return b->p.mode == LBM_BATCH_AUTO && b->p.variant != LBM_VARIANT_REGISTER &&
-         b->p.window >= 4 && b->p.b > 1e-12 && b->p.b < 1e12;
+         b->p.window >= 4 && b->p.b > 1e-12 && b->p.b < 1e12 &&
+         std::any_of(b->desc.begin(), b->desc.end(), takes_two_steps);
 }
 
 std::vector<TwoLattice> two_lattices(const lbm_batch* b) {
   std::vector<TwoLattice> lat;
   lat.reserve(b->active.size());
-  for (int i : b->active) lat.push_back(TwoLattice{i, b->desc[i].nx, b->desc[i].ny});
+  for (int i : b->active)
+    if (takes_two_steps(b->desc[i]))
+      lat.push_back(TwoLattice{i, b->desc[i].nx, b->desc[i].ny});
   two_layouts(lat);
   return lat;
+}
+
+// Grid of a class kernel for the current active set (worklist_grid for the
+// work list); 0 when the class has no active instance.
+int class_grid(const lbm_batch* b, int mode, int cls) {
+  if (b->class_items[cls] == 0) return 0;
+  if (mode == LBM_BATCH_PERSISTENT) return b->pers_grid_max;
+  if (mode == LBM_BATCH_BALANCED) return b->wl_grid[cls];
+  return worklist_grid(b->class_items[cls], kWorklistThreads / 32, b->wl_grid[cls]);
 }
 
 // Rebuild the active list (two-column instances first), the work-list prefix
@@ -806,6 +827,8 @@ lbm_status upload_tables(lbm_batch* b, int mode, int rows) {
       b->two_chain.push_back({chain.layout, two_item_grid(n)});
       total += n;
     }
+    if (b->class_items[1] > 0)  // (the one-column class)
+      b->two_chain.push_back({kTwoBatchSingle, class_grid(b, LBM_BATCH_WORKLIST, 1)});
     LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_items, b->h_two_items, total * sizeof(int4),
                                  cudaMemcpyHostToDevice, b->stream));
     LBM_BCUDA(b, cudaMemcpyAsync(b->d_two_chain, b->h_two_chain, c * sizeof(int2),
@@ -830,18 +853,17 @@ lbm_status upload_tables(lbm_batch* b, int mode, int rows) {
   return LBM_OK;
 }
 
-// Grid of a class kernel for the current active set (worklist_grid for the
-// work list); 0 when the class has no active instance.
-int class_grid(const lbm_batch* b, int mode, int cls) {
-  if (b->class_items[cls] == 0) return 0;
-  if (mode == LBM_BATCH_PERSISTENT) return b->pers_grid_max;
-  if (mode == LBM_BATCH_BALANCED) return b->wl_grid[cls];
-  return worklist_grid(b->class_items[cls], kWorklistThreads / 32, b->wl_grid[cls]);
-}
-
-// Launch s of chain c of a two-step window.
+// Launch s of chain c of a two-step window (of one-column lattices: the two
+// launches of its two steps, from buf[0] back to it).
 void two_step_chain(lbm_batch* b, int c, int s, cudaStream_t q) {
   const int layout = b->two_chain[c].first, grid = b->two_chain[c].second;
+  if (layout == kTwoBatchSingle) {
+    for (int k = 0; k < 2; ++k)
+      batch_worklist_kernel<false><<<grid, kWorklistThreads, 0, q>>>(
+          b->d_inst, b->d_active, b->d_prefix, b->d_n_active, b->buf[k], b->buf[1 - k],
+          b->d_status);
+    return;
+  }
   const auto kernel = layout == kTwoBatchPairs  ? batch_two_step_kernel<kFlatEven>
                       : layout == kTwoBatchRing ? batch_two_step_kernel<kRing>
                                                 : batch_two_step_kernel<kAnyWidth>;
@@ -1181,7 +1203,7 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
     d.nx = s.nx;
     d.ny = s.ny;
     d.pair = (s.nx % 2 == 0 || s.nx >= 3) && p->variant != LBM_VARIANT_REGISTER;
-    d.pitch = s.nx % 2 && p->variant != LBM_VARIANT_REGISTER ? s.nx + 3 : s.nx;
+    d.pitch = d.pair && s.nx % 2 ? s.nx + 3 : s.nx;
     d.n_strips = d.pair ? (s.nx + 63) / 64 : (s.nx + 31) / 32;
     d.scheme = s.scheme;
     d.row_off = roff;
@@ -1503,7 +1525,10 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
   for (int w = 0; w < max_windows && !b->active.empty(); ++w) {
     int mode = LBM_BATCH_WORKLIST, rows = 32;
     choose_config(b, mode, rows);
-    for (auto& d : b->desc) set_geometry(d, rows > 0 ? rows : 32);
+    for (auto& d : b->desc)
+      set_geometry(d, mode == kBatchTwoStep && !takes_two_steps(d) ? kSingleRows
+                      : rows > 0                                   ? rows
+                                                                   : 32);
     lbm_status st = upload_tables(b, mode, rows);
     if (st != LBM_OK) return st;
     cudaGraphExec_t g = nullptr;
@@ -1534,9 +1559,10 @@ lbm_status lbm_batch_run(lbm_batch* b, int max_windows, int* n_active) {
     const unsigned long long classes =
         (class_grid(b, mode, 0) > 0 ? 1 : 0) + (class_grid(b, mode, 1) > 0 ? 1 : 0);
     const unsigned long long W = b->p.window;
+    unsigned long long per_two = 0;  // of all chains, for two steps
+    for (const auto& c : b->two_chain) per_two += c.first == kTwoBatchSingle ? 2 : 1;
     const unsigned long long nl =
-        1 + (mode == kBatchTwoStep
-                 ? b->two_chain.size() * (W / 4 * 2) + (W % 4 ? 2 * classes + 1 : 0)
+        1 + (mode == kBatchTwoStep ? per_two * (W / 4 * 2) + (W % 4 ? 2 * classes + 1 : 0)
              : mode == LBM_BATCH_COOPERATIVE ? 1
              : mode == LBM_BATCH_PERSISTENT  ? classes
                                              : classes * W);
