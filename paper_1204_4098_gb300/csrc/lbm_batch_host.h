@@ -155,10 +155,11 @@ inline int two_item_strips(const TwoLattice& t) {
 inline int two_item_halves(const TwoLattice& t) {
   return t.layout == kTwoBatchRing && t.nx <= 32 ? 2 : 1;
 }
-// Items over the height of one strip for bands of `rows` rows.
+// Items over the height of one strip for bands of `rows` rows (any height; one
+// taller than the lattice is the lattice).
 inline int two_item_bands(const TwoLattice& t, int rows) {
-  const int span = two_item_halves(t) * rows;
-  return (t.ny + span - 1) / span;
+  const int span = two_item_halves(t) * std::min(rows, t.ny);
+  return (t.ny - 1) / span + 1;
 }
 
 // Items for bands of about `rows` rows (each strip cut evenly), longest first.
