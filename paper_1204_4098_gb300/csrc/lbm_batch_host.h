@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "lbm.h"
+#include "lbm_geometry.h"
 
 namespace lbm {
 
@@ -123,7 +124,6 @@ struct TwoLattice {
   int inst, nx, ny;
   int layout = kTwoBatchAny;
 };
-constexpr int kTwoItemCols = 56;  // columns of a strip
 
 // Layouts for the lattices of a window.  Pairs are the fastest for even nx and
 // rings for narrow lattices, but several kernels side by side cost each other
@@ -150,7 +150,7 @@ inline void two_layouts(std::vector<TwoLattice>& lat) {
 // A ring is one strip of whole rows; up to 32 columns a warp takes two bands of
 // it at once.
 inline int two_item_strips(const TwoLattice& t) {
-  return t.layout == kTwoBatchRing ? 1 : (t.nx + kTwoItemCols - 1) / kTwoItemCols;
+  return t.layout == kTwoBatchRing ? 1 : (t.nx + kTwoStepCols - 1) / kTwoStepCols;
 }
 inline int two_item_halves(const TwoLattice& t) {
   return t.layout == kTwoBatchRing && t.nx <= 32 ? 2 : 1;
@@ -230,7 +230,7 @@ inline int two_item_grid(int items) {
 // work, plus the last items' share.
 inline int two_item_rows(const std::vector<TwoLattice>& lat, int sm_count) {
   const double iter[3] = {0.70, 1.10, 1.45};
-  const double resident = 12.0 * sm_count;
+  const double resident = double(kTwoStepWarps) * sm_count;
   int best_rows = 32;
   double best = 0.0;
   for (int rows : {4, 5, 6, 7, 8, 9, 10, 11, 12, 14, 16, 18, 20, 23, 26, 30, 34, 39, 45, 52, 60, 69,
