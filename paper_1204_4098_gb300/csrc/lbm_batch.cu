@@ -1287,9 +1287,11 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
     ok &= cudaMalloc(&b->d_bal_begin, 2 * size_t(warps_max(b) + 1) * sizeof(int)) ==
           cudaSuccess;
   }
-  {
+  const bool two = two_step_windows(b);
+  if (two) {
     long long items = 0;
     for (const BatchInst& d : b->desc) {  // (no layout has more items than this one)
+      if (!takes_two_steps(d)) continue;
       const TwoLattice t{0, d.nx, d.ny, kTwoBatchAny};
       items += (long long)two_item_strips(t) * two_item_bands(t, kTwoMinRows);
     }
@@ -1323,7 +1325,6 @@ lbm_status lbm_batch_create(const lbm_batch_params* p, const lbm_instance* in, i
       cudaMemsetAsync(b->buf[1], 0, off * sizeof(float), b->stream) != cudaSuccess ||
       cudaStreamSynchronize(b->stream) != cudaSuccess)
     return bail(LBM_E_CUDA, "memset");
-  const bool two = two_step_windows(b);
   if (two) {
     for (int rows : {4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256})
       b->tuner.add(kBatchTwoStep, rows);

@@ -71,3 +71,16 @@ def test_windows_of_any_length(window):
             lat.step(2 * window, d["scheme"], d["tau"], d["sigma"])
             for got, want in zip(b.moments(k), lat.observe()):
                 assert np.array_equal(got, want), (k, d)
+
+
+def test_a_batch_of_another_mode_holds_no_two_step_tables():
+    torch = pytest.importorskip("torch")
+    nx, ny = 2, 1 << 24  # (two-step items of 4 rows: 64 MB)
+    held = {}
+    for mode in (lbm.BATCH_AUTO, lbm.BATCH_WORKLIST):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        b = lbm.Batch([dict(SMALL[0], nx=nx, ny=ny)], mode=mode)
+        held[mode] = before - torch.cuda.mem_get_info()[0]
+        b.close()
+    assert held[lbm.BATCH_AUTO] - held[lbm.BATCH_WORKLIST] > 60 << 20
