@@ -705,16 +705,16 @@ lbm_status lbm_mlp_predict(lbm_mlp* m, const float* X, int n, float* Y) {
   const int groups = (n + kPredictSamples - 1) / kPredictSamples;
   const int grid = std::min(groups, 4 * m->sm_count);
   const std::unique_lock<std::mutex> stage(m->stage_mutex, std::try_to_lock);
-  if (n <= kStageSamples && stage) {
+  if (n <= kStageSamples && stage && !m->h_stage &&
+      cudaMallocHost(&m->h_stage, size_t(kStageSamples) * (kIn + kOut) * sizeof(float)) !=
+          cudaSuccess) {
+    cudaGetLastError();  // (no page-locked memory to be had: through the device's)
+    m->h_stage = nullptr;
+  }
+  if (n <= kStageSamples && stage && m->h_stage) {
     // small calls: the kernel reads and writes page-locked host memory, so the
     // call is one launch and one wait (256 samples: 58 -> 22 us against two
     // allocations, two copies and one CTA per 256 samples)
-    if (!m->h_stage &&
-        cudaMallocHost(&m->h_stage, size_t(kStageSamples) * (kIn + kOut) * sizeof(float)) !=
-            cudaSuccess) {
-      m->h_stage = nullptr;
-      return mfail(m, LBM_E_NOMEM, "cudaMallocHost of the sample staging failed");
-    }
     float* const hx = m->h_stage;
     float* const hy = m->h_stage + size_t(kStageSamples) * kIn;
     std::memcpy(hx, X, xb);
