@@ -12,8 +12,9 @@
  *   (5) BGK collision (Eqs. 1-2) with the chosen forcing scheme (or, for
  *       LBM_SCHEME_MRT, the multiple-relaxation-time form of the improved
  *       scheme).
- * All of it runs in one fused CUDA kernel per step; the host only validates
- * arguments, launches, and copies data in and out.
+ * All of it runs in fused CUDA kernels that take one to four steps per launch
+ * (lbm_step); the host only validates arguments, launches, and copies data in
+ * and out.
  *
  * Lattice: D2Q9, e0 = (0,0); e1..e4 = (1,0), (0,1), (-1,0), (0,-1);
  * e5..e8 = (1,1), (-1,1), (-1,-1), (1,-1).  Host arrays are row-major
@@ -181,18 +182,19 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
  * tau > 1/2 (sigma is read by LBM_SCHEME_IMPROVED only).  Kernels are queued
  * on the context stream: one per step, or, with the AUTO variant and band
  * height, one per up to four steps on small FP32 lattices (four up to about
- * 270^2 cells, three or two up to about 370^2) and one per two steps on larger ones and for 16-bit storage with even
- * nx (an odd last step goes alone); on lattices of at most 2048^2 cells runs
+ * 270^2 cells, three or two up to about 370^2) and one per two steps on larger
+ * ones (but for 1 and 3 columns) and for 16-bit storage with even nx from 176^2
+ * cells (an odd last step goes alone); on lattices of at most 2048^2 cells runs
  * of 16 steps, and of 64 in runs of at least 128 (of 4 and 16 launches where a
  * launch takes several steps of a small lattice), go through a CUDA graph of
  * these kernels, captured on first use for the current buffer and launch
  * arguments and kept until the context is destroyed (bit-identical to single
  * launches); while the caller captures the context stream into a graph of its
- * own, lbm_step_async records the launches one by one instead.  The call then waits for the kernels and
- * reads the device status word once (so lbm_step itself cannot be
- * captured).  LBM_E_DIVERGED if psi became undefined in any step (the state
- * is then unspecified but the context stays usable and destroyable);
- * LBM_E_STATE before lbm_init_density / lbm_set_populations. */
+ * own, lbm_step_async records the launches one by one instead.  The call then
+ * waits for the kernels and reads the device status word once (so lbm_step
+ * itself cannot be captured).  LBM_E_DIVERGED if psi became undefined in any
+ * step (the state is then unspecified but the context stays usable and
+ * destroyable); LBM_E_STATE before lbm_init_density / lbm_set_populations. */
 lbm_status lbm_step(lbm_ctx *ctx, int n, int scheme, double tau, double sigma);
 
 /* Queue n steps without waiting and without reading the status (for timing
@@ -274,14 +276,15 @@ lbm_status lbm_set_mrt_rates(lbm_ctx *ctx, double s_e, double s_eps, double s_q)
  * at least 4 rows each).  Changes only speed, never results. */
 lbm_status lbm_set_band_rows(lbm_ctx *ctx, int band_rows);
 
-/* The launch geometry lbm_step would use for `scheme`: column strips (32
- * columns wide, 64 with the PAIR variant), rows per band, bands, and CTAs of
- * 128 threads. */
+/* The geometry of a launch of one step of `scheme`: column strips (32 columns
+ * wide, 64 with the PAIR variant), rows per band, bands, and CTAs of 128
+ * threads.  Launches of several steps (lbm_step, AUTO variant and band height)
+ * have kernels and geometries of their own, which no call reports. */
 lbm_status lbm_get_launch_geometry(lbm_ctx *ctx, int scheme, int *n_strips,
                                    int *band_rows, int *n_bands, int *grid);
 
-/* The kernel variant lbm_step resolves to (REGISTER, STAGED or PAIR) for the
- * context's storage type, lattice width and requested variant. */
+/* The variant (REGISTER, STAGED or PAIR) that a launch of one step resolves to
+ * for the context's storage type, lattice size and requested variant. */
 lbm_status lbm_get_kernel_variant(lbm_ctx *ctx, int *variant);
 
 /* ---- batched parameter sweeps ------------------------------------------- */
@@ -290,7 +293,7 @@ lbm_status lbm_get_kernel_variant(lbm_ctx *ctx, int *variant);
  * tau, sigma and forcing scheme, advanced together in FP32 until each one
  * converges, diverges or reaches a step cap.  Each instance is the method of
  * lbm_step (the same fused kernel body); the batch packs all populations in
- * one buffer pair and runs windows of `window` steps as one CUDA graph:
+ * one buffer pair and runs windows of `window` steps as CUDA graphs:
  * WORKLIST: one launch per step and instance class (two columns per lane
  * for even nx, one for odd nx) over a work list of the active instances'
  * strip x band items; PERSISTENT: one launch per window in which each CTA
@@ -298,9 +301,11 @@ lbm_status lbm_get_kernel_variant(lbm_ctx *ctx, int *variant);
  * COOPERATIVE: one cooperative launch per window (every CTA resident) whose
  * warps take the work-list items of each step and meet at a bounded grid
  * barrier between steps (LBM_E_TIMEOUT if it ever gives up).  AUTO advances
- * every active instance two steps per launch (one launch for all of them) and
- * times a few band heights on live windows to keep the fastest; with the
- * REGISTER variant it times the modes above instead.  After every window an FP64 reduction per instance gives the
+ * every active instance two steps per launch (instances of one column one), in
+ * up to ten chains of launches that run side by side, and times a few band
+ * heights on live windows to keep the fastest; with the REGISTER variant, a
+ * window of two steps or instances of one column only it times the modes above
+ * instead.  After every window an FP64 reduction per instance gives the
  * coexistence densities of the flat interface (Eq. 36 slab: rho_g from rows
  * 0 and ny-1, rho_l from rows ny/2-1 and ny/2), the interface width
  * (rho_l - rho_g) / max_y |d rho_row / dy|, the mass, and the largest density
@@ -325,10 +330,10 @@ typedef struct {
  * BALANCED: per step and class, one wave of resident warps, each taking an
  * equal share of all the class's rows (the rows of every strip laid end to
  * end and cut into equal pieces, at least 8 rows each; rows_per_item does
- * not apply).  AUTO: two steps per launch for all active instances, with a band
- * height timed on live windows (reported as WORKLIST with that height); with
- * the REGISTER variant, the fastest of the modes above.  Every mode gives the
- * same results bit for bit. */
+ * not apply).  AUTO: two steps per launch, with a band height timed on live
+ * windows (reported as WORKLIST with that height), or the fastest of the modes
+ * above (see there).  Every mode gives the same results bit for bit, but for
+ * instances that diverged (LBM_RUN_DIVERGED). */
 enum { LBM_BATCH_AUTO = 0, LBM_BATCH_WORKLIST = 1, LBM_BATCH_PERSISTENT = 2,
        LBM_BATCH_COOPERATIVE = 3, LBM_BATCH_WORKLIST_DYNAMIC = 4, LBM_BATCH_BALANCED = 5 };
 /* Convergence rules.  CELL: every cell changed by less than
@@ -354,7 +359,8 @@ enum { LBM_BATCH_AUTO = 0, LBM_BATCH_WORKLIST = 1, LBM_BATCH_PERSISTENT = 2,
 enum { LBM_CONV_COEX = 0, LBM_CONV_CELL = 1, LBM_CONV_NONE = 2 /* run to max_steps */,
        LBM_CONV_TREND = 3 };
 /* An instance that diverges has its verdict at the end of the window; its state
- * and the other values of its result are then unspecified. */
+ * and the densities, width, mass and change of its result are then unspecified
+ * (and need not be the same in another run: it is not advanced any further). */
 enum { LBM_RUN_ACTIVE = 0, LBM_RUN_CONVERGED = 1, LBM_RUN_DIVERGED = 2, LBM_RUN_CAPPED = 3 };
 
 typedef struct {

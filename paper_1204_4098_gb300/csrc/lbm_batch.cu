@@ -9,9 +9,10 @@
 // column, the other two by the lanes holding columns 1 and 2), so pairs stay
 // aligned and the last column meets its periodic neighbours.  Instances fall
 // in two classes by body, each with kernels of its own (separate register
-// budgets).  A window of `window` steps is one CUDA graph.  By default it is
-// two-step launches over one list of items for all instances
-// (batch_two_step_kernel); the launch modes that can be asked for are
+// budgets).  By default a window of `window` steps is two-step launches over
+// lists of items (batch_two_step_kernel), in a few chains of launches side by
+// side, captured as graphs of 50 launches per chain and one of what is left; in
+// the launch modes that can be asked for it is one graph:
 //   work list   -- per step, one launch per class; warps take strip x band
 //                  items of the class's active instances from a prefix table
 //                  (balanced for any mix of sizes); the two class kernels are
@@ -247,7 +248,7 @@ batch_balanced_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
 // chains of launches that run side by side (two_step_graph).  Measured, us
 // per step, best work-list or balanced mode -> this: 96 slabs of 32 columns
 // 31.3 -> 9.1 (118k MLUPS), 600 of them 148 -> 37.8, 48 mixed slabs (4.7 M cells)
-// 79 -> 38.8 (122k MLUPS), 128 mixed slabs 179 -> 97.8, 6 slabs 17.6 -> 7.8.  Bound
+// 79 -> 39.0 (122k MLUPS), 128 mixed slabs 179 -> 98.1, 6 slabs 17.6 -> 7.8.  Bound
 // by the latency and issue of its instructions, like two_step_kernel.
 template <int SCHEME, int LAYOUT>
 __device__ __noinline__ void batch_two_general(const StripArgs<StoreF32>& A, int strip, int lane,
@@ -261,8 +262,8 @@ template <int LAYOUT>
 __device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int scheme, int strip,
                                                int lane, TwoSmem<StoreF32>& sm,
                                                StripArgs<StoreF32>& shared) {
-  // (two_form's choices spill here; even slabs 35.4 -> 34.9 us per step, odd 39.7
-  // -> 39.5, slabs of 32 columns 9.23 -> 9.13 against neither)
+  // (two_form's choices spill here; us per step against neither: even slabs 35.4
+  // -> 35.2, odd 39.7 -> 39.6, slabs of 32 columns 9.23 -> 9.05)
   constexpr int kForm =
       LAYOUT == kFlatEven ? kFetchIf : (LAYOUT == kRing ? kEarlyRow : kStoreIf | kFetchIf);
   if (scheme != kNoForce &&
@@ -291,7 +292,9 @@ batch_two_step_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
   const int4 it = items[range.x + blockIdx.x];  // instance, strip, first row, end row
   const int i = it.x;
   // An instance that has left the domain of psi has its verdict; its state is
-  // of no further use and is not advanced.
+  // of no further use and is not advanced.  (Every item of it would take the full
+  // forms to the end of the window: 48 slabs of which 3 diverge, first window 42.2
+  // ms, 48.5 if they go on.)
   if (inst_status[i] & kStatusDiverged) return;
   const BatchInst& I = inst[i];
   StripArgs<StoreF32> A;

@@ -452,8 +452,7 @@ int next_launch(const StepPlan& plan, int n) {
   return plan.kind == kTwoSteps && n >= 2 ? 2 : 1;
 }
 
-// Queue up to n steps on `stream`; *done counts the steps, *launches the
-// kernels.
+// Queue n steps on `stream`; *launches counts the kernels.
 cudaError_t run_plan(lbm_ctx* c, int scheme, StepPlan& plan, int n, cudaStream_t stream,
                      int* launches) {
   for (int k = 0; k < n;) {

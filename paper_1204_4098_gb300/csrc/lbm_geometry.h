@@ -144,8 +144,8 @@ inline bool two_step_applies(int requested, int precision, int nx, int ny,
 // scheme, the first two in the kernel for few CTAs), so short bands of many
 // warps pay only while the rows dominate.  us per step with 4 / 8 / 12 warps,
 // one kernel: 512^2 4.78 / 4.99 / 5.37, 768^2 7.30 / 6.79 / 7.30, 1024^2 11.1 /
-// 9.87 / 10.5, 2048^2 38.9 / 31.3 / 30.5; now 512^2 4.30, 768^2 6.37, 1024^2 9.37,
-// 2048^2 30.0.
+// 9.87 / 10.5, 2048^2 38.9 / 31.3 / 30.5; now 512^2 4.32, 768^2 6.35, 1024^2 9.29,
+// 2048^2 29.9.
 inline StripGeometry two_step_geometry(int nx, int ny, int sm_count) {
   StripGeometry g;
   g.n_strips = (nx + kTwoStepCols - 1) / kTwoStepCols;
@@ -183,15 +183,15 @@ struct TileGeometry {
 
 // Tiles for a lattice that they cover in one wave, one CTA per SM: as many
 // rows of tiles as there are SMs for, at most 48 lattice rows each with the
-// halo of two cells per step.  Up to there tiles are the fastest at every size
-// (128^2: 1.41 us per step with 152 tiles of 7 rows, 1.66 with 72 of 15; a
-// second wave only ties with two-step launches: 300^2 with four steps 3.02).
-// Fewer steps leave more columns and rows to a tile, so a lattice takes the
-// most steps that fit, us per step with 4 / 3 / 2 and of the two-step strips
-// (300^2):
-// 64^2 1.10 / 1.29 / 1.42, 128^2 1.26 / 1.42 / 1.55, 200^2 1.71 / 1.72 / 1.93,
-// 256^2 2.12 / 2.06 / 2.12, 300^2 - / 2.40 / 2.57 / 3.02.  (Five steps gain 3 %
-// at 16^2 and 1 % at 64^2 and lose from 96^2 on.)  The same requirements on
+// halo of two cells per step.  Up to there tiles are the fastest at every size,
+// and a second wave only ties with two-step launches.  (With fewer, taller tiles
+// the kernel's first version took 18 % longer at 128^2.)  Fewer steps leave more
+// columns and rows to a tile, so a lattice takes the most steps that fit, us per
+// step with 4 / 3 / 2 and, last, on strips (one step per launch below 176^2, two
+// from there): 64^2 1.06 / 1.17 / 1.42 / 2.57, 128^2 1.22 / 1.38 / 1.54 / 2.63,
+// 200^2 1.68 / 1.72 / 1.93 / 2.54, 256^2 2.07 / 2.06 / 2.12 / 2.76, 300^2 - / 2.32 /
+// 2.57 / 2.86, 360^2 - / - / 2.95 / 3.34.  (Five steps gain 3 % at 16^2 and 1 % at
+// 64^2 and lose from 96^2 on.)  The same requirements on
 // variant, storage, band height and covolume as two_step_applies.
 inline TileGeometry tile_geometry(int requested, int precision, int nx, int ny,
                                   int band_rows_override, double b, int sm_count) {

@@ -23,9 +23,9 @@
 // again with the full forms.
 //
 // Measured, us per step in step graphs (improved scheme), best other kernel ->
-// this: 32^2 2.69 -> 1.03, 64^2 2.69 -> 1.07, 128^2 2.76 -> 1.23, 200^2 3.20 ->
-// 1.68, 256^2 3.46 -> 2.09 with four steps, 300^2 3.02 -> 2.32 with three, 360^2
-// 3.53 -> 2.95 with two.  A launch takes about 1.8 us + 0.24 us and 0.03 us per
+// this: 32^2 2.54 -> 1.03, 64^2 2.57 -> 1.06, 128^2 2.63 -> 1.22, 200^2 2.54 ->
+// 1.68, 256^2 2.76 -> 2.07 with four steps, 300^2 2.86 -> 2.32 with three, 360^2
+// 3.34 -> 2.95 with two.  A launch takes about 1.8 us + 0.24 us and 0.03 us per
 // active row for every step + 0.03 us per row loaded: at 64^2 a third of its 4.3
 // us is the launch itself, the rest mostly one warp's serial row of arithmetic.
 // Tried without gain: one row per warp, programmatic dependent launch (64^2:
@@ -58,8 +58,8 @@ __device__ __forceinline__ F2 psi_normal_masked(F2 rho, const Phys<float>& P, bo
 }
 
 // The tile whose first owned cell is (x0, y0), `rows` owned rows; f: shared
-// memory, kQ planes of populations and one of psi, H x 32 floats each, H = 2
-// warps >= rows + 2 halo; 1 <= steps <= halo / 2.
+// memory, kQ planes of populations and one of psi of H x 32 floats each,
+// kTilePlane apart, H = 2 warps >= rows + 2 halo; 1 <= steps <= halo / 2.
 // Returns (to every thread of the CTA) whether every check held.
 template <int SCHEME, bool kNormal>
 __device__ __forceinline__ bool run_tile(const StripArgs<StoreF32>& A, int steps, int halo,

@@ -37,17 +37,17 @@
 // Measured on the way (improved scheme, 4096^2, us per step; one-step kernel
 // 197.5): first version 141; unrolled by two 134; bare divisions and roots
 // 128; no branches 123; step 2 one row behind 118; one warp per CTA 114; the
-// arriving row read first and predicated copies 112.2 (149k MLUPS, DRAM at
+// arriving row read first and predicated copies 111.9 (150k MLUPS, DRAM at
 // 0.78 of the measured copy bandwidth, FMA pipes 60 % busy, 12 warps per SM).
 // 13 to 16 warps per SM (128 registers, spilling) 119-122; rows of step 1 kept
 // in registers 141 (spills).  Small launches, whose SMs get 4 or 8 warps, are
 // latency bound and take a kernel with 255 registers and more overlap
-// (two_form): 512^2 4.65 -> 4.30, 1024^2 9.75 -> 9.37.
+// (two_form): 512^2 4.65 -> 4.32, 1024^2 9.75 -> 9.29.
 //
 // 16-bit storage gains from the instructions that two separate steps repeat
 // (the row copies, the halo's psi) and from the bare divisions: it was bound
 // by issue, not by memory (BF16, us per step, one-step -> two-step: 4096^2 186 ->
-// 129, 2048^2 51.1 -> 34.4, 1024^2 16.6 -> 10.8, 512^2 7.4 -> 5.1, 256^2 4.2 ->
+// 129, 2048^2 51.1 -> 34.4, 1024^2 16.6 -> 10.7, 512^2 7.4 -> 5.1, 256^2 4.2 ->
 // 3.4; FP16 the same).
 #pragma once
 
@@ -117,7 +117,7 @@ __device__ __forceinline__ F2 psi_normal(F2 rho, const Phys<float>& P, bool& ok)
 // kFetchIf: the stores and the row copies are predicated instead of branched
 // around, so that step 2 and step 1 share a block of instructions.  More
 // overlap takes registers, so what pays differs, us per step with neither / the
-// form taken: even nx, 12 CTAs per SM: 512^2 4.65 / 4.49, 1024^2 9.71 / 9.61,
+// form taken (as measured when the form was chosen): even nx, 12 CTAs per SM: 512^2 4.65 / 4.49, 1024^2 9.71 / 9.61,
 // 4096^2 113.1 / 112.3, MRT 2048^2 32.6 / 31.6; 8 CTAs per SM: 512^2 4.62 / 4.27,
 // 1024^2 9.72 / 9.38, BF16 1024^2 10.90 / 10.71; odd nx: 1023x1025 11.31 / 10.97
 // with 8.  All three with 12 CTAs spill (4096^2 114.0).
