@@ -114,6 +114,10 @@ MEASURED_TRAFFIC = {
     # (one step), 630.7 + 558.8 (two), x4 cells
     ("cfed21be853ad9c9", "fp32", 8192, "pair"): 4.6868e9,
     ("cfed21be853ad9c9", "fp32", 8192, "two_step"): 4.7578e9,
+    # the same step kernels after a change to the initial-state kernel: 616.7 + 554.9
+    # MB (one step), 630.5 + 558.9 (two), x4 cells
+    ("cb3cb42e492074c8", "fp32", 8192, "pair"): 4.6863e9,
+    ("cb3cb42e492074c8", "fp32", 8192, "two_step"): 4.7574e9,
 }
 
 

@@ -1031,6 +1031,9 @@ __global__ void set_state_kernel(typename S::T* dst, float* rho_dst, int nx, int
                                  const double* uy, const double* f_in, Phys<double> P,
                                  Phys<float> F, unsigned* status) {
   const size_t n = size_t(pitch) * ny;
+  // (at rest f_eq is one product, not eleven operations of the FP64 pipe that
+  // bounds this kernel, and the same value: the call on BF16 1024^2 258 -> 140 us)
+  const bool rest = !ux && !uy;
   bool bad = false;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x) {
@@ -1046,6 +1049,8 @@ __global__ void set_state_kernel(typename S::T* dst, float* rho_dst, int nx, int
       double v;
       if (f_in) {
         v = f_in[a * (size_t(nx) * ny) + j];  // unpadded [9][ny][nx]
+      } else if (rest) {
+        v = w_of<double>(a) * rho[j];
       } else {
         v = equilibrium(a, rho[j], ux ? ux[j] : 0.0, uy ? uy[j] : 0.0);
       }
