@@ -404,6 +404,10 @@ constexpr int kGraphSteps = 16;
 // us per step, 200^2 1.92 -> 1.70, 1024^2 9.87 -> 9.75; four times as long
 // again gains another 1 %).
 constexpr int kLongGraphSteps = 64;
+// The capture of 64 one-step launches takes the host 70 us more than that of 16,
+// what ~900 steps gain from it: a shorter run with new arguments leaves it to the
+// next one (BF16 64^2, first call of a context, 128 steps: 581 -> 513 us).
+constexpr int kLongAtOnce = 16 * kLongGraphSteps;
 // Graphs of tile launches: 4 launches and 16, however many steps each takes.
 constexpr int kGraphTiles = 4, kLongGraphTiles = 16;
 static_assert(kGraphTiles % 2 == 0 && kLongGraphTiles % 2 == 0 && kGraphSteps % 4 == 0 &&
@@ -508,24 +512,34 @@ bool same_launch(const StripLaunch& x, const StripLaunch& y) {
          x.s_q == y.s_q;
 }
 
-// The cached graph (the shorter or the longer one) of steps from the current
-// buffer, captured again when any kernel argument, the scheme, the kernel variant or the grid
-// changed; nullptr when capture is unavailable (the caller then launches
-// step by step).  The number of launches is even, so a replay leaves the
-// state in the same buffer.
+// What a step graph (the shorter or the longer one) from the current buffer has
+// to have been captured with, exec left out, and whether the kept one was.
+lbm_ctx::StepGraph graph_key(const lbm_ctx* c, int scheme, const StepPlan& plan) {
+  const bool single = plan.kind == kSingleSteps;
+  lbm_ctx::StepGraph g;
+  g.L = single ? plan.one : plan.many;
+  g.L.src = c->f[c->cur];
+  g.L.dst = c->f[1 - c->cur];
+  g.L.rho_src = c->rho[c->cur];
+  g.L.rho_dst = c->rho[1 - c->cur];
+  g.scheme = scheme;
+  g.variant = single ? pick_variant(c, kStepMode) : -plan.kind;
+  g.grid = single ? plan.one_grid : plan.many_grid;
+  return g;
+}
+bool graph_kept(const lbm_ctx* c, int scheme, const StepPlan& plan, bool longer) {
+  const lbm_ctx::StepGraph &g = c->graph[longer][c->cur], key = graph_key(c, scheme, plan);
+  return g.exec && g.scheme == key.scheme && g.variant == key.variant && g.grid == key.grid &&
+         same_launch(g.L, key.L);
+}
+
+// The kept graph, captured again when any kernel argument, the scheme, the kernel
+// variant or the grid changed; nullptr when capture is unavailable (the caller
+// then launches step by step).  The number of launches is even, so a replay
+// leaves the state in the same buffer.
 cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan, bool longer) {
   lbm_ctx::StepGraph& g = c->graph[longer][c->cur];
-  const bool single = plan.kind == kSingleSteps;
-  const int variant = single ? pick_variant(c, kStepMode) : -plan.kind;
-  const int grid = single ? plan.one_grid : plan.many_grid;
-  StripLaunch first = single ? plan.one : plan.many;  // the key
-  first.src = c->f[c->cur];
-  first.dst = c->f[1 - c->cur];
-  first.rho_src = c->rho[c->cur];
-  first.rho_dst = c->rho[1 - c->cur];
-  if (g.exec && g.scheme == scheme && g.variant == variant && g.grid == grid &&
-      same_launch(g.L, first))
-    return g.exec;
+  if (graph_kept(c, scheme, plan, longer)) return g.exec;
   if (g.exec) {
     cudaGraphExecDestroy(g.exec);
     g.exec = nullptr;
@@ -554,11 +568,8 @@ cudaGraphExec_t step_graph(lbm_ctx* c, int scheme, const StepPlan& plan, bool lo
     cudaGetLastError();
     return nullptr;
   }
+  g = graph_key(c, scheme, plan);
   g.exec = exec;
-  g.L = first;
-  g.scheme = scheme;
-  g.variant = variant;
-  g.grid = grid;
   return exec;
 }
 
@@ -620,6 +631,9 @@ lbm_status queue_steps(lbm_ctx* c, int n, int scheme, double tau, double sigma) 
     for (const bool longer : {true, false}) {
       const int steps = graph_steps(plan, longer);
       if (n - k < (longer ? 2 * steps : steps)) continue;
+      if (longer && plan.kind == kSingleSteps && n < kLongAtOnce &&
+          !graph_kept(c, scheme, plan, true) && !graph_kept(c, scheme, plan, false))
+        continue;
       const cudaGraphExec_t g = step_graph(c, scheme, plan, longer);
       if (!g) break;
       for (; k + steps <= n; k += steps) {

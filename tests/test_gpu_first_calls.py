@@ -1,0 +1,48 @@
+"""The first call of a context: what it captures, it has to gain back."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_1204_4098_gb300 import lbm
+
+pytestmark = pytest.mark.gpu
+
+
+def first_call(steps, precision):
+    rho = np.full((64, 64), 0.12)
+    out = []
+    for _ in range(15):
+        with lbm.Lattice(64, 64, 0.9, precision=precision) as lat:
+            lat.init_density(rho)
+            t = time.perf_counter()
+            lat.step(steps, lbm.IMPROVED, 0.8, 0.1)
+            out.append(time.perf_counter() - t)
+    return min(out)
+
+
+@pytest.mark.parametrize("precision", [lbm.BF16DEV, lbm.FP16DEV])
+def test_first_call_of_one_step_launches(precision):
+    first_call(64, precision)
+    # twice as many steps share one capture, launch and wait; a longer graph on
+    # top (70 us) would make it more than twice
+    assert first_call(128, precision) < 1.93 * first_call(64, precision)
+
+
+@pytest.mark.parametrize("nx,ny,precision", [(64, 48, lbm.BF16DEV), (60, 50, lbm.FP64),
+                                             (97, 60, lbm.FP32)])
+def test_calls_in_a_row(nx, ny, precision):
+    # from either buffer, with the shorter graph only, both, and new arguments
+    calls = [(128, 0.8), (1, 0.8), (200, 0.8), (130, 0.8), (3, 0.8), (129, 0.9), (64, 0.9),
+             (1024, 0.9), (16, 0.8), (128, 0.8)]
+    rho = 0.12 * np.random.default_rng(1).uniform(0.999, 1.001, (ny, nx))
+    got = []
+    for one_by_one in (False, True):
+        with lbm.Lattice(nx, ny, 0.9, precision=precision) as lat:
+            lat.set_variant(lbm.VARIANT_REGISTER)
+            lat.init_density(rho)
+            for n, tau in calls:
+                for m in [1] * n if one_by_one else [n]:
+                    lat.step(m, lbm.IMPROVED, tau, 0.1)
+            got.append(lat.populations())
+    assert np.array_equal(*got)
