@@ -118,6 +118,10 @@ MEASURED_TRAFFIC = {
     # MB (one step), 630.5 + 558.9 (two), x4 cells
     ("cb3cb42e492074c8", "fp32", 8192, "pair"): 4.6863e9,
     ("cb3cb42e492074c8", "fp32", 8192, "two_step"): 4.7574e9,
+    # the same with another form of the check in the kernels of odd widths: 616.8 +
+    # 554.9 MB (one step), 630.7 + 558.7 (two), x4 cells
+    ("c45cc41a05887764", "fp32", 8192, "pair"): 4.6868e9,
+    ("c45cc41a05887764", "fp32", 8192, "two_step"): 4.7576e9,
 }
 
 

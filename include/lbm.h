@@ -189,10 +189,10 @@ lbm_status lbm_init_density_at_rest(lbm_ctx *ctx, const double *rho);
  * launch takes several steps of a small lattice), go through a CUDA graph of
  * these kernels, captured on first use for the current buffer and launch
  * arguments (64 one-step launches on the second, or from 1024 steps on) and kept
- * until the context is destroyed (bit-identical to single launches); while the caller captures the context stream into a graph of its
- * own, lbm_step_async records the launches one by one instead.  The call then
- * waits for the kernels and reads the device status word once (so lbm_step
- * itself cannot be captured).  LBM_E_DIVERGED if psi became undefined in any
+ * until the context is destroyed (bit-identical to single launches); while the
+ * caller captures the context stream into a graph of its own, lbm_step_async
+ * records the launches one by one instead.  The call then waits for the kernels
+ * and reads the device status word once (so lbm_step itself cannot be captured).  LBM_E_DIVERGED if psi became undefined in any
  * step (the state is then unspecified but the context stays usable and
  * destroyable); LBM_E_STATE before lbm_init_density / lbm_set_populations. */
 lbm_status lbm_step(lbm_ctx *ctx, int n, int scheme, double tau, double sigma);

@@ -248,7 +248,7 @@ batch_balanced_kernel(const BatchInst* __restrict__ inst, const int4* __restrict
 // chains of launches that run side by side (two_step_graph).  Measured, us
 // per step, best work-list or balanced mode -> this: 96 slabs of 32 columns
 // 31.3 -> 9.1 (118k MLUPS), 600 of them 148 -> 37.8, 48 mixed slabs (4.7 M cells)
-// 79 -> 39.0 (122k MLUPS), 128 mixed slabs 179 -> 98.1, 6 slabs 17.6 -> 7.8.  Bound
+// 79 -> 38.8 (122k MLUPS), 128 mixed slabs 179 -> 97.4, 6 slabs 17.6 -> 7.8.  Bound
 // by the latency and issue of its instructions, like two_step_kernel.
 template <int SCHEME, int LAYOUT>
 __device__ __noinline__ void batch_two_general(const StripArgs<StoreF32>& A, int strip, int lane,
@@ -263,9 +263,8 @@ __device__ __forceinline__ void batch_two_item(const StripArgs<StoreF32>& A, int
                                                int lane, TwoSmem<StoreF32>& sm,
                                                StripArgs<StoreF32>& shared) {
   // (two_form's choices spill here; us per step against neither: even slabs 35.4
-  // -> 35.2, odd 39.7 -> 39.6, slabs of 32 columns 9.23 -> 9.05)
-  constexpr int kForm =
-      LAYOUT == kFlatEven ? kFetchIf : (LAYOUT == kRing ? kEarlyRow : kStoreIf | kFetchIf);
+  // -> 34.8, odd 39.7 -> 39.5, slabs of 32 columns 9.23 -> 9.05)
+  constexpr int kForm = LAYOUT == kRing ? kEarlyRow : kStoreIf | kFetchIf;
   if (scheme != kNoForce &&
       strip_run_two<StoreF32, kBlend, LAYOUT, true, kForm>(A, strip, 0, lane, sm))
     return;
